@@ -16,6 +16,7 @@
 // zeta sketch rows with FP64 atomics in L2, as the dense path does below
 // m n = 2^24 (rounding order not fixed).
 #include "lsq_common.cuh"
+#include "lsq_dev.cuh"
 
 namespace lsq {
 
@@ -120,13 +121,15 @@ __global__ void __launch_bounds__(kCsrThreads)
                     const double *__restrict__ x, double *__restrict__ part,
                     double *__restrict__ r2_part, int npad, const DevState *gate,
                     const double *bscale, double *rout) {
-  if (gate != nullptr && *(volatile const int *)&gate->done) return;
+  griddep_launch();
   extern __shared__ double csm[];
   __shared__ double r2w[kCsrWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double *hw = csm + (size_t)warp * npad;
   for (int j = lane; j < npad; j += 32) hw[j] = 0.0;
   __syncwarp();
+  griddep_wait();
+  if (gate != nullptr && *(volatile const int *)&gate->done) return;
   const double bs = (MODE == 1 && bscale != nullptr) ? *bscale : 1.0;
   double r2 = 0.0;
   int64_t r0, r1;
@@ -224,12 +227,12 @@ cudaError_t launch_csr_pass(int mode, const int64_t *rp, const int32_t *col, con
   const void *fn = mode == 0 ? (const void *)csr_pass_kernel<0> : (const void *)csr_pass_kernel<1>;
   cudaError_t e = ensure_smem_attr(fn, smem);
   if (e != cudaSuccess) return e;
-  if (mode == 0)
-    csr_pass_kernel<0><<<grid, kCsrThreads, smem, s>>>(rp, col, val, m, b, x, part, r2_part, npad,
-                                                       gate, bscale, rout);
-  else
-    csr_pass_kernel<1><<<grid, kCsrThreads, smem, s>>>(rp, col, val, m, b, x, part, r2_part, npad,
-                                                       gate, bscale, rout);
+  auto *k = mode == 0 ? csr_pass_kernel<0> : csr_pass_kernel<1>;
+  if (gate != nullptr)
+    return launch_pdl(k, dim3(grid), dim3(kCsrThreads), (size_t)smem, s, rp, col, val, m, b, x,
+                      part, r2_part, npad, gate, bscale, rout);
+  k<<<grid, kCsrThreads, smem, s>>>(rp, col, val, m, b, x, part, r2_part, npad, gate, bscale,
+                                    rout);
   return cudaGetLastError();
 }
 

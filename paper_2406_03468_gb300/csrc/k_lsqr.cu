@@ -13,7 +13,8 @@
 // pass is shaped like the residual pass: the m-vector s holds -q_k, the pass
 // computes r = bscale s - A z (= -q_{k+1}, with bscale = alpha_k / beta_k in
 // the sign convention below), writes it back to s, and sums A^T r and
-// ||r||^2 = beta_{k+1}^2.  The n-vector recurrences run on one CTA.
+// ||r||^2 = beta_{k+1}^2.  The n-vector recurrences run in k_inner.cu's
+// kernels (method 2).
 //
 // Sign convention: s starts as r_i = q_1 (written by the step's FP64
 // residual pass), so the first pass takes bscale = +alpha_1 / beta_1; every
@@ -56,7 +57,7 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
                    int64_t m, int n, const double *__restrict__ z, double *s,
                    const double *bscale, double *__restrict__ part, double *__restrict__ r2part,
                    int npad, const DevState *gate, int *err) {
-  if (gate != nullptr && *(volatile const int *)&gate->done) return;
+  griddep_launch();
   extern __shared__ __align__(16) double lacc[];
   __shared__ double wmax[kPassThreads / 32];
   __shared__ double wr2[kPassThreads / 32];
@@ -85,10 +86,17 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
       bulk_g2s(dh + NC * 64, Alo + i * ld32, row_bytes, wbar + stg, pol);
     }
   };
+  // the planes were complete before the inner loop began (as atax_df_kernel)
   for (int64_t q = 0; q < kLqStages; q++) issue(q);
 
   double *hw = lacc + (size_t)warp * NC * 64;
   for (int i = lane; i < NC * 64; i += 32) hw[i] = 0.0;
+  griddep_wait();
+  if (gate != nullptr && *(volatile const int *)&gate->done) {
+    if (lane == 0)
+      for (int64_t q = 0; q < kLqStages && q < nrows; q++) mbar_wait(wbar + q, 0, kLqWaitNs);
+    return;
+  }
   double zr[2 * NC];
   lq_load_vec<NC>(z, n, lane, zr);
   double zmax = 0.0;
@@ -236,65 +244,14 @@ __global__ void __launch_bounds__(kVecThreads)
     const double alpha = live ? cn / beta : 0.0;
     st->lq_alpha = alpha;
     st->lq_beta = beta;
-    st->lq_phibar = beta;
-    st->lq_rhobar = alpha;
+    st->lq_phibar[0] = beta;
+    st->lq_rhobar[0] = alpha;
     st->lq_bscale = live ? alpha / beta : 0.0;
     st->iters = 0;
     st->max_iters = max_iters;
     st->use_thresh = use_thresh;
     st->dnorm2 = 0.0;
     st->done = (max_iters <= 0 || !live) ? 1 : 0;
-  }
-}
-
-// One LSQR iteration after the pass: p = R^{-T} D^{-1} A^T s = -B^T q_{k+1},
-// beta_{k+1}^2 = st->lq_b2.  v <- (B^T u_{k+1} - beta v) / alpha, the plane
-// rotation, dy += (phi / rho) w, w <- v - (theta / rho) w, and the stop test
-// of SPIR's rules on the step (phi / rho) w.
-__global__ void __launch_bounds__(kVecThreads)
-    lsqr_update_kernel(int n, const double *__restrict__ p, double *v, double *w, double *dy,
-                       DevState *st) {
-  if (*(volatile int *)&st->done) return;
-  __shared__ double scratch[32];
-  const double beta = sqrt(st->lq_b2);
-  const double ib = beta > 0.0 ? 1.0 / beta : 0.0;
-  double aa = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double vi = -p[i] * ib - beta * v[i];
-    v[i] = vi;
-    aa = fma(vi, vi, aa);
-  }
-  aa = block_sum(aa, scratch);
-  const double alpha = sqrt(aa);
-  const double ia = alpha > 0.0 ? 1.0 / alpha : 0.0;
-  const double rhobar = st->lq_rhobar, phibar = st->lq_phibar;
-  const double rho = hypot(rhobar, beta);
-  const double cs = rhobar / rho, sn = beta / rho;
-  const double theta = sn * alpha;
-  const double phi = cs * phibar;
-  const double tstep = phi / rho, tw = theta / rho;
-  double ss = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double vi = v[i] * ia;
-    v[i] = vi;
-    const double step = tstep * w[i];
-    dy[i] += step;
-    w[i] = vi - tw * w[i];
-    ss = fma(step, step, ss);
-  }
-  ss = block_sum(ss, scratch);
-  if (threadIdx.x == 0) {
-    st->lq_alpha = alpha;
-    st->lq_beta = beta;
-    st->lq_rhobar = -cs * alpha;
-    st->lq_phibar = sn * phibar;
-    st->lq_bscale = beta > 0.0 ? -alpha / beta : 0.0;
-    const int it = st->iters + 1;
-    st->iters = it;
-    st->dnorm2 = ss;
-    bool stop = it >= st->max_iters || !(alpha > 0.0) || !(sn * phibar != 0.0);
-    if (st->use_thresh && sqrt(ss) <= st->thresh1) stop = true;
-    if (stop) st->done = 1;
   }
 }
 
@@ -315,9 +272,8 @@ cudaError_t launch_pass_lsqr_df(const float *Ahi, const float *Alo, int64_t ld32
       cudaError_t e = ensure_smem_attr((const void *)lsqr_df_kernel<NCV>, (int)smem);         \
       if (e != cudaSuccess) return e;                                                         \
     }                                                                                         \
-    lsqr_df_kernel<NCV><<<grid, kPassThreads, smem, st>>>(Ahi, Alo, ld32, m, n, z, s, bscale,   \
-                                                          part, r2part, npad, gate, err);     \
-    break;                                                                                    \
+    return launch_pdl(lsqr_df_kernel<NCV>, dim3(grid), dim3(kPassThreads), smem, st, Ahi, Alo, \
+                      ld32, m, n, z, s, bscale, part, r2part, npad, gate, err);               \
   }
     LSQ_LQ_CASE(1)
     LSQ_LQ_CASE(2)
@@ -334,12 +290,6 @@ cudaError_t launch_pass_lsqr_df(const float *Ahi, const float *Alo, int64_t ld32
 cudaError_t launch_lsqr_init(int n, const double *c, int step, double *v, double *w, double *dy,
                              int max_iters, int use_thresh, DevState *st, cudaStream_t s) {
   lsqr_init_kernel<<<1, kVecThreads, 0, s>>>(n, c, step, v, w, dy, max_iters, use_thresh, st);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lsqr_update(int n, const double *p, double *v, double *w, double *dy,
-                               DevState *st, cudaStream_t s) {
-  lsqr_update_kernel<<<1, kVecThreads, 0, s>>>(n, p, v, w, dy, st);
   return cudaGetLastError();
 }
 

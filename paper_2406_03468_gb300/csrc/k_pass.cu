@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
                    int64_t m, int n, const double *__restrict__ z, double *__restrict__ part,
                    int npad, const DevState *gate, int *err, int64_t zstride,
                    int64_t pstride) {
-  if (gate != nullptr && *(volatile const int *)&gate->done) return;
+  griddep_launch();
   // many right-hand sides: grid row blockIdx.y works on vector z_(blockIdx.y)
   z += (int64_t)blockIdx.y * zstride;
   part += (int64_t)blockIdx.y * pstride;
@@ -267,10 +267,18 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
       bulk_g2s(dh + NC * 64, Alo + i * ld32, row_bytes, wbar + stg, pol);
     }
   };
+  // the planes were complete before the inner loop began: the first rows are
+  // on their way while the kernel that forms z ends
   for (int64_t q = 0; q < kDfStages; q++) issue(q);
 
   double *hw = hacc + (size_t)warp * NC * 64;
   for (int i = lane; i < NC * 64; i += 32) hw[i] = 0.0;
+  griddep_wait();
+  if (gate != nullptr && *(volatile const int *)&gate->done) {
+    if (lane == 0)  // the copies in flight land before the CTA's memory is released
+      for (int64_t q = 0; q < kDfStages && q < nrows; q++) mbar_wait(wbar + q, 0, kDfWaitNs);
+    return;
+  }
   double zr[2 * NC];
   load_vec<NC>(z, n, lane, zr);
   double zmax = 0.0;
@@ -410,7 +418,7 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
     atax32_kernel(const float *__restrict__ A32, int64_t ld32, int64_t m, int n,
                   const double *__restrict__ z, double *__restrict__ part, int npad,
                   const DevState *gate, int *err) {
-  if (gate != nullptr && *(volatile const int *)&gate->done) return;
+  griddep_launch();
   // dynamic shared memory: [warps][k32Stages][NC*64] FP32 row stages, then
   // the mbarriers
   extern __shared__ __align__(16) float rst[];
@@ -439,6 +447,12 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
     }
   };
   for (int64_t q = 0; q < k32Stages; q++) issue(q);
+  griddep_wait();
+  if (gate != nullptr && *(volatile const int *)&gate->done) {
+    if (lane == 0)
+      for (int64_t q = 0; q < k32Stages && q < nrows; q++) mbar_wait(wbar + q, 0, kDfWaitNs);
+    return;
+  }
   double zr[2 * NC];
   load_vec<NC>(z, n, lane, zr);
   double zmax = 0.0;
@@ -740,49 +754,63 @@ __global__ void reduce_batched_kernel(const double *__restrict__ part, int grid,
   out[idx] = scale ? scale[j] * s : s;
 }
 
-// out[j] = scale[j] sum_g part[g npad + j]; *r2 = sum_g r2_part[g] (CTA 0).
-// One CTA per 32 columns: warp w sums the partials g = w, w + 8, ... of the
-// lane's column, then warp 0 adds the 8 warp sums in order (a fixed order,
-// so the result is deterministic).  A sub-partition issues one FP64 warp
-// instruction per 64 cycles, so the partials of a column are spread over
-// all four sub-partitions rather than summed by one thread.
+// out[j] = scale[j] sum_g part[g npad + j]; *r2 = sum_g r2_part[g] (one CTA
+// more).  One CTA per 8 columns, 32 threads per column, each the partials
+// g = t, t + 32, ...; the 32 sums by shuffles and, across the warps, in
+// shared memory (a fixed order, so the result is deterministic).  It is bound
+// by latency: a sub-partition issues one FP64 warp instruction per 64 cycles,
+// so the n G additions are spread over all SMs.  At G = 304, n = 500: 63 CTAs
+// of about 10 additions per thread; CTAs of 32 columns with 38 per thread
+// took 6.5 us in the inner loop.
 constexpr int kReduceThreads = 256;
+constexpr int kReduceCols = 8;
 __global__ void __launch_bounds__(kReduceThreads)
     reduce_kernel(const double *__restrict__ part, int grid, int npad, int n,
                   const double *__restrict__ scale, double *__restrict__ out,
-                  const double *__restrict__ r2_part, double *r2, const DevState *gate) {
-  if (gate != nullptr && *(volatile const int *)&gate->done) return;
-  __shared__ double red[kReduceThreads / 32][33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kReduceThreads / 32;
-  const int j = blockIdx.x * 32 + lane;
-  double s0 = 0.0, s1 = 0.0;
-  if (j < n) {
-    int g = warp;
-    for (; g + nw < grid; g += 2 * nw) {
-      s0 += part[(size_t)g * npad + j];
-      s1 += part[(size_t)(g + nw) * npad + j];
-    }
-    if (g < grid) s0 += part[(size_t)g * npad + j];
+                  const double *__restrict__ r2_part, double *r2, DevState *gate) {
+  griddep_launch();
+  griddep_wait();
+  if (gate != nullptr) {
+    const int done = *(volatile const int *)&gate->done;
+    if (blockIdx.x == 0 && threadIdx.x == 0) gate->ugate = done;
+    if (done) return;
   }
-  red[warp][lane] = s0 + s1;
-  __syncthreads();
-  if (warp == 0 && j < n) {
-    double s = 0.0;
-    for (int w = 0; w < nw; w++) s += red[w][lane];
-    out[j] = scale ? scale[j] * s : s;
-  }
-  if (r2 != nullptr && blockIdx.x == 0) {
-    __syncthreads();
+  constexpr int kGroups = kReduceThreads / kReduceCols, kW = kReduceThreads / 32;
+  __shared__ double red[kW][kReduceCols];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (r2 != nullptr && blockIdx.x == gridDim.x - 1) {
     double t = 0.0;
     for (int g = threadIdx.x; g < grid; g += kReduceThreads) t += r2_part[g];
     t = warp_sum(t);
-    if (lane == 0) red[warp][32] = t;
+    if (lane == 0) red[warp][0] = t;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double u = 0.0;
-      for (int w = 0; w < nw; w++) u += red[w][32];
-      *r2 = u;
+    if (warp == 0) {
+      t = warp_sum(lane < kW ? red[lane][0] : 0.0);
+      if (lane == 0) *r2 = t;
     }
+    return;
+  }
+  const int c = threadIdx.x % kReduceCols, t0 = threadIdx.x / kReduceCols;
+  const int j = blockIdx.x * kReduceCols + c;  // < npad
+  double s0 = 0.0, s1 = 0.0;
+  int g = t0;
+#pragma unroll 4
+  for (; g + kGroups < grid; g += 2 * kGroups) {
+    s0 += part[(size_t)g * npad + j];
+    s1 += part[(size_t)(g + kGroups) * npad + j];
+  }
+  if (g < grid) s0 += part[(size_t)g * npad + j];
+  double s = s0 + s1;
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  if (lane < kReduceCols) red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+    const int q = lane >> 3;
+    s = red[q][c] + red[q + 4][c];
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    if (lane < kReduceCols && j < n) out[j] = scale ? scale[j] * s : s;
   }
 }
 
@@ -840,6 +868,9 @@ cudaError_t launch_pass_atax_df(const float *Ahi, const float *Alo, int64_t ld32
       cudaError_t e = ensure_smem_attr((const void *)atax_df_kernel<NC>, (int)smem);
       if (e != cudaSuccess) return e;
     }
+    if (gate != nullptr)
+      return launch_pdl(atax_df_kernel<NC>, g, dim3(kPassThreads), smem, s, Ahi, Alo, ld32, m, n,
+                        z, part, npad, gate, err, zstride, pstride);
     atax_df_kernel<NC><<<g, kPassThreads, smem, s>>>(Ahi, Alo, ld32, m, n, z, part, npad, gate,
                                                      err, zstride, pstride);
   });
@@ -857,7 +888,8 @@ cudaError_t launch_pass_atax32(const float *A32, int64_t ld32, int64_t m, int n,
       cudaError_t e = ensure_smem_attr((const void *)atax32_kernel<NC>, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    atax32_kernel<NC><<<grid, kPassThreads, smem, s>>>(A32, ld32, m, n, z, part, npad, gate, err);
+    return launch_pdl(atax32_kernel<NC>, dim3(grid), dim3(kPassThreads), smem, s, A32, ld32, m, n,
+                      z, part, npad, gate, err);
   });
   return cudaGetLastError();
 }
@@ -912,10 +944,13 @@ cudaError_t launch_reduce_batched(const double *part, int grid, int npad, int n,
 }
 
 cudaError_t launch_reduce(const double *part, int grid, int npad, int n, const double *scale,
-                          double *out, const double *r2_part, double *r2, const DevState *gate,
+                          double *out, const double *r2_part, double *r2, DevState *gate,
                           cudaStream_t s) {
-  reduce_kernel<<<(n + 31) / 32, kReduceThreads, 0, s>>>(part, grid, npad, n, scale, out, r2_part,
-                                                       r2, gate);
+  const int g = (n + kReduceCols - 1) / kReduceCols + (r2 != nullptr ? 1 : 0);
+  if (gate != nullptr)
+    return launch_pdl(reduce_kernel, dim3(g), dim3(kReduceThreads), 0, s, part, grid, npad, n,
+                      scale, out, r2_part, r2, gate);
+  reduce_kernel<<<g, kReduceThreads, 0, s>>>(part, grid, npad, n, scale, out, r2_part, r2, gate);
   return cudaGetLastError();
 }
 

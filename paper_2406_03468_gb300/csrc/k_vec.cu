@@ -1,4 +1,5 @@
-// n-vector steps of the inner solvers, one CTA each (n <= LSQ_MAX_N):
+// n-vector steps of the inner solvers, one CTA each (n <= LSQ_MAX_N; a plan's
+// iterations run them inside k_inner.cu's kernels, the batched engine here):
 //   Polyak heavy ball (Alg. 5, in the loop form of Alg. 4):
 //     Delta = alpha (c - M dy) + beta (dy - dy_old);  (dy, dy_old) <- (dy + Delta, dy)
 //   conjugate gradient on M dy = c from dy = 0 (Alg. 3's inner solver)
@@ -34,6 +35,7 @@ __device__ void inner_init_body(int method, int n, const double *__restrict__ c,
   s = block_sum(s, scratch);
   if (threadIdx.x == 0) {
     st->rho = s;
+    st->rho_ab[0] = s;
     st->iters = 0;
     st->max_iters = max_iters;
     st->use_thresh = use_thresh;
@@ -76,13 +78,6 @@ __device__ void polyak_body(int n, const double *__restrict__ c, const double *_
   if (threadIdx.x == 0) finish_update(st, s, false);
 }
 
-__global__ void __launch_bounds__(kVecThreads)
-    polyak_update_kernel(int n, const double *__restrict__ c, const double *__restrict__ w,
-                         double *dy, double *dy_old, DevState *st) {
-  if (*(volatile int *)&st->done) return;
-  polyak_body(n, c, w, dy, dy_old, st);
-}
-
 __device__ void cg_body(int n, const double *__restrict__ q, double *p, double *res, double *dy,
                         DevState *st) {
   __shared__ double scratch[32];
@@ -109,13 +104,6 @@ __device__ void cg_body(int n, const double *__restrict__ q, double *p, double *
     st->rho = rr;
     finish_update(st, ss, !(rr > 0.0));
   }
-}
-
-__global__ void __launch_bounds__(kVecThreads)
-    cg_update_kernel(int n, const double *__restrict__ q, double *p, double *res, double *dy,
-                     DevState *st) {
-  if (*(volatile int *)&st->done) return;
-  cg_body(n, q, p, res, dy, st);
 }
 
 // Batched forms (one CTA per item, lsq_batch.cu).  b_init: at step 0 the
@@ -214,18 +202,6 @@ cudaError_t launch_inner_init(int method, int n, const double *c, double *dy, do
                               DevState *st, cudaStream_t s) {
   inner_init_kernel<<<1, kVecThreads, 0, s>>>(method, n, c, dy, dy_old, res, p, max_iters,
                                               use_thresh, st);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_polyak_update(int n, const double *c, const double *w, double *dy,
-                                 double *dy_old, DevState *st, cudaStream_t s) {
-  polyak_update_kernel<<<1, kVecThreads, 0, s>>>(n, c, w, dy, dy_old, st);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cg_update(int n, const double *q, double *p, double *res, double *dy,
-                             DevState *st, cudaStream_t s) {
-  cg_update_kernel<<<1, kVecThreads, 0, s>>>(n, q, p, res, dy, st);
   return cudaGetLastError();
 }
 

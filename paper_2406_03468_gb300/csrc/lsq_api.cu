@@ -47,7 +47,8 @@ lsq_status fail(lsq_status st, const std::string &msg) {
 
 constexpr uint64_t kBarrierTimeoutNs = 5ull * 1000 * 1000 * 1000;  // 5 s per inter-CTA wait
 constexpr int kCondestIters = 10;
-constexpr int kStopPollEvery = 4;  // step 1: read the device stop flag every 4 updates
+constexpr int kStopPollEvery = 4;  // many right-hand sides, step 1: read the stop flag every 4 updates
+constexpr int kRunAhead = 3;       // step 1: updates enqueued beyond the one the device has finished
 constexpr int kHostChunksMax = 16;             // host entry: row chunks of A at most
 constexpr double kHostChunkBytes = 128.0e6;    // and at least this many bytes each
 
@@ -80,6 +81,9 @@ struct lsq_plan_s {
   double *SAb = nullptr, *W = nullptr, *part = nullptr, *r2part = nullptr, *cpart = nullptr;
   double *dcol = nullptr, *dinv = nullptr, *Rcm = nullptr, *Rrm = nullptr, *rinv = nullptr;
   double *Dt = nullptr;  // scaled diagonal blocks of R (launch_diag_tiles)
+  double *Xcm = nullptr, *Xrm = nullptr;  // R^-1 (launch_tri_inv), the inner iterations' operator
+  double *res2 = nullptr, *p2 = nullptr, *pn = nullptr;  // second buffers and partials (InnerVecs)
+  int *hprog = nullptr;  // page-locked: the inner loop's progress word, written by the device
   double *t = nullptr, *vbuf = nullptr;
   double *xs = nullptr, *xo = nullptr, *c = nullptr, *g = nullptr, *dy = nullptr;
   double *dyold = nullptr, *z = nullptr, *h = nullptr, *w = nullptr, *res = nullptr, *p = nullptr;
@@ -285,6 +289,32 @@ lsq_status read_state(lsq_plan P) {
   return LSQ_OK;
 }
 
+// Wait until the device has finished update `need` of the running inner loop
+// or stopped it (*done); no synchronisation, so the iterations behind it stay
+// enqueued.  The stream running empty first means the loop never started
+// (done before the first update) or an error: the state tells.
+lsq_status wait_progress(lsq_plan P, int need, bool *done) {
+  volatile const int *hp = P->hprog;
+  for (int spin = 0;; spin++) {
+    const int v = *hp;
+    if (v & kProgDone) {
+      *done = true;
+      return LSQ_OK;
+    }
+    if (v >= need) return LSQ_OK;
+    if ((spin & 255) == 255) {
+      const cudaError_t q = cudaStreamQuery(P->s);
+      if (q == cudaErrorNotReady) continue;
+      LSQ_CU(q);
+      if (*hp == v) {
+        LSQ_TRY(read_state(P));
+        *done = P->st_host->done != 0;
+        return LSQ_OK;
+      }
+    }
+  }
+}
+
 // Timing events (opt-in): a growing pool of begin/end pairs.
 cudaError_t tev_pair(lsq_plan P, int *idx) {
   while ((int)P->tev.size() < 2 * (P->tev_used + 1)) {
@@ -405,7 +435,7 @@ lsq_status do_sketch(lsq_plan P, const double *dA, const double *db, bool defer_
   LSQ_CU(launch_sketch_finalize(P->cpart, P->gpass, P->npad, n, P->d, P->zeta, P->o.col_scale,
                                 P->SAb, P->W, P->dcol, P->dinv, P->st, P->s));
   LSQ_CU(cudaEventRecord(P->ev[1], P->s));
-  P->launches += 3 + 5;  // sketch, colnorm, transpose; qr, extract, tiles, condest, x0 solve
+  P->launches += 3 + 6;  // sketch, colnorm, transpose; qr, extract, tiles, inverse, condest, x0
   if (P->stepwise_qr)
     LSQ_CU(launch_qr_stepwise(P->W, P->d, n, n + 1, P->vbuf, qr_step_grid(n + 1, P->nsm), P->s));
   else
@@ -415,6 +445,7 @@ lsq_status do_sketch(lsq_plan P, const double *dA, const double *db, bool defer_
   LSQ_CU(launch_diag_tiles(P->Rcm, P->Rrm, P->rinv, n, P->Dt, P->s));
   LSQ_CU(cudaEventRecord(P->ev_fork, P->s));
   LSQ_CU(cudaStreamWaitEvent(P->s2, P->ev_fork, 0));
+  LSQ_CU(launch_tri_inv(P->Rcm, P->rinv, P->Dt, n, P->Xcm, P->Xrm, P->s2));
   LSQ_CU(launch_condest(P->Rcm, P->Rrm, P->rinv, P->Dt, n, kCondestIters, P->st, P->s2));
   LSQ_CU(cudaEventRecord(P->ev_join, P->s2));
   P->condest_pending = true;
@@ -562,12 +593,14 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
     // pass's operator holds A to 2^-48, which leaves step 2's answer a few u
     // ||A||_F from backward stable on kappa ~ 1e12 problems, above the bound.
     const bool df = P->use_df && !kw, eft = P->use_eft && !kw;
+    // the step's first z = D^{-1} R^{-1} (dy or p)
+    const InnerVecs iv = {n, P->Xcm, P->Xrm, P->dinv, P->h, P->c, P->w, P->z, P->dy, P->dyold,
+                          {P->res, P->res2}, {P->p, P->p2}, P->pn, P->st, P->hprog};
+    LSQ_CU(launch_inner_z(method, iv, P->s));
+    P->launches++;
+    *P->hprog = 0;  // every earlier update has finished (the step before ended in read_state)
     for (int it = 0; it < cap; it++) {
-      const double *src = (method == 0) ? P->dy : P->p;
-      // z = D^{-1} R^{-1} src;  h = D^{-1} A^T (A z);  w = R^{-T} h
-      LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 0, src, nullptr, nullptr, P->dinv, P->z,
-                         nullptr, nullptr, P->st, P->s, 1, 0,
-                       &P->st->err));
+      // h = D^{-1} A^T (A z);  w = R^{-T} h, the update, the next z
       int tj = -1;
       if (P->o.timing) {
         LSQ_CU(tev_pair(P, &tj));
@@ -601,22 +634,16 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
         LSQ_CU(launch_pass_atax(dA, P->lda, P->m, n, P->z, P->part, P->gpass, P->npad, P->st,
                                 P->s));
       if (tj >= 0) LSQ_CU(cudaEventRecord(P->tev[2 * tj + 1], P->s));
-      P->launches += 5;
+      P->launches += 4;
       LSQ_CU(launch_reduce(P->part, P->gpass, P->npad, n, P->dinv, P->h,
                            method == 2 ? P->r2part : nullptr,
                            method == 2 ? &P->st->lq_b2 : nullptr, P->st, P->s));
-      LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 1, P->h, nullptr, P->w, nullptr, nullptr,
-                         nullptr, nullptr, P->st, P->s, 1, 0,
-                       &P->st->err));
-      if (method == 0)
-        LSQ_CU(launch_polyak_update(n, P->c, P->w, P->dy, P->dyold, P->st, P->s));
-      else if (method == 1)
-        LSQ_CU(launch_cg_update(n, P->w, P->p, P->res, P->dy, P->st, P->s));
-      else
-        LSQ_CU(launch_lsqr_update(n, P->w, P->p, P->res, P->dy, P->st, P->s));
-      if (use_thresh && (it % kStopPollEvery) == kStopPollEvery - 1 && it + 1 < cap) {
-        LSQ_TRY(read_state(P));
-        if (P->st_host->done) break;
+      LSQ_CU(launch_inner_w(method, iv, it & 1, P->s));
+      LSQ_CU(launch_inner_u(method, iv, it & 1, P->s));
+      if (use_thresh && it + 1 >= kRunAhead && it + 1 < cap) {
+        bool done = false;
+        LSQ_TRY(wait_progress(P, it + 1 - kRunAhead, &done));
+        if (done) break;
       }
       if (kw && it % 5 == 0) {
         // x_hat = x_s + R^{-1} dy (scaled) and D^{-1} x_hat, then the estimate
@@ -896,7 +923,7 @@ void free_plan(lsq_plan P) {
                   P->dyold, P->z, P->h, P->w, P->res, P->p, P->st, P->qflag, P->stageA,
                   P->stageb, P->stagex, P->Ahi, P->Alo, P->SBb, P->cpartB, P->mpart, P->mpartdf, P->mr2part,
                   P->mT, P->mXs, P->mXo, P->mC, P->mG, P->mDY, P->mDYold, P->mZ, P->mH,
-                  P->mW, P->mstate, P->tcnt, P->tlmax, P->colexp, P->cshift,
+                  P->mW, P->mstate, P->Xcm, P->Xrm, P->res2, P->p2, P->pn, P->tcnt, P->tlmax, P->colexp, P->cshift,
                   P->tptr, P->tsrc, P->cpow, P->Qfix, P->Qbfix, P->lsqr_s, P->W2, P->R2cm,
                   P->R2rm, P->rinv2, P->Dt2, P->vhead2, P->xk, P->xko, P->gk, P->qflag2,
                   P->part2};
@@ -904,6 +931,7 @@ void free_plan(lsq_plan P) {
     if (b) cudaFree(b);
   if (P->st_host) cudaFreeHost(P->st_host);
   if (P->dcol_host) cudaFreeHost(P->dcol_host);
+  if (P->hprog) cudaFreeHost(P->hprog);
   for (auto &e : P->ev)
     if (e) cudaEventDestroy(e);
   if (P->ev_fork) cudaEventDestroy(P->ev_fork);
@@ -1004,6 +1032,11 @@ lsq_status lsq_plan_create(const lsq_options *opt, void *cuda_stream, lsq_plan *
   A(dalloc(&P->Rcm, nn));
   A(dalloc(&P->Rrm, nn));
   A(dalloc(&P->rinv, n));
+  A(dalloc(&P->Xcm, nn));
+  A(dalloc(&P->Xrm, nn));
+  A(dalloc(&P->res2, n));
+  A(dalloc(&P->p2, n));
+  A(dalloc(&P->pn, (size_t)inner_partials(n)));
   A(dalloc(&P->Dt, (size_t)2 * ((n + 31) / 32) * 1024));
   A(dalloc(&P->t, n));
   A(dalloc(&P->vbuf, 2 * (size_t)P->d_cap));
@@ -1025,6 +1058,7 @@ lsq_status lsq_plan_create(const lsq_options *opt, void *cuda_stream, lsq_plan *
   A(dalloc(&P->part2, (size_t)P->gpass * 2 * P->npad));
   A(cudaMallocHost((void **)&P->st_host, sizeof(DevState)));
   A(cudaMallocHost((void **)&P->dcol_host, sizeof(double) * n));
+  A(cudaMallocHost((void **)&P->hprog, sizeof(int)));
   // hi / lo FP32 planes of A: the double-float inner pass and the FP32 tier read them
   if (!P->o.sparse && (!P->o.inner_fp64_fma || P->o.precision == LSQ_PREC_AUTO ||
                        P->o.precision == LSQ_PREC_FP32_INNER)) {

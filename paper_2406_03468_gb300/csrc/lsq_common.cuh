@@ -19,6 +19,7 @@ constexpr int kPassCtasPerSm = 2;
 constexpr int kCsrCtasPerSm = 5;                // CTAs per SM of a sparse plan's pass grid
 constexpr int kVecThreads = 1024;               // threads of the single-CTA vector kernels
 constexpr int kMaxZeta = 32;
+constexpr int kProgDone = 1 << 30;              // progress word: the inner loop has stopped
 
 // Device-resident scalars of one solve.  Kernels of the inner loop read
 // `done` first and return at once when it is set, so the host may enqueue a
@@ -41,9 +42,11 @@ struct DevState {
   int zero_col;          // a column norm is zero
   int q2;                // batched solves: the step-2 update count (Theorem 7.1's q0 - 1)
   // LSQR (LSQR-based SPIR): the bidiagonalisation's alpha, beta, the
-  // rotation's phibar, rhobar, the next pass's coefficient of s, and the
-  // last pass's ||s||^2
-  double lq_alpha, lq_beta, lq_phibar, lq_rhobar, lq_bscale, lq_b2;
+  // rotation's phibar, rhobar (by the iteration's parity), the next pass's
+  // coefficient of s, and the last pass's ||s||^2
+  double lq_alpha, lq_beta, lq_phibar[2], lq_rhobar[2], lq_bscale, lq_b2;
+  double rho_ab[2];      // CG on a plan: r^T r by the iteration's parity
+  int ugate;             // `done` as the reduction before the small kernels saw it (k_inner.cu)
   // sketched Karlson-Walden estimate (Alg. 4's step-2 test): ||b||^2, and
   // for the iterate checked ||x||^2 (scaled coordinates), ||r||^2, the
   // factor theta / sqrt(1 + theta^2 ||x||^2), ||R_lam^-T g||^2, the estimate
@@ -80,15 +83,21 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // Sum over the block; every thread gets the result.  `scratch` needs
 // blockDim.x / 32 doubles of shared memory.  Fixed order for a fixed blockDim.
+// Warp 0 alone adds the warps' sums (a butterfly of 5 adds): with every warp
+// adding all of them, 32 warps put 32 x 32 FP64 warp instructions of 64 cycles
+// on the SM's four sub-partitions, 8 us per sum.
 __device__ __forceinline__ double block_sum(double v, double *scratch) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   v = warp_sum(v);
   __syncthreads();
   if (lane == 0) scratch[warp] = v;
   __syncthreads();
-  double s = 0.0;
-  for (int w = 0; w < nw; w++) s += scratch[w];
-  return s;
+  if (warp == 0) {
+    const double s = warp_sum(lane < nw ? scratch[lane] : 0.0);
+    if (lane == 0) scratch[0] = s;
+  }
+  __syncthreads();
+  return scratch[0];
 }
 
 __device__ __forceinline__ uint64_t global_ns() {
@@ -313,9 +322,10 @@ cudaError_t launch_pass_resid_dot2(const double *A, int64_t lda, int64_t m, int 
 cudaError_t launch_reduce_dot2(const double *part2, int grid, int npad, int n, const double *scale,
                                double *out, const double *r2_part, double *r2, cudaStream_t s);
 // out[j] = scale[j] * sum_g part[g][j] (scale may be NULL); r2 (if non-NULL)
-// = sum_g r2_part[g]; gated.
+// = sum_g r2_part[g].  gate: the inner loop's form, a programmatic dependent
+// of the pass that copies gate->done to gate->ugate and returns when it is set.
 cudaError_t launch_reduce(const double *part, int grid, int npad, int n, const double *scale,
-                          double *out, const double *r2_part, double *r2, const DevState *gate,
+                          double *out, const double *r2_part, double *r2, DevState *gate,
                           cudaStream_t s);
 int pass_npad(int n);
 
@@ -354,9 +364,6 @@ cudaError_t launch_pass_lsqr_df(const float *Ahi, const float *Alo, int64_t ld32
 // ||r_i||^2 = st->r2): v = w = c / ||c||, dy = 0, the scalars in st.
 cudaError_t launch_lsqr_init(int n, const double *c, int step, double *v, double *w, double *dy,
                              int max_iters, int use_thresh, DevState *st, cudaStream_t s);
-// One LSQR iteration from p = R^{-T} D^{-1} A^T s and st->lq_b2 (gated).
-cudaError_t launch_lsqr_update(int n, const double *p, double *v, double *w, double *dy,
-                               DevState *st, cudaStream_t s);
 
 // Batched phases (lsq_batch.cu): every launch covers all `count` items of
 // the table; row-parallel launches take `grid` CTAs, CTA g working on item
@@ -414,14 +421,33 @@ cudaError_t launch_kw_build(const double *Rcm, int n, const double *dcol, const 
 cudaError_t launch_kw_finish(DevState *st, cudaStream_t s);
 cudaError_t launch_scale_vec(int n, const double *sc, const double *x, double *y, cudaStream_t s);
 
+// The inner iteration's small kernels (k_inner.cu).  X = R^-1 in both
+// layouts (n x n, upper triangle), from R, 1 / R_ii and the diagonal tiles.
+cudaError_t launch_tri_inv(const double *Rcm, const double *rinv, const double *Dt, int n,
+                           double *Xcm, double *Xrm, cudaStream_t s);
+struct InnerVecs {
+  int n;
+  const double *Xcm, *Xrm, *dinv;
+  const double *h;        // D^-1 A^T (A z), from the reduction
+  const double *c;        // the step's right-hand side
+  double *w, *z, *dy, *dyold;
+  double *res[2], *p[2];  // CG: r and p by parity; LSQR: w by parity, v = p[0]
+  double *pn;             // inner_partials(n) partial sums
+  DevState *st;
+  int *hprog;             // progress word in page-locked host memory (may be NULL)
+};
+int inner_partials(int n);
+// First half of the update of iteration `par` (its parity), after the
+// reduction; second half and the next z; the step's first z (after
+// launch_inner_init / launch_lsqr_init).
+cudaError_t launch_inner_w(int method, const InnerVecs &v, int par, cudaStream_t s);
+cudaError_t launch_inner_u(int method, const InnerVecs &v, int par, cudaStream_t s);
+cudaError_t launch_inner_z(int method, const InnerVecs &v, cudaStream_t s);
+
 // Inner-solver kernels (single CTA).
 cudaError_t launch_inner_init(int method, int n, const double *c, double *dy, double *dy_old,
                               double *res, double *p, int max_iters, int use_thresh,
                               DevState *st, cudaStream_t s);
-cudaError_t launch_polyak_update(int n, const double *c, const double *w, double *dy,
-                                 double *dy_old, DevState *st, cudaStream_t s);
-cudaError_t launch_cg_update(int n, const double *q, double *p, double *res, double *dy,
-                             DevState *st, cudaStream_t s);
 // thresh1 = u (gamma normest ||x0|| + rho condest sqrt(r2)); records cnorm2[0].
 cudaError_t launch_set_thresh(double gamma, double rho, DevState *st, cudaStream_t s);
 

@@ -10,6 +10,41 @@
 
 namespace lsq {
 
+// Programmatic dependent launch: let the next kernel of the stream take its
+// slots, and wait until the previous ones have completed (a no-op in a
+// kernel that was launched without the attribute).
+__device__ __forceinline__ void griddep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// A load that stays on its side of griddep_wait: the compiler may move an
+// ordinary read-only load down to its first use.
+__device__ __forceinline__ double ld_early(const double *p) {
+  double v;
+  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+// Launch as a programmatic dependent of the kernel before it in the stream.
+// Such a kernel calls griddep_wait before it touches anything that an
+// earlier kernel of the chain writes, or that an earlier one still reads.
+template <typename... K, typename... T>
+cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       T... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
 // Knuth's TwoSum: s + e = a + b exactly.
 __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) {
   s = __fadd_rn(a, b);

@@ -217,7 +217,8 @@ __device__ double block_normalize(double *sv, int n, double *scratch) {
 }
 
 // sigma_max(R) by power iteration on R^T R and sigma_min(R) by inverse power
-// iteration on (R^T R)^{-1}, from a fixed start vector.
+// iteration on (R^T R)^{-1}, from a fixed start vector (the batched engine's
+// items; a plan's estimate is launch_condest in k_inner.cu).
 __device__ void condest_body(const double *__restrict__ Rcm, const double *__restrict__ Rrm,
                              const double *__restrict__ rinv, const double *__restrict__ Dt, int n,
                              int iters, DevState *st, double *sm) {
@@ -250,14 +251,6 @@ __device__ void condest_body(const double *__restrict__ Rcm, const double *__res
     st->normest = smax;
     st->condest = (smin > 0.0) ? smax / smin : INFINITY;
   }
-}
-
-__global__ void __launch_bounds__(kVecThreads)
-    condest_kernel(const double *__restrict__ Rcm, const double *__restrict__ Rrm,
-                   const double *__restrict__ rinv, const double *__restrict__ Dt, int n, int iters,
-                   DevState *st) {
-  extern __shared__ double sm[];
-  condest_body(Rcm, Rrm, rinv, Dt, n, iters, st, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -640,13 +633,6 @@ cudaError_t launch_b_trsv(const BItem *items, int count, int mode, int step, int
   cudaError_t e = ensure_smem_attr((const void *)b_trsv_kernel, (int)smem);
   if (e != cudaSuccess) return e;
   b_trsv_kernel<<<count, kVecThreads, smem, s>>>(items, mode, step);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_condest(const double *Rcm, const double *Rrm, const double *rinv,
-                           const double *Dt, int n, int iters, DevState *st, cudaStream_t s) {
-  const size_t smem = (size_t)(2 * n + 32 + 3 * kTile) * sizeof(double);
-  condest_kernel<<<1, kVecThreads, smem, s>>>(Rcm, Rrm, rinv, Dt, n, iters, st);
   return cudaGetLastError();
 }
 

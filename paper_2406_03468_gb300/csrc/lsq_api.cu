@@ -83,6 +83,7 @@ struct lsq_plan_s {
   double *Dt = nullptr;  // scaled diagonal blocks of R (launch_diag_tiles)
   double *Xcm = nullptr, *Xrm = nullptr;  // R^-1 (launch_tri_inv), the inner iterations' operator
   double *res2 = nullptr, *p2 = nullptr, *pn = nullptr;  // second buffers and partials (InnerVecs)
+  double *cwork = nullptr;  // condition estimate's vectors (cond_work)
   int *hprog = nullptr;  // page-locked: the inner loop's progress word, written by the device
   double *t = nullptr, *vbuf = nullptr;
   double *xs = nullptr, *xo = nullptr, *c = nullptr, *g = nullptr, *dy = nullptr;
@@ -435,7 +436,8 @@ lsq_status do_sketch(lsq_plan P, const double *dA, const double *db, bool defer_
   LSQ_CU(launch_sketch_finalize(P->cpart, P->gpass, P->npad, n, P->d, P->zeta, P->o.col_scale,
                                 P->SAb, P->W, P->dcol, P->dinv, P->st, P->s));
   LSQ_CU(cudaEventRecord(P->ev[1], P->s));
-  P->launches += 3 + 6;  // sketch, colnorm, transpose; qr, extract, tiles, inverse, condest, x0
+  // sketch, colnorm, transpose; qr, extract, tiles, inverse, x0; the condition estimate's steps
+  P->launches += 3 + 5 + 2 * kCondestIters + 2;
   if (P->stepwise_qr)
     LSQ_CU(launch_qr_stepwise(P->W, P->d, n, n + 1, P->vbuf, qr_step_grid(n + 1, P->nsm), P->s));
   else
@@ -446,7 +448,7 @@ lsq_status do_sketch(lsq_plan P, const double *dA, const double *db, bool defer_
   LSQ_CU(cudaEventRecord(P->ev_fork, P->s));
   LSQ_CU(cudaStreamWaitEvent(P->s2, P->ev_fork, 0));
   LSQ_CU(launch_tri_inv(P->Rcm, P->rinv, P->Dt, n, P->Xcm, P->Xrm, P->s2));
-  LSQ_CU(launch_condest(P->Rcm, P->Rrm, P->rinv, P->Dt, n, kCondestIters, P->st, P->s2));
+  LSQ_CU(launch_condest(P->Rcm, P->Rrm, P->Xcm, P->Xrm, n, kCondestIters, P->cwork, P->st, P->s2));
   LSQ_CU(cudaEventRecord(P->ev_join, P->s2));
   P->condest_pending = true;
   // sketch-and-solve x0 = R^{-1} t (scaled coordinates) and x0 / d (original)
@@ -775,11 +777,12 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
                    qr_grid(n + k, P->nsm), qr_timeout_ns(P), P->s, &P->qb));
   LSQ_CU(launch_extract_r(P->W, d, n, k, P->Rcm, P->Rrm, P->rinv, P->mT, P->s));
   LSQ_CU(launch_diag_tiles(P->Rcm, P->Rrm, P->rinv, n, P->Dt, P->s));
-  LSQ_CU(launch_condest(P->Rcm, P->Rrm, P->rinv, P->Dt, n, kCondestIters, P->st, P->s));
+  LSQ_CU(launch_tri_inv(P->Rcm, P->rinv, P->Dt, n, P->Xcm, P->Xrm, P->s));
+  LSQ_CU(launch_condest(P->Rcm, P->Rrm, P->Xcm, P->Xrm, n, kCondestIters, P->cwork, P->st, P->s));
   LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 0, P->mT, nullptr, P->mXs, P->dinv, P->mXo,
                      nullptr, x0n2, nullptr, P->s, k, n));
   LSQ_CU(cudaEventRecord(P->ev[2], P->s));
-  P->launches += 12;
+  P->launches += 12 + 2 * kCondestIters + 2;
   LSQ_CU(cudaMemcpyAsync(P->dcol_host, P->dcol, sizeof(double) * n, cudaMemcpyDeviceToHost, P->s));
   LSQ_TRY(read_state(P));
   // the inner pass: all k vectors through the double-float pass on the planes
@@ -923,7 +926,7 @@ void free_plan(lsq_plan P) {
                   P->dyold, P->z, P->h, P->w, P->res, P->p, P->st, P->qflag, P->stageA,
                   P->stageb, P->stagex, P->Ahi, P->Alo, P->SBb, P->cpartB, P->mpart, P->mpartdf, P->mr2part,
                   P->mT, P->mXs, P->mXo, P->mC, P->mG, P->mDY, P->mDYold, P->mZ, P->mH,
-                  P->mW, P->mstate, P->Xcm, P->Xrm, P->res2, P->p2, P->pn, P->tcnt, P->tlmax, P->colexp, P->cshift,
+                  P->mW, P->mstate, P->Xcm, P->Xrm, P->res2, P->p2, P->pn, P->cwork, P->tcnt, P->tlmax, P->colexp, P->cshift,
                   P->tptr, P->tsrc, P->cpow, P->Qfix, P->Qbfix, P->lsqr_s, P->W2, P->R2cm,
                   P->R2rm, P->rinv2, P->Dt2, P->vhead2, P->xk, P->xko, P->gk, P->qflag2,
                   P->part2};
@@ -1037,6 +1040,7 @@ lsq_status lsq_plan_create(const lsq_options *opt, void *cuda_stream, lsq_plan *
   A(dalloc(&P->res2, n));
   A(dalloc(&P->p2, n));
   A(dalloc(&P->pn, (size_t)inner_partials(n)));
+  A(dalloc(&P->cwork, cond_work(n)));
   A(dalloc(&P->Dt, (size_t)2 * ((n + 31) / 32) * 1024));
   A(dalloc(&P->t, n));
   A(dalloc(&P->vbuf, 2 * (size_t)P->d_cap));

@@ -239,9 +239,6 @@ cudaError_t launch_qr_stepwise(double *W, int d, int n, int ncols, double *vhead
 // R (upper n x n of W) to Rcm / Rrm, 1/R_ii, t = W[0:n, n:n+nb] (column-major n x nb).
 cudaError_t launch_extract_r(const double *W, int d, int n, int nb, double *Rcm, double *Rrm,
                              double *rinv, double *t, cudaStream_t s);
-// condest / normest of R by power and inverse power iteration.
-cudaError_t launch_condest(const double *Rcm, const double *Rrm, const double *rinv,
-                           const double *Dt, int n, int iters, DevState *st, cudaStream_t s);
 // Dt (2 ceil(n/32) 1024 doubles): the diagonal 32 x 32 blocks of R for both
 // solve directions with each entry scaled by 1 / R_ll of the row it updates
 // (the triangular solves run the block chains on these).
@@ -425,6 +422,12 @@ cudaError_t launch_scale_vec(int n, const double *sc, const double *x, double *y
 // layouts (n x n, upper triangle), from R, 1 / R_ii and the diagonal tiles.
 cudaError_t launch_tri_inv(const double *Rcm, const double *rinv, const double *Dt, int n,
                            double *Xcm, double *Xrm, cudaStream_t s);
+// condest / normest of R into st by power iteration with R and, for
+// sigma_min, with X = R^-1; work: cond_work(n) doubles.
+size_t cond_work(int n);
+cudaError_t launch_condest(const double *Rcm, const double *Rrm, const double *Xcm,
+                           const double *Xrm, int n, int iters, double *work, DevState *st,
+                           cudaStream_t s);
 struct InnerVecs {
   int n;
   const double *Xcm, *Xrm, *dinv;

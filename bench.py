@@ -327,15 +327,12 @@ KERNEL_SRC = os.path.join(ROOT, "paper_2406_03468_gb300", "csrc")
 
 
 def kernel_source_sha256():
-    """sha256 of the inner pass's own source: the atax_df_kernel section of
-    k_pass.cu (from its header comment to the next kernel's) and the device
-    helpers it includes (lsq_dev.cuh).  Edits elsewhere in the library leave
-    it unchanged; any edit to the kernel changes it."""
+    """sha256 of the inner pass's own source: its body (lsq_dfpass.cuh) and the
+    device helpers it includes (lsq_dev.cuh).  Edits elsewhere in the library
+    leave it unchanged; any edit to the kernel changes it."""
     import hashlib
-    src = open(os.path.join(KERNEL_SRC, "k_pass.cu")).read()
-    i = src.index("// Inner pass on the hi / lo FP32 planes of A")
-    j = src.index("// FP32 inner pass of the mixed-precision tier")
-    text = src[i:j] + open(os.path.join(KERNEL_SRC, "lsq_dev.cuh")).read()
+    text = "".join(open(os.path.join(KERNEL_SRC, f)).read()
+                   for f in ("lsq_dfpass.cuh", "lsq_dev.cuh"))
     return hashlib.sha256(text.encode()).hexdigest()
 
 
@@ -824,8 +821,8 @@ def run_ours(args):
 
     # roofline of the dominant kernel: the fused A^T(A z) inner pass
     pk, pk_kind = peaks()
-    kname = {0: "atax_kernel", 1: "atax_eft_kernel", 2: "atax32_kernel",
-             3: "atax_df_kernel"}[infos[-1]["inner_kernel"]]
+    kname = {0: "atax_kernel", 1: "atax_eft_kernel", 2: "df_pass_kernel (FP32 tier)",
+             3: "df_pass_kernel"}[infos[-1]["inner_kernel"]]
     roof = pass_roofline(infos, kname + " (fused A^T(A z) inner pass)", pk, pk_kind,
                          traffic_per_launch())
     passes = statistics.mean(i["passes"] for i in infos)

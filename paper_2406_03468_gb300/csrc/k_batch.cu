@@ -11,14 +11,13 @@
 // item whose inner loop has stopped (st->done), so the launch costs nothing
 // for the items that are done.
 #include "lsq_common.cuh"
-#include "lsq_dev.cuh"
+#include "lsq_dfpass.cuh"
 
 namespace lsq {
 
 namespace {
 
-constexpr int kBThreads = 256;
-constexpr int kBFlush = 32;
+constexpr int kBThreads = kPassThreads;
 
 template <int NC>
 __device__ __forceinline__ void b_load_vec(const double *__restrict__ x, int n, int lane,
@@ -96,176 +95,6 @@ __device__ void b_resid_body(const BItem &it, int local, double *sh, double *r2s
   }
 }
 
-// The inner pass of one item's CTA: the structure of atax_df_kernel (the hi /
-// lo planes staged by TMA bulk copies, kBStages per warp in flight, bounded
-// mbarrier waits, drain on a timeout) over the item's row share.  A stage
-// holds a block of consecutive rows, as many as fit in kBStageFloats floats
-// per plane (16 rows at n = 32, 2 at n = 256), so that short rows still keep
-// about 2 KB per plane and warp in flight; the warp takes its blocks in turn
-// and the rows of a block one after the other.
-// Shared memory: hacc [8 warps][256] FP64, stages [8][kBStages][2][512] FP32,
-// then the mbarriers.
-constexpr int kBStages = 2;
-constexpr int kBStageFloats = 512;
-constexpr uint64_t kBWaitNs = 1000ull * 1000 * 1000;  // 1 s
-constexpr size_t kBInnerSmem =
-    (size_t)(kBThreads / 32) * 256 * sizeof(double) +
-    (size_t)(kBThreads / 32) * kBStages * 2 * kBStageFloats * sizeof(float) +
-    (size_t)(kBThreads / 32) * kBStages * sizeof(uint64_t);
-
-template <int NC>
-__device__ void b_inner_body(const BItem &it, int local, double *hacc, double *wmax) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int n = it.n;
-  const int64_t m = it.m, per = (m + it.ncta - 1) / it.ncta;
-  const int64_t r0 = min(m, (int64_t)local * per), r1 = min(m, r0 + per);
-  float *stages = reinterpret_cast<float *>(hacc + (size_t)nw * 256);
-  uint64_t *bars = reinterpret_cast<uint64_t *>(stages + (size_t)nw * kBStages * 2 * kBStageFloats);
-  float *wst = stages + (size_t)warp * kBStages * 2 * kBStageFloats;
-  uint64_t *wbar = bars + warp * kBStages;
-  const int ld32 = it.ld32;
-  const int rb = kBStageFloats / ld32;  // rows per block (ld32 <= 256: at least 2)
-  const int64_t nblk_all = (r1 - r0 + rb - 1) / rb;
-  const int64_t nblks = (nblk_all - warp + nw - 1) / nw > 0 ? (nblk_all - warp + nw - 1) / nw : 0;
-  if (lane == 0) {
-    for (int st = 0; st < kBStages; st++) mbar_init(wbar + st, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
-  const uint64_t pol = l2_evict_first();
-  // the warp's q-th block: rows r0 + (warp + q nw) rb .. (at most rb, within r1)
-  auto block_rows = [&](int64_t q, int64_t &i0) {
-    i0 = r0 + (warp + q * nw) * (int64_t)rb;
-    return (int)min((int64_t)rb, r1 - i0);
-  };
-  auto issue = [&](int64_t q) {
-    if (lane == 0 && q < nblks) {
-      int64_t i0;
-      const int rows = block_rows(q, i0);
-      const unsigned bytes = (unsigned)(rows * ld32 * sizeof(float));
-      const int stg = (int)(q % kBStages);
-      float *dh = wst + (size_t)stg * 2 * kBStageFloats;
-      mbar_expect_tx(wbar + stg, 2 * bytes);
-      bulk_g2s(dh, it.Ahi + i0 * ld32, bytes, wbar + stg, pol);
-      bulk_g2s(dh + kBStageFloats, it.Alo + i0 * ld32, bytes, wbar + stg, pol);
-    }
-  };
-  for (int64_t q = 0; q < kBStages; q++) issue(q);
-  double *hw = hacc + (size_t)warp * 256;
-  for (int i = lane; i < NC * 64; i += 32) hw[i] = 0.0;
-  double zr[2 * NC];
-  b_load_vec<NC>(it.z, n, lane, zr);
-  double zmax = 0.0;
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) zmax = fmax(zmax, fabs(zr[k]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-  if (lane == 0) wmax[warp] = zmax;
-  __syncthreads();
-  zmax = 0.0;
-  for (int w = 0; w < nw; w++) zmax = fmax(zmax, wmax[w]);
-  int fz = 0;
-  if (zmax > 0.0) frexp(zmax, &fz);
-  const double down = ldexp(1.0, -fz), up = ldexp(1.0, fz);
-  f2_t zh[NC], zl[NC], zn[NC], hh[NC], hl[NC];
-#pragma unroll
-  for (int k = 0; k < NC; k++) {
-    const double v0 = zr[2 * k] * down, v1 = zr[2 * k + 1] * down;
-    const float h0 = __double2float_rn(v0), h1 = __double2float_rn(v1);
-    zh[k] = f2_pack(h0, h1);
-    zl[k] = f2_pack(__double2float_rn(v0 - (double)h0), __double2float_rn(v1 - (double)h1));
-    zn[k] = f2_pack(-h0, -h1);
-    hh[k] = hl[k] = 0ull;
-  }
-  int blk = 0;
-  int64_t qfail = -1;
-  for (int64_t q = 0; q < nblks; q++) {
-    const int stg = (int)(q % kBStages);
-    if (!__all_sync(0xffffffffu, mbar_wait(wbar + stg, (unsigned)((q / kBStages) & 1), kBWaitNs))) {
-      qfail = q;
-      break;
-    }
-    int64_t i0;
-    const int rows = block_rows(q, i0);
-    for (int rr = 0; rr < rows; rr++) {
-    const float *rh = wst + (size_t)stg * 2 * kBStageFloats + (size_t)rr * ld32;
-    const float *rl = rh + kBStageFloats;
-    f2_t ah[NC], al[NC];
-#pragma unroll
-    for (int k = 0; k < NC; k++) {
-      const int col = 64 * k + 2 * lane;
-      if (col + 1 < n) {
-        ah[k] = *reinterpret_cast<const f2_t *>(rh + col);
-        al[k] = *reinterpret_cast<const f2_t *>(rl + col);
-      } else {
-        ah[k] = (col < n) ? f2_pack(rh[col], 0.0f) : 0ull;
-        al[k] = (col < n) ? f2_pack(rl[col], 0.0f) : 0ull;
-      }
-    }
-    if (rr == rows - 1) {
-      // every lane has the block's values: the stage may be refilled
-      __syncwarp();
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(q + kBStages);
-    }
-    f2_t shp = 0ull, slp = 0ull;
-#pragma unroll
-    for (int k = 0; k < NC; k++) f2_dd_step(shp, slp, ah[k], al[k], zh[k], zl[k], zn[k]);
-    float sh_, sl_;
-    {
-      float er;
-      two_sum_f(f2_lo(shp), f2_hi(shp), sh_, er);
-      sl_ = __fadd_rn(__fadd_rn(f2_lo(slp), f2_hi(slp)), er);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, sh_, o);
-      const float ol = __shfl_xor_sync(0xffffffffu, sl_, o);
-      float s, er;
-      two_sum_f(sh_, oh, s, er);
-      sh_ = s;
-      sl_ = __fadd_rn(__fadd_rn(sl_, ol), er);
-    }
-    const float th = __fadd_rn(sh_, sl_);
-    const float tl = __fsub_rn(sl_, __fsub_rn(th, sh_));
-    const f2_t th2 = f2_pack(th, th), tl2 = f2_pack(tl, tl), tn2 = f2_pack(-th, -th);
-#pragma unroll
-    for (int k = 0; k < NC; k++) f2_dd_step(hh[k], hl[k], ah[k], al[k], th2, tl2, tn2);
-    if (++blk == kBFlush) {
-      blk = 0;
-#pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        hw[col] += widen(f2_lo(hh[k])) + widen(f2_lo(hl[k]));
-        hw[col + 1] += widen(f2_hi(hh[k])) + widen(f2_hi(hl[k]));
-        hh[k] = hl[k] = 0ull;
-      }
-    }
-    }  // rows of the block
-  }
-  if (qfail >= 0) {
-    if (lane == 0) {
-      atomicCAS(&it.st->err, 0, (int)LSQ_ERR_TIMEOUT);
-      for (int64_t r = qfail; r < qfail + kBStages && r < nblks; r++)
-        mbar_wait(wbar + (r % kBStages), (unsigned)((r / kBStages) & 1), kBWaitNs);
-    }
-    __syncwarp();
-  }
-#pragma unroll
-  for (int k = 0; k < NC; k++) {
-    const int col = 64 * k + 2 * lane;
-    hw[col] += widen(f2_lo(hh[k])) + widen(f2_lo(hl[k]));
-    hw[col + 1] += widen(f2_hi(hh[k])) + widen(f2_hi(hl[k]));
-  }
-  __syncthreads();
-  double *part = it.part + (size_t)local * it.npad;
-  for (int c = threadIdx.x; c < it.npad; c += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < nw; w++) s += hacc[(size_t)w * 256 + c];
-    part[c] = s * up;
-  }
-}
-
 __global__ void __launch_bounds__(kBThreads, 2)
     b_resid_kernel(const BItem *__restrict__ items, const int *__restrict__ cta_item) {
   __shared__ double sh[4 * 64];
@@ -282,19 +111,29 @@ __global__ void __launch_bounds__(kBThreads, 2)
   }
 }
 
+// The inner pass of one item's CTA over the item's row share (lsq_dfpass.cuh),
+// in the tile its n takes (at most 8 pairs of columns per lane: n <= 256).
 __global__ void __launch_bounds__(kBThreads, 2)
     b_inner_kernel(const BItem *__restrict__ items, const int *__restrict__ cta_item) {
-  extern __shared__ __align__(16) double hacc[];
-  __shared__ double wmax[kBThreads / 32];
+  extern __shared__ __align__(16) double dsm[];
   const int idx = cta_item[blockIdx.x];
   if (idx < 0) return;
   const BItem &it = items[idx];
   if (*(volatile const int *)&it.st->done) return;
   const int local = blockIdx.x - it.cta0;
-  switch (it.npad / 64) {
-    case 1: b_inner_body<1>(it, local, hacc, wmax); break;
-    case 2: b_inner_body<2>(it, local, hacc, wmax); break;
-    case 4: b_inner_body<4>(it, local, hacc, wmax); break;
+  const int64_t per = (it.m + it.ncta - 1) / it.ncta;
+  const int64_t r0 = min(it.m, (int64_t)local * per), r1 = min(it.m, r0 + per);
+  const DfTile t = df_tile(it.n);
+  switch (t.G * 100 + t.P) {
+#define LSQ_BDF(GV, PV)                                                                         \
+  case GV * 100 + PV:                                                                           \
+    df_pass_body<GV, PV, 0>(it.Ahi, it.Alo, it.ld32, r0, r1, it.n, it.z, nullptr, nullptr,      \
+                            it.part + (size_t)local * it.npad, nullptr, it.npad, nullptr,       \
+                            &it.st->err, false, dsm);                                           \
+    break;
+    LSQ_BDF(8, 1) LSQ_BDF(8, 2) LSQ_BDF(8, 3) LSQ_BDF(8, 4) LSQ_BDF(8, 5) LSQ_BDF(8, 6)
+    LSQ_BDF(8, 7) LSQ_BDF(8, 8) LSQ_BDF(16, 5) LSQ_BDF(16, 6) LSQ_BDF(16, 7) LSQ_BDF(16, 8)
+#undef LSQ_BDF
     default: break;
   }
 }
@@ -416,11 +255,11 @@ cudaError_t launch_b_resid(const BItem *items, const int *cta_item, int grid, cu
 }
 
 cudaError_t prepare_b_inner() {
-  return ensure_smem_attr((const void *)b_inner_kernel, (int)kBInnerSmem);
+  return ensure_smem_attr((const void *)b_inner_kernel, (int)df_smem(16, 8, 0));
 }
 
 cudaError_t launch_b_inner(const BItem *items, const int *cta_item, int grid, cudaStream_t s) {
-  b_inner_kernel<<<grid, kBThreads, kBInnerSmem, s>>>(items, cta_item);
+  b_inner_kernel<<<grid, kBThreads, df_smem(16, 8, 0), s>>>(items, cta_item);
   return cudaGetLastError();
 }
 

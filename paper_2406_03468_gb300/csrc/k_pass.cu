@@ -1,4 +1,5 @@
-// The two streaming passes over A of the refinement loop (Alg. 1):
+// The streaming passes over A itself of the refinement loop (Alg. 1; the
+// default inner passes, over the FP32 planes of A, are in k_pass_df.cu):
 //   pass_resid:  r = b - A x,  g = A^T r,  ||r||^2       (refinement RHS)
 //   pass_atax:   h = A^T (A z)                           (inner operator)
 // Each reads A exactly once.  One warp owns one row at a time: 16-byte
@@ -194,349 +195,6 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
 #pragma unroll
   for (int k = 0; k < 2 * NC; k++) h[k] *= up;
   cta_store_partial<NC>(h, sh, part, npad);
-}
-
-// ---------------------------------------------------------------------------
-// Inner pass on the hi / lo FP32 planes of A (written by the sketch pass,
-// a = hi + lo to 2^-48 |a|), all arithmetic on the FP32 pipe:
-//   t_i = sum_j a_ij z_j : TwoProd of hi*z_hi, the cross terms hi*z_lo and
-//         lo*z_hi added to the error word, TwoSum accumulation, double-float
-//         warp reduction;
-//   h_j += a_ij t_i      : the same products against t = t_hi + t_lo, each
-//         column a double-float accumulator (TwoSum into the high word, the
-//         error terms into the low word) flushed into an FP64 shared-memory
-//         accumulator every kDfFlush = 32 rows of the warp.  A flush costs 32
-//         FP64 warp instructions per warp (64 cycles each on its sub-
-//         partition): every 8 rows it held the pass at 0.76 ms, every 32 rows
-//         0.69 ms.  The low word then gathers up to 32 rows of error terms,
-//         a worst-case relative error of about 2^-43 of the sums (2^-45 at 8
-//         rows; every 128 rows, 2^-41, gained only 2% more).
-// The FP64 pipe only sees the flushes (1/8 of an add per element), so the
-// pass is no longer capped by GB300's FP64 rate.  z is scaled by a common
-// power of two 2^-Fz; h is scaled back.
-//
-// Rows reach shared memory by TMA bulk copies (cp.async.bulk with mbarrier
-// completion), kDfStages rows per warp in flight: lane 0 of each warp issues
-// the copies of the rows its warp will process next while the warp computes
-// on the current one, so the bytes in flight no longer depend on registers.
-// Every mbarrier wait is bounded (kDfWaitNs); on a timeout the kernel
-// records LSQ_ERR_TIMEOUT, waits (bounded) for its copies in flight and
-// returns.
-// ---------------------------------------------------------------------------
-constexpr int kDfFlush = 32;
-constexpr int kDfStages = 2;
-constexpr uint64_t kDfWaitNs = 1000ull * 1000 * 1000;  // 1 s
-
-template <int NC>
-__global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
-    atax_df_kernel(const float *__restrict__ Ahi, const float *__restrict__ Alo, int64_t ld32,
-                   int64_t m, int n, const double *__restrict__ z, double *__restrict__ part,
-                   int npad, const DevState *gate, int *err, int64_t zstride,
-                   int64_t pstride) {
-  griddep_launch();
-  // many right-hand sides: grid row blockIdx.y works on vector z_(blockIdx.y)
-  z += (int64_t)blockIdx.y * zstride;
-  part += (int64_t)blockIdx.y * pstride;
-  // dynamic shared memory: [warps][NC*64] FP64 flush accumulators, then
-  // [warps][kDfStages][2][NC*64] FP32 row stages (hi, lo), then the mbarriers
-  extern __shared__ __align__(16) double hacc[];
-  __shared__ double wmax[kPassThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float *stages = reinterpret_cast<float *>(hacc + (size_t)nw * NC * 64);
-  uint64_t *bars = reinterpret_cast<uint64_t *>(stages + (size_t)nw * kDfStages * 2 * NC * 64);
-  float *wst = stages + (size_t)warp * kDfStages * 2 * NC * 64;
-  uint64_t *wbar = bars + warp * kDfStages;
-  const int64_t per = (m + gridDim.x - 1) / gridDim.x;
-  const int64_t r0 = min(m, (int64_t)blockIdx.x * per), r1 = min(m, r0 + per);
-  const int64_t nrows = (r1 - r0 - warp + nw - 1) / nw > 0 ? (r1 - r0 - warp + nw - 1) / nw : 0;
-  const unsigned row_bytes = (unsigned)(ld32 * sizeof(float));
-  if (lane == 0) {
-    for (int st = 0; st < kDfStages; st++) mbar_init(wbar + st, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
-  // lane 0: bulk copies of the warp's q-th row (hi and lo) into stage q % kDfStages
-  const uint64_t pol = l2_evict_first();
-  auto issue = [&](int64_t q) {
-    if (lane == 0 && q < nrows) {
-      const int64_t i = r0 + warp + q * nw;
-      const int stg = (int)(q % kDfStages);
-      float *dh = wst + (size_t)stg * 2 * NC * 64;
-      mbar_expect_tx(wbar + stg, 2 * row_bytes);
-      bulk_g2s(dh, Ahi + i * ld32, row_bytes, wbar + stg, pol);
-      bulk_g2s(dh + NC * 64, Alo + i * ld32, row_bytes, wbar + stg, pol);
-    }
-  };
-  // the planes were complete before the inner loop began: the first rows are
-  // on their way while the kernel that forms z ends
-  for (int64_t q = 0; q < kDfStages; q++) issue(q);
-
-  double *hw = hacc + (size_t)warp * NC * 64;
-  for (int i = lane; i < NC * 64; i += 32) hw[i] = 0.0;
-  griddep_wait();
-  if (gate != nullptr && *(volatile const int *)&gate->done) {
-    if (lane == 0)  // the copies in flight land before the CTA's memory is released
-      for (int64_t q = 0; q < kDfStages && q < nrows; q++) mbar_wait(wbar + q, 0, kDfWaitNs);
-    return;
-  }
-  double zr[2 * NC];
-  load_vec<NC>(z, n, lane, zr);
-  double zmax = 0.0;
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) zmax = fmax(zmax, fabs(zr[k]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-  if (lane == 0) wmax[warp] = zmax;
-  __syncthreads();
-  zmax = 0.0;
-  for (int w = 0; w < nw; w++) zmax = fmax(zmax, wmax[w]);
-  int fz = 0;
-  if (zmax > 0.0) frexp(zmax, &fz);
-  const double down = ldexp(1.0, -fz), up = ldexp(1.0, fz);
-  // column pairs (2k, 2k + 1) of this lane: z hi / lo / -hi and the
-  // double-float column sums, packed
-  f2_t zh[NC], zl[NC], zn[NC], hh[NC], hl[NC];
-#pragma unroll
-  for (int k = 0; k < NC; k++) {
-    const double v0 = zr[2 * k] * down, v1 = zr[2 * k + 1] * down;
-    const float h0 = __double2float_rn(v0), h1 = __double2float_rn(v1);
-    zh[k] = f2_pack(h0, h1);
-    zl[k] = f2_pack(__double2float_rn(v0 - (double)h0), __double2float_rn(v1 - (double)h1));
-    zn[k] = f2_pack(-h0, -h1);
-    hh[k] = hl[k] = 0ull;
-  }
-  int blk = 0;
-  int64_t qfail = -1;
-  for (int64_t q = 0; q < nrows; q++) {
-    const int stg = (int)(q % kDfStages);
-    // one decision per warp: a lane whose wait ran out takes the whole warp
-    // to the drain below
-    if (!__all_sync(0xffffffffu, mbar_wait(wbar + stg, (unsigned)((q / kDfStages) & 1), kDfWaitNs))) {
-      qfail = q;
-      break;
-    }
-    const float *rh = wst + (size_t)stg * 2 * NC * 64;
-    const float *rl = rh + NC * 64;
-    f2_t ah[NC], al[NC];
-#pragma unroll
-    for (int k = 0; k < NC; k++) {
-      const int col = 64 * k + 2 * lane;
-      if (col + 1 < n) {
-        ah[k] = *reinterpret_cast<const f2_t *>(rh + col);
-        al[k] = *reinterpret_cast<const f2_t *>(rl + col);
-      } else {
-        ah[k] = (col < n) ? f2_pack(rh[col], 0.0f) : 0ull;
-        al[k] = (col < n) ? f2_pack(rl[col], 0.0f) : 0ull;
-      }
-    }
-    // every lane has its values: the stage may be refilled (generic reads
-    // before the async-proxy writes of the next copy)
-    __syncwarp();
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    issue(q + kDfStages);
-    // two independent double-float accumulators (even / odd column, the
-    // halves of one packed pair) halve the dependent TwoSum chain
-    f2_t shp = 0ull, slp = 0ull;
-#pragma unroll
-    for (int k = 0; k < NC; k++) f2_dd_step(shp, slp, ah[k], al[k], zh[k], zl[k], zn[k]);
-    float sh_, sl_;
-    {
-      float er;
-      two_sum_f(f2_lo(shp), f2_hi(shp), sh_, er);
-      sl_ = __fadd_rn(__fadd_rn(f2_lo(slp), f2_hi(slp)), er);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, sh_, o);
-      const float ol = __shfl_xor_sync(0xffffffffu, sl_, o);
-      float s, er;
-      two_sum_f(sh_, oh, s, er);
-      sh_ = s;
-      sl_ = __fadd_rn(__fadd_rn(sl_, ol), er);
-    }
-    // renormalise t (Fast2Sum: |sh_| >= |sl_| after the sums above)
-    const float th = __fadd_rn(sh_, sl_);
-    const float tl = __fsub_rn(sl_, __fsub_rn(th, sh_));
-    // column sums: TwoSum into the high word, error terms into the low word;
-    // the low word only gathers kDfFlush rows of small terms before the FP64
-    // flush, so it is not renormalised row by row
-    const f2_t th2 = f2_pack(th, th), tl2 = f2_pack(tl, tl), tn2 = f2_pack(-th, -th);
-#pragma unroll
-    for (int k = 0; k < NC; k++) f2_dd_step(hh[k], hl[k], ah[k], al[k], th2, tl2, tn2);
-    if (++blk == kDfFlush) {
-      blk = 0;
-#pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        hw[col] += widen(f2_lo(hh[k])) + widen(f2_lo(hl[k]));
-        hw[col + 1] += widen(f2_hi(hh[k])) + widen(f2_hi(hl[k]));
-        hh[k] = hl[k] = 0ull;
-      }
-    }
-  }
-  if (qfail >= 0) {
-    // record the error; let the copies this warp has in flight (rows qfail
-    // .. qfail + kDfStages - 1, one per stage) land before the CTA's shared
-    // memory is released (bounded again)
-    if (lane == 0) {
-      if (err != nullptr) atomicCAS(err, 0, (int)LSQ_ERR_TIMEOUT);
-      for (int64_t r = qfail; r < qfail + kDfStages && r < nrows; r++)
-        mbar_wait(wbar + (r % kDfStages), (unsigned)((r / kDfStages) & 1), kDfWaitNs);
-    }
-    __syncwarp();
-  }
-#pragma unroll
-  for (int k = 0; k < NC; k++) {
-    const int col = 64 * k + 2 * lane;
-    hw[col] += widen(f2_lo(hh[k])) + widen(f2_lo(hl[k]));
-    hw[col + 1] += widen(f2_hi(hh[k])) + widen(f2_hi(hl[k]));
-  }
-  __syncthreads();
-  // fixed-order sum over the warps of this CTA, scaled back by 2^Fz
-  for (int c = threadIdx.x; c < npad; c += blockDim.x) {
-    double sacc = 0.0;
-    for (int w = 0; w < nw; w++) sacc += hacc[(size_t)w * NC * 64 + c];
-    part[(size_t)blockIdx.x * npad + c] = sacc * up;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// FP32 inner pass of the mixed-precision tier (condest below the gate): reads
-// the hi plane of A (A rounded to FP32, 4 bytes per element), FP32 row
-// products, FP32 column sums flushed into FP64 accumulators every 32 rows
-// (bounds the FP32 accumulation error at about 32 u_32 per block).  z is
-// scaled by a common power of two so that it sits in FP32 range; h is scaled
-// back.  Rows reach shared memory by TMA bulk copies, k32Stages rows per
-// warp in flight (lane 0 issues the copies of the rows its warp will take
-// next while the warp works on the current one), with the same bounded
-// mbarrier waits and drain as the double-float pass.
-// ---------------------------------------------------------------------------
-constexpr int k32Stages = 4;
-
-template <int NC>
-__global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
-    atax32_kernel(const float *__restrict__ A32, int64_t ld32, int64_t m, int n,
-                  const double *__restrict__ z, double *__restrict__ part, int npad,
-                  const DevState *gate, int *err) {
-  griddep_launch();
-  // dynamic shared memory: [warps][k32Stages][NC*64] FP32 row stages, then
-  // the mbarriers
-  extern __shared__ __align__(16) float rst[];
-  __shared__ double sh[NC * 64];
-  __shared__ double wmax[kPassThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float *wst = rst + (size_t)warp * k32Stages * NC * 64;
-  uint64_t *bars = reinterpret_cast<uint64_t *>(rst + (size_t)nw * k32Stages * NC * 64);
-  uint64_t *wbar = bars + warp * k32Stages;
-  const int64_t per = (m + gridDim.x - 1) / gridDim.x;
-  const int64_t r0 = min(m, (int64_t)blockIdx.x * per), r1 = min(m, r0 + per);
-  const int64_t nrows = (r1 - r0 - warp + nw - 1) / nw > 0 ? (r1 - r0 - warp + nw - 1) / nw : 0;
-  const unsigned row_bytes = (unsigned)(ld32 * sizeof(float));
-  if (lane == 0) {
-    for (int st = 0; st < k32Stages; st++) mbar_init(wbar + st, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
-  const uint64_t pol = l2_evict_first();
-  auto issue = [&](int64_t q) {
-    if (lane == 0 && q < nrows) {
-      const int64_t i = r0 + warp + q * nw;
-      const int stg = (int)(q % k32Stages);
-      mbar_expect_tx(wbar + stg, row_bytes);
-      bulk_g2s(wst + (size_t)stg * NC * 64, A32 + i * ld32, row_bytes, wbar + stg, pol);
-    }
-  };
-  for (int64_t q = 0; q < k32Stages; q++) issue(q);
-  griddep_wait();
-  if (gate != nullptr && *(volatile const int *)&gate->done) {
-    if (lane == 0)
-      for (int64_t q = 0; q < k32Stages && q < nrows; q++) mbar_wait(wbar + q, 0, kDfWaitNs);
-    return;
-  }
-  double zr[2 * NC];
-  load_vec<NC>(z, n, lane, zr);
-  double zmax = 0.0;
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) zmax = fmax(zmax, fabs(zr[k]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-  if (lane == 0) wmax[warp] = zmax;
-  __syncthreads();
-  zmax = 0.0;
-  for (int w = 0; w < nw; w++) zmax = fmax(zmax, wmax[w]);
-  int fz = 0;
-  if (zmax > 0.0) frexp(zmax, &fz);
-  const double down = ldexp(1.0, -fz), up = ldexp(1.0, fz);
-  float zf[2 * NC], hf[2 * NC];
-  double hd[2 * NC];
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) {
-    zf[k] = __double2float_rn(zr[k] * down);
-    hf[k] = 0.0f;
-    hd[k] = 0.0;
-  }
-  int blk = 0;
-  int64_t qfail = -1;
-  for (int64_t q = 0; q < nrows; q++) {
-    const int stg = (int)(q % k32Stages);
-    // one decision per warp: a lane whose wait ran out takes the whole warp
-    // to the drain below
-    if (!__all_sync(0xffffffffu, mbar_wait(wbar + stg, (unsigned)((q / k32Stages) & 1), kDfWaitNs))) {
-      qfail = q;
-      break;
-    }
-    const float *row = wst + (size_t)stg * NC * 64;
-    float a[2 * NC];
-#pragma unroll
-    for (int k = 0; k < NC; k++) {
-      const int col = 64 * k + 2 * lane;
-      if (col + 1 < n) {
-        const float2 v = *reinterpret_cast<const float2 *>(row + col);
-        a[2 * k] = v.x;
-        a[2 * k + 1] = v.y;
-      } else {
-        a[2 * k] = (col < n) ? row[col] : 0.0f;
-        a[2 * k + 1] = 0.0f;
-      }
-    }
-    // every lane has its values: the stage may be refilled
-    __syncwarp();
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    issue(q + k32Stages);
-    float t0 = 0.0f, t1 = 0.0f;
-#pragma unroll
-    for (int k = 0; k < NC; k++) {
-      t0 = __fmaf_rn(a[2 * k], zf[2 * k], t0);
-      t1 = __fmaf_rn(a[2 * k + 1], zf[2 * k + 1], t1);
-    }
-    float t = t0 + t1;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-#pragma unroll
-    for (int k = 0; k < 2 * NC; k++) hf[k] = __fmaf_rn(a[k], t, hf[k]);
-    if (++blk == 32) {
-      blk = 0;
-#pragma unroll
-      for (int k = 0; k < 2 * NC; k++) {
-        hd[k] += (double)hf[k];
-        hf[k] = 0.0f;
-      }
-    }
-  }
-  if (qfail >= 0) {
-    // record the error; let the copies this warp has in flight (rows qfail
-    // .. qfail + k32Stages - 1, one per stage) land before the CTA's shared
-    // memory is released
-    if (lane == 0) {
-      if (err != nullptr) atomicCAS(err, 0, (int)LSQ_ERR_TIMEOUT);
-      for (int64_t r = qfail; r < qfail + k32Stages && r < nrows; r++)
-        mbar_wait(wbar + (r % k32Stages), (unsigned)((r / k32Stages) & 1), kDfWaitNs);
-    }
-    __syncwarp();
-  }
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) hd[k] = (hd[k] + (double)hf[k]) * up;
-  cta_store_partial<NC>(hd, sh, part, npad);
 }
 
 // With Ahi != NULL the pass also writes the hi / lo FP32 planes of A: this
@@ -850,46 +508,6 @@ cudaError_t launch_pass_atax_eft(const double *A, int64_t lda, int64_t m, int n,
   LSQ_PASS_SWITCH(npad, {
     if (vec) atax_eft_kernel<NC, true><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, z, ebias, zscale, part, npad, gate);
     else atax_eft_kernel<NC, false><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, z, ebias, zscale, part, npad, gate);
-  });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pass_atax_df(const float *Ahi, const float *Alo, int64_t ld32, int64_t m, int n,
-                                const double *z, double *part, int grid, int npad,
-                                const DevState *gate, int *err, cudaStream_t s, int batch,
-                                int64_t zstride, int64_t pstride) {
-  const int nw = kPassThreads / 32;
-  const size_t smem = (size_t)nw * npad * sizeof(double) +
-                      (size_t)nw * kDfStages * 2 * npad * sizeof(float) +
-                      (size_t)nw * kDfStages * sizeof(uint64_t);
-  const dim3 g(grid, batch);
-  LSQ_PASS_SWITCH(npad, {
-    if (smem > 48 * 1024) {
-      cudaError_t e = ensure_smem_attr((const void *)atax_df_kernel<NC>, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    if (gate != nullptr)
-      return launch_pdl(atax_df_kernel<NC>, g, dim3(kPassThreads), smem, s, Ahi, Alo, ld32, m, n,
-                        z, part, npad, gate, err, zstride, pstride);
-    atax_df_kernel<NC><<<g, kPassThreads, smem, s>>>(Ahi, Alo, ld32, m, n, z, part, npad, gate,
-                                                     err, zstride, pstride);
-  });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pass_atax32(const float *A32, int64_t ld32, int64_t m, int n, const double *z,
-                               double *part, int grid, int npad, const DevState *gate, int *err,
-                               cudaStream_t s) {
-  const int nw = kPassThreads / 32;
-  const size_t smem = (size_t)nw * k32Stages * npad * sizeof(float) +
-                      (size_t)nw * k32Stages * sizeof(uint64_t);
-  LSQ_PASS_SWITCH(npad, {
-    if (smem > 48 * 1024) {
-      cudaError_t e = ensure_smem_attr((const void *)atax32_kernel<NC>, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    return launch_pdl(atax32_kernel<NC>, dim3(grid), dim3(kPassThreads), smem, s, A32, ld32, m, n,
-                      z, part, npad, gate, err);
   });
   return cudaGetLastError();
 }

@@ -595,6 +595,9 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
     // pass's operator holds A to 2^-48, which leaves step 2's answer a few u
     // ||A||_F from backward stable on kappa ~ 1e12 problems, above the bound.
     const bool df = P->use_df && !kw, eft = P->use_eft && !kw;
+    // CTAs (and partial sums) of the step's inner passes
+    const int gin = (P->csr.rp == nullptr && (df || tier))
+                        ? pass_df_grid(P->m, n, P->ld32, P->gpass) : P->gpass;
     // the step's first z = D^{-1} R^{-1} (dy or p)
     const InnerVecs iv = {n, P->Xcm, P->Xrm, P->dinv, P->h, P->c, P->w, P->z, P->dy, P->dyold,
                           {P->res, P->res2}, {P->p, P->p2}, P->pn, P->st, P->hprog};
@@ -617,17 +620,17 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
                                method == 2 ? P->lsqr_s : nullptr, P->s));
       else if (method == 2 && df)
         LSQ_CU(launch_pass_lsqr_df(P->Ahi, P->Alo, P->ld32, P->m, n, P->z, P->lsqr_s,
-                                   &P->st->lq_bscale, P->part, P->r2part, P->gpass, P->npad, P->st,
+                                   &P->st->lq_bscale, P->part, P->r2part, gin, P->npad, P->st,
                                    &P->st->err, P->s));
       else if (method == 2)
         LSQ_CU(launch_pass_resid(dA, P->lda, P->m, n, P->lsqr_s, P->z, P->part, P->r2part,
                                  P->gpass, P->npad, P->s, nullptr, nullptr, 0, P->st,
                                  &P->st->lq_bscale, P->lsqr_s));
       else if (tier)
-        LSQ_CU(launch_pass_atax32(P->Ahi, P->ld32, P->m, n, P->z, P->part, P->gpass, P->npad,
+        LSQ_CU(launch_pass_atax32(P->Ahi, P->ld32, P->m, n, P->z, P->part, gin, P->npad,
                                   P->st, &P->st->err, P->s));
       else if (df)
-        LSQ_CU(launch_pass_atax_df(P->Ahi, P->Alo, P->ld32, P->m, n, P->z, P->part, P->gpass,
+        LSQ_CU(launch_pass_atax_df(P->Ahi, P->Alo, P->ld32, P->m, n, P->z, P->part, gin,
                                    P->npad, P->st, &P->st->err, P->s));
       else if (eft)
         LSQ_CU(launch_pass_atax_eft(dA, P->lda, P->m, n, P->z, P->col_exp, P->part, P->gpass,
@@ -637,7 +640,7 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
                                 P->s));
       if (tj >= 0) LSQ_CU(cudaEventRecord(P->tev[2 * tj + 1], P->s));
       P->launches += 4;
-      LSQ_CU(launch_reduce(P->part, P->gpass, P->npad, n, P->dinv, P->h,
+      LSQ_CU(launch_reduce(P->part, gin, P->npad, n, P->dinv, P->h,
                            method == 2 ? P->r2part : nullptr,
                            method == 2 ? &P->st->lq_b2 : nullptr, P->st, P->s));
       LSQ_CU(launch_inner_w(method, iv, it & 1, P->s));
@@ -1087,6 +1090,13 @@ lsq_status lsq_plan_create(const lsq_options *opt, void *cuda_stream, lsq_plan *
     return fail(oom ? LSQ_ERR_OOM : LSQ_ERR_CUDA, std::string("plan allocation: ") + cudaGetErrorString(e));
   }
   e = cudaMemsetAsync(P->st, 0, sizeof(DevState), P->s);
+  // the passes over the planes read to the end of their column tiles: every
+  // value there must be finite, the rows' pads included
+  if (e == cudaSuccess && P->Ahi) {
+    const size_t pb = sizeof(float) * (size_t)P->m_cap * (size_t)((n + 3) / 4 * 4);
+    e = cudaMemsetAsync(P->Ahi, 0, pb, P->s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(P->Alo, 0, pb, P->s);
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(P->qflag, 0, sizeof(int) * (size_t)P->n_cap, P->s);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->qflag2, 0, sizeof(int) * (size_t)P->n_cap, P->s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(P->s);

@@ -218,6 +218,9 @@ lsq_status lsq_batch_create(int max_items, int64_t n_max, int64_t elems_max, voi
   A(cudaMallocHost((void **)&B->h_st, sizeof(DevState) * (size_t)max_items));
   A(cudaMalloc((void **)&B->d_qmap, sizeof(int) * (size_t)b_qr_max_ctas(B->nsm)));
   A(cudaMallocHost((void **)&B->h_qmap, sizeof(int) * (size_t)b_qr_max_ctas(B->nsm)));
+  // the passes over the planes read to the end of their column tiles: every
+  // value there must be finite
+  if (e == cudaSuccess) A(cudaMemset(B->planes, 0, sizeof(float) * 2 * (size_t)elems_max + 256));
   // the QR flags start at 0 (a flag is ready when it equals the launch's epoch)
   if (e == cudaSuccess) A(cudaMemset(B->ws, 0, L.total * (size_t)max_items));
   A(prepare_b_kernels((int)n_max));

@@ -17,6 +17,10 @@ constexpr double kUKwStop = 2.220446049250313e-16;
 constexpr int kPassThreads = 256;               // threads per CTA of the streaming passes
 constexpr int kPassCtasPerSm = 2;
 constexpr int kCsrCtasPerSm = 5;                // CTAs per SM of a sparse plan's pass grid
+// Planes up to this size are kept in L2 (129 MB; evict-last copies): 20000 x
+// 500, 80 MB, 36.9 us per iteration against 38.2 with evict-first; at 123 MB
+// keeping them costs 6%.
+constexpr double kL2KeepBytes = 96.0e6;
 constexpr int kVecThreads = 1024;               // threads of the single-CTA vector kernels
 constexpr int kMaxZeta = 32;
 constexpr int kProgDone = 1 << 30;              // progress word: the inner loop has stopped
@@ -276,9 +280,8 @@ cudaError_t launch_pass_atax_eft(const double *A, int64_t lda, int64_t m, int n,
 cudaError_t launch_pass_atax32(const float *A32, int64_t ld32, int64_t m, int n, const double *z,
                                double *part, int grid, int npad, const DevState *gate, int *err,
                                cudaStream_t s);
-// Inner pass on the hi / lo FP32 planes: row and column sums both in
-// double-float on the FP32 pipe (column sums flushed into FP64 every 8 rows);
-// rows staged by TMA bulk copies.  ld32: a multiple of 4 (16-byte rows);
+// Inner pass on the hi / lo FP32 planes (k_pass_df.cu): row and column sums
+// both in double-float on the FP32 pipe; rows staged by TMA bulk copies.  ld32: a multiple of 4 (16-byte rows);
 // Ahi / Alo 16-byte aligned.  err: LSQ_ERR_TIMEOUT if a copy never landed.
 // batch > 1: grid rows c < batch work on z + c zstride into part + c pstride.
 cudaError_t launch_pass_atax_df(const float *Ahi, const float *Alo, int64_t ld32, int64_t m, int n,
@@ -289,6 +292,9 @@ cudaError_t launch_pass_atax_df(const float *Ahi, const float *Alo, int64_t ld32
 // the partial sums of H = A^T (A Z) for k <= 64 vectors (Z n x k column-
 // major), CTA g's for vector c at part + (c grid + g) npad.  Needs n <= 256,
 // ld32 % 4 == 0 and one CTA per SM of shared memory (multi_df_supported).
+// CTAs that the passes over the planes use of `grid` (a block of rows for
+// every warp; fewer partial sums for short problems).
+int pass_df_grid(int64_t m, int n, int64_t ld32, int grid);
 bool multi_df_supported(int n, int k, int64_t ld32);
 cudaError_t launch_pass_atax_df_multi(const float *Ahi, const float *Alo, int64_t ld32, int64_t m,
                                       int n, const double *Z, int k, double *part, int grid,

@@ -52,12 +52,13 @@ __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) 
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// Exact FP32 -> FP64 widening with integer operations (normal and zero inputs).
+// Exact FP32 -> FP64 widening with integer operations (normal and zero
+// inputs; infinities and NaN give NaN or an infinity).
 __device__ __forceinline__ double widen(float f) {
   const unsigned b = __float_as_uint(f);
   const unsigned e = (b >> 23) & 0xffu;
   if (e == 0) return 0.0;
-  const unsigned hw = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
+  const unsigned hw = (b & 0x80000000u) | ((e == 255u ? 2047u : e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
   return __hiloint2double((int)hw, (int)(b << 29));
 }
 
@@ -100,6 +101,20 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
   return pol;
+}
+
+// The opposite: planes that fit in L2 are read dozens of times per solve.
+__device__ __forceinline__ uint64_t l2_evict_last() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
+
+// An FP64 value as hi + lo FP32 words (as split_rn), NaN when it is beyond
+// FP32's range: a conversion would take an FP64 instruction of 64 cycles.
+__device__ __forceinline__ void split_f32x2(double a, float &hi, float &lo) {
+  split_rn(a, hi, lo);
+  if ((((unsigned)__double2hiint(a) >> 20) & 0x7ffu) >= 896u + 254u) hi = __uint_as_float(0x7fffffffu);
 }
 
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar,

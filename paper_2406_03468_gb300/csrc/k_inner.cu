@@ -426,6 +426,50 @@ __global__ void __launch_bounds__(kInThreads)
   }
 }
 
+// k vectors: one warp per entry i of 8 vectors (row i of X, or column i for X^T,
+// loaded once).  n <= 256.  The 8 sums by recursive halving over lanes 16, 8
+// and 4 apart, then two butterflies: 9 FP64 additions instead of 40.
+template <int NB>
+__global__ void __launch_bounds__(kInThreads)
+    multi_xprod_kernel(int n, int trans, const double *__restrict__ X, const double *__restrict__ V,
+                       const double *__restrict__ os, double *__restrict__ out,
+                       const DevState *gate) {
+  if (gate != nullptr && *(volatile const int *)&gate->done) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * kInWarps + warp;
+  if (i >= n) return;
+  V += (size_t)blockIdx.y * 8 * n;
+  double acc[8];
+#pragma unroll
+  for (int c = 0; c < 8; c++) acc[c] = 0.0;
+#pragma unroll
+  for (int k = 0; k < NB; k++) {
+    if (trans ? 32 * k <= i : 32 * k + 31 >= i) {
+      const int j = 32 * k + lane;
+      const bool in = j < n && (trans ? j <= i : j >= i);
+      const double x = in ? X[(size_t)i * n + j] : 0.0;
+#pragma unroll
+      for (int c = 0; c < 8; c++) acc[c] = fma(x, in ? V[(size_t)c * n + j] : 0.0, acc[c]);
+    }
+  }
+#pragma unroll
+  for (int q = 4, o = 16; q >= 1; q >>= 1, o >>= 1) {
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int c = 0; c < q; c++) {
+      const double keep = hi ? acc[c + q] : acc[c], send = hi ? acc[c] : acc[c + q];
+      acc[c] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double t = acc[0];
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  // lane's vector: 4 (bit 4) + 2 (bit 3) + 1 (bit 2)
+  const int c = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+  if ((lane & 3) == 0)
+    out[((size_t)blockIdx.y * 8 + c) * n + i] = os != nullptr ? os[i] * t : t;
+}
+
 }  // namespace
 
 // columns of 32 rows of X held in registers by a warp: the power of two that
@@ -512,6 +556,17 @@ cudaError_t launch_inner_u(int method, const InnerVecs &v, int par, cudaStream_t
                           v.res[par ^ 1], (const double *)nullptr, v.p[0], v.dy,
                           (const double *)v.pn, par, v.st, v.hprog);
     }
+  });
+}
+
+cudaError_t launch_multi_xprod(int n, int k, int trans, const double *X, const double *V,
+                               const double *os, double *out, const DevState *gate,
+                               cudaStream_t s) {
+  const dim3 grid(inner_partials(n), k / 8);
+  if (n > 256) return cudaErrorInvalidValue;
+  LSQ_NB_SWITCH(n, {
+    multi_xprod_kernel<NB><<<grid, kInThreads, 0, s>>>(n, trans, X, V, os, out, gate);
+    return cudaGetLastError();
   });
 }
 

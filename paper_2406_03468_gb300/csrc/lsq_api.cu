@@ -135,6 +135,9 @@ struct lsq_plan_s {
   int k = 0;
   bool multi_planes = false;        // the planes hold the A of the last multi solve
   double *SBb = nullptr, *cpartB = nullptr, *mpart = nullptr, *mr2part = nullptr, *mT = nullptr;
+  TcBufs tc{};                // tensor-core pass: digits of A, z, y, partial sums
+  bool tc_alloc = false, use_tc = false;
+  TcCol *col_host = nullptr;
   double *mpartdf = nullptr;  // partials of the batched double-float pass (k x gpass x npad)
   double *mXs = nullptr, *mXo = nullptr, *mC = nullptr, *mG = nullptr, *mDY = nullptr;
   double *mDYold = nullptr, *mZ = nullptr, *mH = nullptr, *mW = nullptr, *mstate = nullptr;
@@ -725,7 +728,8 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
   return status;
 }
 
-// Many right-hand sides, inner pass in double-float on the planes: the
+// Many right-hand sides, inner pass: on the tensor cores in fixed point, unless
+// a column of A is dominated by few entries; then in double-float on the planes, the
 // k-tiled pass (every row block of A applied to all k vectors while it is in
 // shared memory) when its tiles fit, else one launch of the single-vector
 // pass over k grid rows (each vector re-reads A).  H (n x k column-major) =
@@ -733,6 +737,8 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
 cudaError_t launch_multi_df_pass(lsq_plan P, const double *Z, double *H, const double *scale,
                                  const DevState *gate) {
   const int n = (int)P->n, k = P->k;
+  if (P->use_tc)
+    return launch_multi_tc_pass(P->m, n, k, Z, H, scale, P->tc, P->nsm, gate, &P->st->err, P->s);
   if (multi_df_supported(n, k, P->ld32)) {
     cudaError_t e = launch_pass_atax_df_multi(P->Ahi, P->Alo, P->ld32, P->m, n, Z, k, P->mpartdf,
                                               P->nsm, P->npad, gate, &P->st->err, P->s);
@@ -775,6 +781,12 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   LSQ_CU(launch_sketch_finalize(P->cpart, P->gpass, P->npad, n, d, P->zeta, P->o.col_scale,
                                 P->SAb, P->W, P->dcol, P->dinv, P->st, P->s));
   LSQ_CU(launch_sketch_b_to_w(P->SBb, d, n, k, P->zeta, P->W, P->st, P->s));
+  if (P->tc_alloc && P->want32) {
+    LSQ_CU(launch_multi_tc_prepare(dA, P->lda, P->m, n, P->tc, P->nsm, P->s));
+    LSQ_CU(cudaMemcpyAsync(P->col_host, P->tc.col, sizeof(TcCol) * n, cudaMemcpyDeviceToHost,
+                           P->s));
+    P->launches += 2;
+  }
   LSQ_CU(cudaEventRecord(P->ev[1], P->s));
   LSQ_CU(launch_qr(P->W, d, n, n + k, P->vbuf, P->qflag, next_epoch(P), P->st,
                    qr_grid(n + k, P->nsm), qr_timeout_ns(P), P->s, &P->qb));
@@ -793,6 +805,10 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   // FP64 tensor-core contraction
   choose_inner_kernel(P);
   const bool multi_df = P->use_df;
+  P->use_tc = multi_df && P->tc_alloc && multi_tc_columns_ok(n, P->col_host, 8.0);
+  // the residual's A x and A^T r stand in for FP64 sums: only where 56-bit fixed
+  // point is no further off than FP64's rounding
+  const bool tc_resid = P->use_tc && multi_tc_columns_ok(n, P->col_host, 5.0);
   P->multi_planes = P->want32;  // the sketch above wrote the planes of this A
   if (P->st_host->nonfinite) return fail(LSQ_ERR_NONFINITE, "A or B holds NaN or Inf");
   if (P->st_host->zero_col) return fail(LSQ_ERR_INVALID, "A has a zero column (column scaling)");
@@ -804,10 +820,15 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   std::vector<double> hc(k);
   std::vector<int> inner_ev[LSQ_MAX_REFINE];
   for (int i = 0; i < nref; i++) {
-    LSQ_CU(launch_multi_resid(dA, P->lda, P->m, n, k, dB, ldb, P->mXo, P->mpart, P->mr2part,
-                              P->nsm, P->s));
-    LSQ_CU(launch_multi_reduce(P->mpart, P->nsm, n, k, P->dinv, P->mG, P->mr2part, r2, nullptr,
-                               P->s));
+    if (tc_resid) {
+      LSQ_CU(launch_multi_tc_resid(P->m, n, k, dB, ldb, P->mXo, P->mG, P->dinv, r2, P->tc, P->nsm,
+                                   &P->st->err, P->s));
+    } else {
+      LSQ_CU(launch_multi_resid(dA, P->lda, P->m, n, k, dB, ldb, P->mXo, P->mpart, P->mr2part,
+                                P->nsm, P->s));
+      LSQ_CU(launch_multi_reduce(P->mpart, P->nsm, n, k, P->dinv, P->mG, P->mr2part, r2, nullptr,
+                                 P->s));
+    }
     LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 1, P->mG, nullptr, P->mC, nullptr, nullptr,
                        nullptr, cn2, nullptr, P->s, k, n));
     if (i == 0)
@@ -818,8 +839,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
     LSQ_CU(launch_multi_init(n, k, P->mC, P->mDY, P->mDYold, cap, use_thresh, P->st, P->s));
     P->launches += 5;
     for (int it = 0; it < cap; it++) {
-      LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 0, P->mDY, nullptr, nullptr, P->dinv, P->mZ,
-                         nullptr, nullptr, P->st, P->s, k, n));
+      LSQ_CU(launch_multi_xprod(n, k, 0, P->Xrm, P->mDY, P->dinv, P->mZ, P->st, P->s));
       int tj = -1;
       if (P->o.timing) {
         LSQ_CU(tev_pair(P, &tj));
@@ -835,8 +855,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
         LSQ_CU(launch_multi_reduce(P->mpart, P->nsm, n, k, P->dinv, P->mH, nullptr, nullptr,
                                    P->st, P->s));
       }
-      LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 1, P->mH, nullptr, P->mW, nullptr, nullptr,
-                         nullptr, nullptr, P->st, P->s, k, n));
+      LSQ_CU(launch_multi_xprod(n, k, 1, P->Xcm, P->mH, nullptr, P->mW, P->st, P->s));
       LSQ_CU(launch_multi_polyak(n, k, P->mC, P->mW, P->mDY, P->mDYold, dn2, thr, P->st, P->s));
       P->launches += 6;
       if (use_thresh && (it % kStopPollEvery) == kStopPollEvery - 1 && it + 1 < cap) {
@@ -922,6 +941,37 @@ void configure_fields(lsq_plan P, const lsq_options *opt) {
   P->multi_planes = false;
 }
 
+void free_tc(lsq_plan P) {
+  void *bufs[] = {P->tc.p1, P->tc.p2, P->tc.q, P->tc.y, P->tc.y64, P->tc.h, P->tc.col, P->tc.F,
+                  P->tc.ybits, P->tc.r2part};
+  for (void *b : bufs)
+    if (b) cudaFree(b);
+  P->tc = TcBufs{};
+  P->tc_alloc = false;
+}
+
+// The tensor-core pass's buffers; without them (not enough memory) the plan
+// uses the double-float form.
+void alloc_tc(lsq_plan P, int n) {
+  const TcSizes z = multi_tc_sizes(P->m_cap, n, P->k, P->nsm);
+  cudaError_t e = cudaMalloc((void **)&P->tc.p1, z.p1);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.p2, z.p2);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.q, z.q);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.y, z.y);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.y64, z.y64);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.h, z.h);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.col, sizeof(TcCol) * 256);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.F, sizeof(int) * 64);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.ybits, sizeof(int) * 128);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.r2part, z.r2);
+  if (e == cudaSuccess) e = cudaMallocHost((void **)&P->col_host, sizeof(TcCol) * 256);
+  P->tc_alloc = e == cudaSuccess;
+  if (!P->tc_alloc) {
+    cudaGetLastError();
+    free_tc(P);
+  }
+}
+
 void free_plan(lsq_plan P) {
   if (!P) return;
   void *bufs[] = {P->pat_rows, P->pat_sb, P->SAb, P->W, P->part, P->r2part, P->cpart, P->dcol, P->dinv,
@@ -935,6 +985,8 @@ void free_plan(lsq_plan P) {
                   P->part2};
   for (void *b : bufs)
     if (b) cudaFree(b);
+  free_tc(P);
+  if (P->col_host) cudaFreeHost(P->col_host);
   if (P->st_host) cudaFreeHost(P->st_host);
   if (P->dcol_host) cudaFreeHost(P->dcol_host);
   if (P->hprog) cudaFreeHost(P->hprog);
@@ -1073,6 +1125,7 @@ lsq_status lsq_plan_create(const lsq_options *opt, void *cuda_stream, lsq_plan *
     A(dalloc(&P->Alo, (size_t)P->m_cap * ((n + 3) / 4 * 4)));
     P->want32 = true;
   }
+  if (e == cudaSuccess && P->k > 0 && P->Ahi) alloc_tc(P, n);
   for (auto &ev : P->ev) A(cudaEventCreate(&ev));
   A(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
   A(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));

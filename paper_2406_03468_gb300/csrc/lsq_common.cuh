@@ -299,6 +299,38 @@ bool multi_df_supported(int n, int k, int64_t ld32);
 cudaError_t launch_pass_atax_df_multi(const float *Ahi, const float *Alo, int64_t ld32, int64_t m,
                                       int n, const double *Z, int k, double *part, int grid,
                                       int npad, const DevState *gate, int *err, cudaStream_t s);
+// The same pass on the tensor cores in fixed point (k_multi_tc.cu): n <= 256,
+// k <= 64.  prepare: the columns' largest exponents and A's digits in both
+// layouts, once per solve; pass: out (n x k column-major) = scale .* A^T (A Z).
+struct TcSizes {
+  size_t p1, p2, q, y, y64, h, r2;  // bytes
+};
+struct TcCol {              // a column of A (zeroed, then tc_colmax_kernel)
+  long long esum;           // sum of the exponents of its nonzero entries
+  int emax, cnt;            // largest biased exponent, nonzero entries
+};
+struct TcBufs {
+  unsigned char *p1, *p2, *q, *y;
+  long long *y64, *h;
+  TcCol *col;               // n
+  int *F, *ybits;           // 64, 128
+  double *r2part;
+};
+TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm);
+cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
+                                    int nsm, cudaStream_t s);
+// Whether every column's typical entry (the mean exponent of its nonzero
+// entries) is within `bits` of its largest: fixed point to the largest entry
+// holds it to 2^(bits - 56).
+bool multi_tc_columns_ok(int n, const TcCol *col, double bits);
+// The residual pass: out = scale .* A^T (B - A X), r2[c] = ||b_c - A x_c||^2 (X n
+// x k column-major, B m x k row-major).
+cudaError_t launch_multi_tc_resid(int64_t m, int n, int k, const double *B, int64_t ldb,
+                                  const double *X, double *out, const double *scale, double *r2,
+                                  const TcBufs &b, int nsm, int *err, cudaStream_t s);
+cudaError_t launch_multi_tc_pass(int64_t m, int n, int k, const double *Z, double *out,
+                                 const double *scale, const TcBufs &b, int nsm,
+                                 const DevState *gate, int *err, cudaStream_t s);
 // out (n x batch, column-major) = scale .* the sums of a batched pass's partials.
 cudaError_t launch_reduce_batched(const double *part, int grid, int npad, int n, int batch,
                                   const double *scale, double *out, const DevState *gate,
@@ -446,6 +478,10 @@ struct InnerVecs {
   int *hprog;             // progress word in page-locked host memory (may be NULL)
 };
 int inner_partials(int n);
+// out_c = os .* X v_c (trans = 0, os may be NULL) or X^T v_c (1) for k vectors
+// (k a multiple of 8; vector c at c n), gated.
+cudaError_t launch_multi_xprod(int n, int k, int trans, const double *X, const double *V,
+                               const double *os, double *out, const DevState *gate, cudaStream_t s);
 // First half of the update of iteration `par` (its parity), after the
 // reduction; second half and the next z; the step's first z (after
 // launch_inner_init / launch_lsqr_init).

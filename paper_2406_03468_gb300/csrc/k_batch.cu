@@ -11,7 +11,7 @@
 // item whose inner loop has stopped (st->done), so the launch costs nothing
 // for the items that are done.
 #include "lsq_common.cuh"
-#include "lsq_dfpass.cuh"
+#include "lsq_resid.cuh"
 
 namespace lsq {
 
@@ -19,94 +19,30 @@ namespace {
 
 constexpr int kBThreads = kPassThreads;
 
-template <int NC>
-__device__ __forceinline__ void b_load_vec(const double *__restrict__ x, int n, int lane,
-                                           double (&v)[2 * NC]) {
-#pragma unroll
-  for (int k = 0; k < NC; k++) {
-    const int col = 64 * k + 2 * lane;
-    v[2 * k] = (col < n) ? x[col] : 0.0;
-    v[2 * k + 1] = (col + 1 < n) ? x[col + 1] : 0.0;
-  }
-}
-
-template <int NC>
-__device__ __forceinline__ void b_load_row(const double *__restrict__ row, int n, int lane,
-                                           double (&a)[2 * NC]) {
-#pragma unroll
-  for (int k = 0; k < NC; k++) {
-    const int col = 64 * k + 2 * lane;
-    a[2 * k] = (col < n) ? __ldcs(row + col) : 0.0;
-    a[2 * k + 1] = (col + 1 < n) ? __ldcs(row + col + 1) : 0.0;
-  }
-}
-
-// Fixed-order sum over the CTA's warps of per-lane column values into
-// part[0 .. npad).
-template <int NC>
-__device__ __forceinline__ void b_store_partial(const double (&h)[2 * NC], double *sh,
-                                                double *__restrict__ part, int npad) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = threadIdx.x; i < NC * 64; i += blockDim.x) sh[i] = 0.0;
-  for (int w = 0; w < nw; w++) {
-    __syncthreads();
-    if (warp == w) {
-#pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        sh[col] += h[2 * k];
-        sh[col + 1] += h[2 * k + 1];
-      }
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < npad; i += blockDim.x) part[i] = sh[i];
-}
-
-template <int NC>
-__device__ void b_resid_body(const BItem &it, int local, double *sh, double *r2sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int n = it.n;
-  const int64_t m = it.m, per = (m + it.ncta - 1) / it.ncta;
-  const int64_t r0 = min(m, (int64_t)local * per), r1 = min(m, r0 + per);
-  double xr[2 * NC], g[2 * NC];
-  b_load_vec<NC>(it.xo, n, lane, xr);
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) g[k] = 0.0;
-  double r2 = 0.0;
-  for (int64_t i = r0 + warp; i < r1; i += nw) {
-    double a[2 * NC];
-    b_load_row<NC>(it.A + i * n, n, lane, a);
-    double s = 0.0;
-#pragma unroll
-    for (int k = 0; k < 2 * NC; k++) s = fma(a[k], xr[k], s);
-    s = warp_sum(s);
-    const double r = it.b[i] - s;
-    r2 = fma(r, r, r2);
-#pragma unroll
-    for (int k = 0; k < 2 * NC; k++) g[k] = fma(a[k], r, g[k]);
-  }
-  if (lane == 0) r2sh[warp] = r2;
-  b_store_partial<NC>(g, sh, it.part + (size_t)local * it.npad, it.npad);
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < nw; w++) s += r2sh[w];
-    it.r2part[local] = s;
-  }
-}
-
+// The FP64 residual pass of one item's CTA (lsq_resid.cuh).  The planes are
+// the sketch's.
 __global__ void __launch_bounds__(kBThreads, 2)
     b_resid_kernel(const BItem *__restrict__ items, const int *__restrict__ cta_item) {
-  __shared__ double sh[4 * 64];
-  __shared__ double r2sh[kBThreads / 32];
+  __shared__ double sh[resid_smem(16, 8)];
   const int idx = cta_item[blockIdx.x];
   if (idx < 0) return;
   const BItem &it = items[idx];
   const int local = blockIdx.x - it.cta0;
-  switch (it.npad / 64) {
-    case 1: b_resid_body<1>(it, local, sh, r2sh); break;
-    case 2: b_resid_body<2>(it, local, sh, r2sh); break;
-    case 4: b_resid_body<4>(it, local, sh, r2sh); break;
+  const int64_t per = (it.m + it.ncta - 1) / it.ncta;
+  const int64_t r0 = min(it.m, (int64_t)local * per), r1 = min(it.m, r0 + per);
+  const ResidArgs a = {it.A, it.n, it.b, nullptr, nullptr, nullptr, nullptr, 0};
+  const bool vec = (reinterpret_cast<uintptr_t>(it.A) & 15) == 0 && it.n % 2 == 0;
+  double *part = it.part + (size_t)local * it.npad, *r2 = it.r2part + local;
+  const DfTile t = df_tile(it.n);
+  switch (t.G * 100 + t.P) {
+#define LSQ_BRES(GV, PV)                                                                \
+  case GV * 100 + PV:                                                                   \
+    if (vec) resid_body<GV, PV, true>(a, r0, r1, it.n, it.xo, part, r2, it.npad, sh);   \
+    else resid_body<GV, PV, false>(a, r0, r1, it.n, it.xo, part, r2, it.npad, sh);      \
+    break;
+    LSQ_BRES(8, 1) LSQ_BRES(8, 2) LSQ_BRES(8, 3) LSQ_BRES(8, 4) LSQ_BRES(8, 5) LSQ_BRES(8, 6)
+    LSQ_BRES(8, 7) LSQ_BRES(8, 8) LSQ_BRES(16, 5) LSQ_BRES(16, 6) LSQ_BRES(16, 7) LSQ_BRES(16, 8)
+#undef LSQ_BRES
     default: break;
   }
 }

@@ -10,7 +10,7 @@
 // partial n-vector and a separate kernel sums the partials in a fixed order,
 // so the result does not depend on scheduling.
 #include "lsq_common.cuh"
-#include "lsq_dev.cuh"
+#include "lsq_resid.cuh"
 
 namespace lsq {
 
@@ -197,68 +197,34 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
   cta_store_partial<NC>(h, sh, part, npad);
 }
 
-// With Ahi != NULL the pass also writes the hi / lo FP32 planes of A: this
-// pass is bound by the FP64 pipe with HBM to spare, so the plane stores cost
-// almost nothing here (the large-problem sketch leaves them to the first
-// residual pass of a solve).
-template <int NC, bool VEC>
-__global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
-    resid_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int n,
-                 const double *b, const double *__restrict__ x,
+// The FP64 residual pass (lsq_resid.cuh).  With Ahi != NULL it also writes the
+// hi / lo FP32 planes of A (the large-problem sketch leaves them to the first
+// residual pass of a solve).  Two CTAs per SM up to 8 pairs per lane, one above.
+template <int G, int P, bool VEC>
+__global__ void __launch_bounds__(kPassThreads, P > 8 ? 1 : kPassCtasPerSm)
+    resid_kernel(const ResidArgs a, int64_t m, int n, const double *__restrict__ x,
                  double *__restrict__ part, double *__restrict__ r2_part, int npad,
-                 float *__restrict__ Ahi, float *__restrict__ Alo, int64_t ld32,
-                 const DevState *gate, const double *bscale, double *rout) {
+                 const DevState *gate) {
   if (gate != nullptr && *(volatile const int *)&gate->done) return;
-  __shared__ double sh[NC * 64];
-  const double bs = bscale != nullptr ? *bscale : 1.0;
-  __shared__ double r2sh[kPassThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  extern __shared__ __align__(16) double rsm[];
   const int64_t per = (m + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = min(m, (int64_t)blockIdx.x * per), r1 = min(m, r0 + per);
-  double xr[2 * NC], g[2 * NC];
-  load_vec<NC>(x, n, lane, xr);
-#pragma unroll
-  for (int k = 0; k < 2 * NC; k++) g[k] = 0.0;
-  double r2 = 0.0;
-  for (int64_t i = r0 + warp; i < r1; i += nw) {
-    double a[2 * NC];
-    load_row<NC, VEC>(A + i * lda, n, lane, a);
-    if (Ahi != nullptr) {
-#pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        float h0, l0, h1, l1;
-        split_rn(a[2 * k], h0, l0);
-        split_rn(a[2 * k + 1], h1, l1);
-        if (col + 1 < n) {
-          __stcs(reinterpret_cast<float2 *>(Ahi + i * ld32 + col), make_float2(h0, h1));
-          __stcs(reinterpret_cast<float2 *>(Alo + i * ld32 + col), make_float2(l0, l1));
-        } else if (col < n) {
-          __stcs(Ahi + i * ld32 + col, h0);
-          __stcs(Alo + i * ld32 + col, l0);
-        }
-      }
-    }
-    double s = 0.0;
-#pragma unroll
-    for (int k = 0; k < 2 * NC; k++) s = fma(a[k], xr[k], s);
-    s = warp_sum(s);
-    const double r = (bscale != nullptr ? bs * b[i] : b[i]) - s;
-    if (rout != nullptr) {
-      __syncwarp();  // every lane has read b[i] (rout may be b)
-      if (lane == 0) rout[i] = r;
-    }
-    r2 = fma(r, r, r2);
-#pragma unroll
-    for (int k = 0; k < 2 * NC; k++) g[k] = fma(a[k], r, g[k]);
+  resid_body<G, P, VEC>(a, r0, r1, n, x, part + (size_t)blockIdx.x * npad, r2_part + blockIdx.x,
+                        npad, rsm);
+}
+
+template <int G, int P>
+cudaError_t resid_launch(const ResidArgs &a, bool vec, int64_t m, int n, const double *x,
+                         double *part, double *r2_part, int grid, int npad, const DevState *gate,
+                         cudaStream_t s) {
+  constexpr int smem = resid_smem(G, P) * (int)sizeof(double);
+  auto *k = vec ? resid_kernel<G, P, true> : resid_kernel<G, P, false>;
+  if (smem > 48 * 1024) {
+    cudaError_t e = ensure_smem_attr((const void *)k, smem);
+    if (e != cudaSuccess) return e;
   }
-  if (lane == 0) r2sh[warp] = r2;
-  cta_store_partial<NC>(g, sh, part, npad);
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < nw; w++) s += r2sh[w];
-    r2_part[blockIdx.x] = s;
-  }
+  k<<<grid, kPassThreads, smem, s>>>(a, m, n, x, part, r2_part, npad, gate);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -420,8 +386,6 @@ __global__ void reduce_batched_kernel(const double *__restrict__ part, int grid,
 // so the n G additions are spread over all SMs.  At G = 304, n = 500: 63 CTAs
 // of about 10 additions per thread; CTAs of 32 columns with 38 per thread
 // took 6.5 us in the inner loop.
-constexpr int kReduceThreads = 256;
-constexpr int kReduceCols = 8;
 __global__ void __launch_bounds__(kReduceThreads)
     reduce_kernel(const double *__restrict__ part, int grid, int npad, int n,
                   const double *__restrict__ scale, double *__restrict__ out,
@@ -433,7 +397,7 @@ __global__ void __launch_bounds__(kReduceThreads)
     if (blockIdx.x == 0 && threadIdx.x == 0) gate->ugate = done;
     if (done) return;
   }
-  constexpr int kGroups = kReduceThreads / kReduceCols, kW = kReduceThreads / 32;
+  constexpr int kW = kReduceThreads / 32;
   __shared__ double red[kW][kReduceCols];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (r2 != nullptr && blockIdx.x == gridDim.x - 1) {
@@ -448,28 +412,10 @@ __global__ void __launch_bounds__(kReduceThreads)
     }
     return;
   }
-  const int c = threadIdx.x % kReduceCols, t0 = threadIdx.x / kReduceCols;
-  const int j = blockIdx.x * kReduceCols + c;  // < npad
-  double s0 = 0.0, s1 = 0.0;
-  int g = t0;
-#pragma unroll 4
-  for (; g + kGroups < grid; g += 2 * kGroups) {
-    s0 += part[(size_t)g * npad + j];
-    s1 += part[(size_t)(g + kGroups) * npad + j];
-  }
-  if (g < grid) s0 += part[(size_t)g * npad + j];
-  double s = s0 + s1;
-  s += __shfl_xor_sync(0xffffffffu, s, 8);
-  s += __shfl_xor_sync(0xffffffffu, s, 16);
-  if (lane < kReduceCols) red[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0) {
-    const int q = lane >> 3;
-    s = red[q][c] + red[q + 4][c];
-    s += __shfl_xor_sync(0xffffffffu, s, 8);
-    s += __shfl_xor_sync(0xffffffffu, s, 16);
-    if (lane < kReduceCols && j < n) out[j] = scale ? scale[j] * s : s;
-  }
+  const int j0 = blockIdx.x * kReduceCols;
+  const double t = sum_partials(part, grid, npad, j0, red);
+  if (threadIdx.x < kReduceCols && j0 + threadIdx.x < n)
+    out[j0 + threadIdx.x] = scale ? scale[j0 + threadIdx.x] * t : t;
 }
 
 bool vec_ok(const double *A, int64_t lda) {
@@ -517,17 +463,20 @@ cudaError_t launch_pass_resid(const double *A, int64_t lda, int64_t m, int n, co
                               cudaStream_t s, float *Ahi, float *Alo, int64_t ld32,
                               const DevState *gate, const double *bscale, double *rout) {
   const bool vec = vec_ok(A, lda);
-  LSQ_PASS_SWITCH(npad, {
-    if (vec)
-      resid_kernel<NC, true><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, x, part, r2_part,
-                                                           npad, Ahi, Alo, ld32, gate, bscale,
-                                                           rout);
-    else
-      resid_kernel<NC, false><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, x, part, r2_part,
-                                                            npad, Ahi, Alo, ld32, gate, bscale,
-                                                            rout);
-  });
-  return cudaGetLastError();
+  const ResidArgs a = {A, lda, b, bscale, rout, Ahi, Alo, ld32};
+  const DfTile t = df_tile(n);
+  switch (t.G * 100 + t.P) {
+#define LSQ_RES(GV, PV) \
+  case GV * 100 + PV:   \
+    return resid_launch<GV, PV>(a, vec, m, n, x, part, r2_part, grid, npad, gate, s);
+    LSQ_RES(8, 1) LSQ_RES(8, 2) LSQ_RES(8, 3) LSQ_RES(8, 4) LSQ_RES(8, 5) LSQ_RES(8, 6)
+    LSQ_RES(8, 7) LSQ_RES(8, 8) LSQ_RES(16, 5) LSQ_RES(16, 6) LSQ_RES(16, 7) LSQ_RES(16, 8)
+    LSQ_RES(32, 5) LSQ_RES(32, 6) LSQ_RES(32, 7) LSQ_RES(32, 8) LSQ_RES(32, 10) LSQ_RES(32, 12)
+    LSQ_RES(32, 14) LSQ_RES(32, 16)
+#undef LSQ_RES
+    default:
+      return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_pass_resid_dot2(const double *A, int64_t lda, int64_t m, int n,

@@ -14,6 +14,7 @@
 // the sums into column norms, applies diag(d)^{-1} and zeta^{-1/2}, and
 // transposes the sketch to the column-major layout the QR works on.
 #include "lsq_common.cuh"
+#include "lsq_dev.cuh"
 
 namespace lsq {
 
@@ -183,12 +184,13 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
     colsq_part[(size_t)blockIdx.x * npad + i] = acc[i];
 }
 
-__global__ void colnorm_kernel(const double *__restrict__ part, int grid, int npad, int n,
-                               int col_scale, double *dcol, double *dinv, DevState *st) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  double s = 0.0;
-  for (int g = 0; g < grid; g++) s += part[(size_t)g * npad + j];
+__global__ void __launch_bounds__(kReduceThreads)
+    colnorm_kernel(const double *part, int grid, int npad, int n, int col_scale, double *dcol,
+                   double *dinv, DevState *st) {
+  __shared__ double red[kReduceThreads / 32][kReduceCols];
+  const double s = sum_partials(part, grid, npad, blockIdx.x * kReduceCols, red);
+  const int j = blockIdx.x * kReduceCols + threadIdx.x;
+  if (threadIdx.x >= kReduceCols || j >= n) return;
   const double nrm = sqrt(s);
   if (!isfinite(nrm)) atomicExch(&st->nonfinite, 1);
   if (col_scale && nrm == 0.0) atomicExch(&st->zero_col, 1);
@@ -813,8 +815,8 @@ cudaError_t launch_sketch(const double *A, int64_t lda, int64_t m, int n, const 
 cudaError_t launch_sketch_finalize(const double *colsq_part, int grid, int npad, int n, int d,
                                    int zeta, int col_scale, const double *SAb, double *W,
                                    double *dcol, double *dinv, DevState *st, cudaStream_t s) {
-  colnorm_kernel<<<(n + 255) / 256, 256, 0, s>>>(colsq_part, grid, npad, n, col_scale, dcol, dinv,
-                                                 st);
+  colnorm_kernel<<<(n + kReduceCols - 1) / kReduceCols, kReduceThreads, 0, s>>>(
+      colsq_part, grid, npad, n, col_scale, dcol, dinv, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   dim3 blk(32, 8), grd((n + 1 + 31) / 32, (d + 31) / 32);

@@ -45,6 +45,39 @@ cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
 }
 
+// Sums over g < grid of part[g npad + j] for the 8 columns j0 .. j0 + 7, by a CTA
+// of 256 threads: 32 threads per column take every 32nd partial, then
+// shuffles and shared memory (a fixed order).  Column j0 + t on thread t < 8.
+constexpr int kReduceThreads = 256;
+constexpr int kReduceCols = 8;
+__device__ __forceinline__ double sum_partials(const double *__restrict__ part, int grid, int npad,
+                                               int j0,
+                                               double (*red)[kReduceCols]) {
+  constexpr int kGroups = kReduceThreads / kReduceCols;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = threadIdx.x % kReduceCols, j = j0 + c;  // < npad
+  double s0 = 0.0, s1 = 0.0;
+  int g = threadIdx.x / kReduceCols;
+#pragma unroll 4
+  for (; g + kGroups < grid; g += 2 * kGroups) {
+    s0 += part[(size_t)g * npad + j];
+    s1 += part[(size_t)(g + kGroups) * npad + j];
+  }
+  if (g < grid) s0 += part[(size_t)g * npad + j];
+  double s = s0 + s1;
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  if (lane < kReduceCols) red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+    const int q = lane >> 3;
+    s = red[q][c] + red[q + 4][c];
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+  }
+  return s;
+}
+
 // Knuth's TwoSum: s + e = a + b exactly.
 __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) {
   s = __fadd_rn(a, b);

@@ -108,11 +108,24 @@ __device__ __forceinline__ void load_row(const double *__restrict__ row, int n, 
 }
 
 
+// A row for the scatter, lane l holding columns l, l + 32, ...: a warp's atomics on
+// 32 consecutive columns touch 8 or 9 sectors of L2 where the pairs of load_row
+// touch 16, each half used.
+template <int NC>
+__device__ __forceinline__ void load_row_lanes(const double *__restrict__ row, int n, int lane,
+                                               double (&a)[2 * NC]) {
+#pragma unroll
+  for (int k = 0; k < 2 * NC; k++) {
+    const int col = 32 * k + lane;
+    a[k] = (col < n) ? __ldcs(row + col) : 0.0;
+  }
+}
+
 __device__ __forceinline__ double flip_sign(double a, bool neg) {
   return __longlong_as_double(__double_as_longlong(a) ^ (neg ? (long long)0x8000000000000000ull : 0ll));
 }
 
-template <int NC, bool VEC>
+template <int NC>
 __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
     sketch_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int n,
                   const double *__restrict__ b, int d, int zeta, const int32_t *__restrict__ rows,
@@ -130,20 +143,16 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
 
   for (int64_t i = r0 + warp; i < r1; i += nw) {
     double a[2 * NC];
-    load_row<NC, VEC>(A + i * lda, n, lane, a);
+    load_row_lanes<NC>(A + i * lda, n, lane, a);
     const int myh = (lane < zeta) ? rows[i * zeta + lane] : 0;
     const uint32_t sb = signbits[i];
     if (Ahi != nullptr) {  // hi / lo FP32 planes of the row, written as it streams
 #pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        float h0, l0, h1, l1;
-        split_rn(a[2 * k], h0, l0);
-        split_rn(a[2 * k + 1], h1, l1);
-        if (col + 1 < n) {
-          __stcs(reinterpret_cast<float2 *>(Ahi + i * ld32 + col), make_float2(h0, h1));
-          __stcs(reinterpret_cast<float2 *>(Alo + i * ld32 + col), make_float2(l0, l1));
-        } else if (col < n) {
+      for (int k = 0; k < 2 * NC; k++) {
+        const int col = 32 * k + lane;
+        float h0, l0;
+        split_rn(a[k], h0, l0);
+        if (col < n) {
           __stcs(Ahi + i * ld32 + col, h0);
           __stcs(Alo + i * ld32 + col, l0);
         }
@@ -160,10 +169,9 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
       const bool neg = (sb >> t) & 1u;
       double *dst = SAb + (size_t)h * ldsa;
 #pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        if (col < n) atomicAdd(dst + col, flip_sign(a[2 * k], neg));
-        if (col + 1 < n) atomicAdd(dst + col + 1, flip_sign(a[2 * k + 1], neg));
+      for (int k = 0; k < 2 * NC; k++) {
+        const int col = 32 * k + lane;
+        if (col < n) atomicAdd(dst + col, flip_sign(a[k], neg));
       }
     }
   }
@@ -172,11 +180,7 @@ __global__ void __launch_bounds__(kPassThreads, NC >= 16 ? 1 : kPassCtasPerSm)
     __syncthreads();
     if (warp == w) {
 #pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        acc[col] += sq[2 * k];
-        acc[col + 1] += sq[2 * k + 1];
-      }
+      for (int k = 0; k < 2 * NC; k++) acc[32 * k + lane] += sq[k];
     }
   }
   __syncthreads();
@@ -636,23 +640,17 @@ __device__ void b_sketch_body(const BItem &it, int local, int zeta) {
     for (int q = 0; q < cnt; q++) {
       const int64_t i = i0 + q;
       double a[2 * NC];
-      load_row<NC, false>(it.A + i * n, n, lane, a);
+      load_row_lanes<NC>(it.A + i * n, n, lane, a);
 #pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        float h0, l0, h1, l1;
-        split_rn(a[2 * k], h0, l0);
-        split_rn(a[2 * k + 1], h1, l1);
+      for (int k = 0; k < 2 * NC; k++) {
+        const int col = 32 * k + lane;
+        float h0, l0;
+        split_rn(a[k], h0, l0);
         if (col < n) {
           __stcs(it.Ahi + i * it.ld32 + col, h0);
           __stcs(it.Alo + i * it.ld32 + col, l0);
         }
-        if (col + 1 < n) {
-          __stcs(it.Ahi + i * it.ld32 + col + 1, h1);
-          __stcs(it.Alo + i * it.ld32 + col + 1, l1);
-        }
-        sq[2 * k] = fma(a[2 * k], a[2 * k], sq[2 * k]);
-        sq[2 * k + 1] = fma(a[2 * k + 1], a[2 * k + 1], sq[2 * k + 1]);
+        sq[k] = fma(a[k], a[k], sq[k]);
       }
       const uint32_t sb = __shfl_sync(0xffffffffu, sbl, q);
       int myh = -1;
@@ -669,10 +667,9 @@ __device__ void b_sketch_body(const BItem &it, int local, int zeta) {
         const bool neg = (sb >> t) & 1u;
         double *dst = it.SAb + (size_t)h * ldsa;
 #pragma unroll
-        for (int k = 0; k < NC; k++) {
-          const int col = 64 * k + 2 * lane;
-          if (col < n) atomicAdd(dst + col, flip_sign(a[2 * k], neg));
-          if (col + 1 < n) atomicAdd(dst + col + 1, flip_sign(a[2 * k + 1], neg));
+        for (int k = 0; k < 2 * NC; k++) {
+          const int col = 32 * k + lane;
+          if (col < n) atomicAdd(dst + col, flip_sign(a[k], neg));
         }
       }
     }
@@ -682,11 +679,7 @@ __device__ void b_sketch_body(const BItem &it, int local, int zeta) {
     __syncthreads();
     if (warp == w) {
 #pragma unroll
-      for (int k = 0; k < NC; k++) {
-        const int col = 64 * k + 2 * lane;
-        acc[col] += sq[2 * k];
-        acc[col + 1] += sq[2 * k + 1];
-      }
+      for (int k = 0; k < 2 * NC; k++) acc[32 * k + lane] += sq[k];
     }
   }
   __syncthreads();
@@ -783,30 +776,16 @@ cudaError_t launch_sketch_pattern(int64_t m, int d, int zeta, uint64_t seed, int
   return cudaGetLastError();
 }
 
-template <int NC>
-static void sketch_dispatch(bool vec, int grid, cudaStream_t s, const double *A, int64_t lda,
-                            int64_t m, int n, const double *b, int d, int zeta,
-                            const int32_t *rows, const uint32_t *sb, double *SAb, double *part,
-                            int npad, float *Ahi, float *Alo, int64_t ld32) {
-  if (vec)
-    sketch_kernel<NC, true><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, sb, SAb,
-                                                          part, npad, Ahi, Alo, ld32);
-  else
-    sketch_kernel<NC, false><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, sb,
-                                                           SAb, part, npad, Ahi, Alo, ld32);
-}
-
 cudaError_t launch_sketch(const double *A, int64_t lda, int64_t m, int n, const double *b, int d,
                           int zeta, const int32_t *rows, const uint32_t *signbits, double *SAb,
                           double *colsq_part, int grid, int npad, float *Ahi, float *Alo,
                           int64_t ld32, cudaStream_t s) {
-  const bool vec = ((reinterpret_cast<uintptr_t>(A) & 15) == 0) && (lda % 2 == 0);
   switch (npad / 64) {
-    case 1: sketch_dispatch<1>(vec, grid, s, A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
-    case 2: sketch_dispatch<2>(vec, grid, s, A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
-    case 4: sketch_dispatch<4>(vec, grid, s, A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
-    case 8: sketch_dispatch<8>(vec, grid, s, A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
-    case 16: sketch_dispatch<16>(vec, grid, s, A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
+    case 1: sketch_kernel<1><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
+    case 2: sketch_kernel<2><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
+    case 4: sketch_kernel<4><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
+    case 8: sketch_kernel<8><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
+    case 16: sketch_kernel<16><<<grid, kPassThreads, 0, s>>>(A, lda, m, n, b, d, zeta, rows, signbits, SAb, colsq_part, npad, Ahi, Alo, ld32); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -16,7 +16,7 @@ from lsq_problems import problem_svd
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [1, 2, 5, 31, 32, 33, 63, 64, 65, 127, 129, 255, 257, 511, 513, 1021, 1024]
+SIZES = [1, 2, 5, 31, 32, 33, 63, 64, 65, 127, 129, 255, 257, 511, 513, 700, 770, 1021, 1024]
 
 
 @pytest.mark.parametrize("method", ["fossils", "spir", "spir_lsqr"])

@@ -35,11 +35,21 @@
 //    columns first, and the next panel is factored on a second,
 //    high-priority stream while the update of panel p's remaining columns
 //    runs; two events per panel order the streams.
+//    Up to kOneStreamMaxN columns the chain of panels is what takes the time,
+//    and a panel that shares its SMs with update CTAs waits for the FP64 pipe
+//    at every step.  There all launches go to one stream: the next panel's
+//    columns, the next panel with all of its SMs' shared memory, so that it
+//    has them alone, and behind it, as a programmatic dependent that starts
+//    once the panel's CTAs are placed, the update of the remaining columns on
+//    the other SMs (they touch different columns).  The update's last
+//    cluster waits for the panel before it ends, so the launch after it finds
+//    both done.
 // Every wait is bounded; on a timeout the kernel records LSQ_ERR_TIMEOUT,
 // waits (bounded) for the transfers addressed to its CTA and returns.
 #include <atomic>
 
 #include "lsq_cluster.cuh"
+#include "lsq_dev.cuh"
 
 namespace lsq {
 
@@ -53,6 +63,11 @@ constexpr int kMaxClusterQ = 16;
 constexpr int kQbMinN = 64;                 // below: the column-by-column kernel
 constexpr uint64_t kDrainNs = 2000ull * 1000 * 1000;  // transfers a timed-out CTA still awaits
 constexpr size_t kQbSmemMax = 227 * 1024;
+// Up to here all launches on one stream, the panel's CTAs alone on their SMs.
+// ms, two streams / one: d = 12 n, n = 128 0.62 / 0.60, 256 1.65 / 1.43, 333 2.61 /
+// 2.19, 500 5.17 / 5.00, 700 11.06 / 10.94, 1000 26.5 / 26.9; d = 1500, n = 500 2.96 /
+// 2.55.
+constexpr int kOneStreamMaxN = 768;
 
 __device__ __forceinline__ void note_timeout(DevState *st) {
   atomicCAS(&st->err, 0, (int)LSQ_ERR_TIMEOUT);
@@ -123,6 +138,7 @@ __global__ void __launch_bounds__(kQbThreads, 1)
     qr_panel_kernel(double *__restrict__ W, int d, int kb, int bw, int S,
                     double *__restrict__ vhead, double *__restrict__ Tp, DevState *st,
                     uint64_t timeout_ns) {
+  griddep_launch();  // one-stream form: the update behind it may start
   extern __shared__ __align__(16) double psm[];
   const unsigned rank = cluster_rank(), pc = cluster_nranks();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -443,6 +459,8 @@ __global__ void __launch_bounds__(kQbThreads, 2)
   }
   __syncthreads();
   cluster_sync_all();
+  // one-stream form: the grid ends after the panel that it started behind
+  if (blockIdx.x + uc >= gridDim.x) griddep_wait();
 }
 
 std::atomic<int> g_qb_pc[64];  // CTAs of the panel cluster per device (0: not chosen yet)
@@ -483,7 +501,7 @@ int rows_per_cta(int Lp, int c) {
 }
 
 cudaError_t launch_panel(double *W, int d, int kb, int bw, int pc, double *vhead, double *Tp,
-                         DevState *st, uint64_t timeout_ns, cudaStream_t s) {
+                         DevState *st, uint64_t timeout_ns, cudaStream_t s, bool alone = false) {
   const int S = rows_per_cta(d - kb, pc);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -493,7 +511,7 @@ cudaError_t launch_panel(double *W, int d, int kb, int bw, int pc, double *vhead
   at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(pc);
   cfg.blockDim = dim3(kQbThreads);
-  cfg.dynamicSmemBytes = panel_smem_bytes(S, pc);
+  cfg.dynamicSmemBytes = alone ? kQbSmemMax : panel_smem_bytes(S, pc);
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
@@ -503,12 +521,12 @@ cudaError_t launch_panel(double *W, int d, int kb, int bw, int pc, double *vhead
 template <int CPB>
 cudaError_t launch_update(double *W, int d, int kb, int bw, int c0, int c1, int uc,
                           const double *vhead, const double *Tp, DevState *st,
-                          uint64_t timeout_ns, cudaStream_t s) {
+                          uint64_t timeout_ns, cudaStream_t s, bool behind = false) {
   if (c1 <= c0) return cudaSuccess;
   const int blocks = (c1 - c0 + CPB - 1) / CPB;
   const int Su = rows_per_cta(d - kb, uc);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = uc;
   at[0].val.clusterDim.y = 1;
@@ -519,6 +537,11 @@ cudaError_t launch_update(double *W, int d, int kb, int bw, int c0, int c1, int 
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  if (behind) {
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, qr_update_kernel<CPB>, W, d, kb, bw, c0, c1, Su, vhead, Tp, st,
                             timeout_ns);
 }
@@ -561,6 +584,27 @@ cudaError_t launch_qr_blocked(double *W, int d, int n, int ncols, double *vhead,
                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   const int np = (n + kQb - 1) / kQb;
+  if (n <= kOneStreamMaxN) {
+    if ((e = launch_panel(W, d, 0, n < kQb ? n : kQb, pc, vhead, tws, st, timeout_ns, s, true)) !=
+        cudaSuccess)
+      return e;
+    for (int p = 0; p < np; p++) {
+      const int kb = p * kQb, bw = n - kb < kQb ? n - kb : kQb;
+      const int kn = kb + bw, bwn = kn < n ? (n - kn < kQb ? n - kn : kQb) : 0;
+      const double *Tp = tws + (size_t)p * kQb * kQb;
+      if (bwn > 0) {
+        e = launch_update<2>(W, d, kb, bw, kn, kn + bwn, pc, vhead, Tp, st, timeout_ns, s);
+        if (e == cudaSuccess)
+          e = launch_panel(W, d, kn, bwn, pc, vhead, tws + (size_t)(p + 1) * kQb * kQb, st,
+                           timeout_ns, s, true);
+        if (e != cudaSuccess) return e;
+      }
+      e = launch_update<4>(W, d, kb, bw, kn + bwn, ncols, uc, vhead, Tp, st, timeout_ns, s,
+                           bwn > 0);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   // ev[0]: the panel stream starts after the work already on s; ev[1..2]:
   // panel p factored (p & 1); ev[3..4]: panel p's remaining columns updated
   if ((e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;

@@ -82,7 +82,14 @@ __global__ void __launch_bounds__(256)
     b_reduce_kernel(const BItem *__restrict__ items, int mode) {
   __shared__ double red[8][33];
   const BItem &it = items[blockIdx.y];
-  if (mode == 1 && *(volatile const int *)&it.st->done) return;
+  if (mode == 1) {
+    const int done = *(volatile const int *)&it.st->done;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the kernels behind (k_inner.cu)
+      it.st->ugate = done;
+      it.st->par = it.st->iters & 1;
+    }
+    if (done) return;
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
   if (blockIdx.x * 32 >= it.n && !(mode == 0 && blockIdx.x == 0)) return;
@@ -115,51 +122,50 @@ __global__ void __launch_bounds__(256)
 // to m n: every item (all = 1) or only the items whose inner loop is still
 // running (all = 0), so that the last items of a batch get the whole GPU.
 // Writes cta0 / ncta of the table and the CTA -> item map (-1: no item).
-// One CTA; the deal is done by thread 0 in a fixed order.
-__global__ void b_redeal_kernel(BItem *__restrict__ items, int count, int *__restrict__ cta_item,
-                                int grid, int all) {
-  __shared__ int cnt[1024];
-  if (threadIdx.x == 0) {
-    double tot = 0.0;
-    int act = 0;
-    for (int i = 0; i < count; i++) {
-      const bool on = all || !*(volatile const int *)&items[i].st->done;
-      cnt[i] = on ? 1 : 0;
-      if (on) {
-        tot += (double)items[i].m * items[i].n;
-        act++;
-      }
+// One CTA of 256 threads, one per item (count <= 256).
+__global__ void __launch_bounds__(256)
+    b_redeal_kernel(BItem *__restrict__ items, int count, int *__restrict__ cta_item, int grid,
+                    int all) {
+  __shared__ double scratch[8];
+  __shared__ int wcnt[8], woff[8];
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+  const bool on = i < count && (all || !*(volatile const int *)&items[i].st->done);
+  const double mn = on ? (double)items[i].m * items[i].n : 0.0;
+  const double tot = block_sum(mn, scratch);
+  // the item's rank among the active ones, and their number
+  auto rank = [&](int v, int &total) {  // exclusive prefix sum over the CTA
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
-    int used = act;
-    if (act > 0 && grid > act) {
-      const int left = grid - act;
-      for (int i = 0; i < count; i++)
-        if (cnt[i]) {
-          const int f = (int)floor((double)items[i].m * items[i].n / tot * left);
-          cnt[i] += f;
-          used += f;
-        }
-      // the rest one at a time, in item order
-      for (int i = 0; used < grid; i = (i + 1) % count)
-        if (cnt[i]) {
-          cnt[i]++;
-          used++;
-        }
+    __syncthreads();
+    if (lane == 31) wcnt[warp] = x;
+    __syncthreads();
+    if (i < 8) {
+      int b = 0;
+      for (int w = 0; w < i; w++) b += wcnt[w];
+      woff[i] = b;
     }
-    int g = 0;
-    for (int i = 0; i < count; i++) {
-      items[i].cta0 = g;
-      items[i].ncta = cnt[i];
-      g += cnt[i];
-    }
+    __syncthreads();
+    total = woff[7] + wcnt[7];
+    return woff[warp] + x - v;
+  };
+  int act = 0, used = 0, end = 0;
+  const int r = rank(on ? 1 : 0, act);
+  int c = on ? 1 : 0;
+  if (on && grid > act) c += (int)floor(mn / tot * (grid - act));
+  rank(c, used);
+  // the rest one at a time, in item order
+  if (on && act > 0 && grid > used) c += (grid - used) / act + (r < (grid - used) % act ? 1 : 0);
+  const int c0 = rank(c, end);
+  if (i < count) {
+    items[i].cta0 = c0;
+    items[i].ncta = c;
   }
-  __syncthreads();
-  for (int i = 0; i < count; i++) {
-    const int c0 = items[i].cta0, c = items[i].ncta;
-    for (int k = threadIdx.x; k < c; k += blockDim.x) cta_item[c0 + k] = i;
-  }
-  const int g = items[count - 1].cta0 + items[count - 1].ncta;
-  for (int k = g + threadIdx.x; k < grid; k += blockDim.x) cta_item[k] = -1;
+  for (int k = 0; k < c; k++) cta_item[c0 + k] = i;
+  for (int k = end + i; k < grid; k += 256) cta_item[k] = -1;
 }
 
 // Zero every item's sketch accumulator SAb (d x (n + 1)) before the scatter.
@@ -175,7 +181,7 @@ __global__ void b_zero_kernel(const BItem *__restrict__ items) {
 
 cudaError_t launch_b_redeal(BItem *items, int count, int *cta_item, int grid, int all,
                             cudaStream_t s) {
-  if (count > 1024) return cudaErrorInvalidValue;
+  if (count > 256) return cudaErrorInvalidValue;
   b_redeal_kernel<<<1, 256, 0, s>>>(items, count, cta_item, grid, all);
   return cudaGetLastError();
 }

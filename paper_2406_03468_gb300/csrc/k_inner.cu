@@ -51,16 +51,16 @@ constexpr int kInThreads = 32 * kInWarps;
 // 0.6 ms at n = 1000), which start first; it runs beside the first
 // residual pass.  X is written in both layouts, zeros below the diagonal
 // only inside the diagonal blocks (nothing reads below it).
-__global__ void __launch_bounds__(kInvThreads)
-    tri_inv_kernel(const double *__restrict__ Rcm, const double *__restrict__ rinv,
-                   const double *__restrict__ Dt, int n, double *__restrict__ Xcm,
-                   double *__restrict__ Xrm) {
-  extern __shared__ double ism[];
+__device__ __forceinline__ void tri_inv_body(const double *__restrict__ Rcm,
+                                             const double *__restrict__ rinv,
+                                             const double *__restrict__ Dt, int n,
+                                             double *__restrict__ Xcm, double *__restrict__ Xrm,
+                                             int cta, double *ism) {
   const int nb = (n + 31) / 32, ldx = 32 * nb;
   double *xs = ism;                          // kInvCols x ldx: the columns so far
   double *red = ism + kInvCols * ldx;        // 8 x kInvCols x 32 partial sums
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j0 = (gridDim.x - 1 - blockIdx.x) * kInvCols;
+  const int j0 = ((n + kInvCols - 1) / kInvCols - 1 - cta) * kInvCols;
   const int jl = min(n, j0 + kInvCols) - 1;  // last column of this CTA
   for (int I = jl / 32; I >= 0; I--) {
     const int r = 32 * I + lane;
@@ -105,6 +105,14 @@ __global__ void __launch_bounds__(kInvThreads)
   }
 }
 
+__global__ void __launch_bounds__(kInvThreads)
+    tri_inv_kernel(const double *__restrict__ Rcm, const double *__restrict__ rinv,
+                   const double *__restrict__ Dt, int n, double *__restrict__ Xcm,
+                   double *__restrict__ Xrm) {
+  extern __shared__ double ism[];
+  tri_inv_body(Rcm, rinv, Dt, n, Xcm, Xrm, blockIdx.x, ism);
+}
+
 // Sum over the CTA of kInWarps warps, for every thread.
 __device__ __forceinline__ double in_sum(double v, double *scratch) {
   v = warp_sum(v);
@@ -121,12 +129,10 @@ __device__ __forceinline__ double in_sum(double v, double *scratch) {
 //   2 LSQR:    w <- -w / beta - beta v (beta^2 = lq_b2); its share of the norm
 // Latency: the column of X is loaded before the dependency wait, then h.
 template <int NB, int METHOD>
-__global__ void __launch_bounds__(kInThreads)
-    inner_w_kernel(int n, const double *__restrict__ Xcm, const double *h, double *w,
-                   const double *c, double *dy, double *dyold, const double *pv, double *pn,
-                   const DevState *st) {
-  griddep_launch();
-  __shared__ double scratch[kInWarps];
+__device__ __forceinline__ void inner_w_body(int n, const double *__restrict__ Xcm,
+                                             const double *h, double *w, const double *c,
+                                             double *dy, double *dyold, const double *pv,
+                                             double *pn, const DevState *st, double *scratch) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * kInWarps + warp;
   double xr[NB];
@@ -190,6 +196,16 @@ __global__ void __launch_bounds__(kInThreads)
   if (threadIdx.x == 0) pn[blockIdx.x] = (scratch[0] + scratch[1]) + (scratch[2] + scratch[3]);
 }
 
+template <int NB, int METHOD>
+__global__ void __launch_bounds__(kInThreads)
+    inner_w_kernel(int n, const double *__restrict__ Xcm, const double *h, double *w,
+                   const double *c, double *dy, double *dyold, const double *pv, double *pn,
+                   const DevState *st) {
+  griddep_launch();
+  __shared__ double scratch[kInWarps];
+  inner_w_body<NB, METHOD>(n, Xcm, h, w, c, dy, dyold, pv, pn, st, scratch);
+}
+
 __device__ __forceinline__ void u_finish(DevState *st, double dn2, bool exhausted, int *hprog) {
   const int it = st->iters + 1;
   st->iters = it;
@@ -212,18 +228,17 @@ __device__ __forceinline__ void u_finish(DevState *st, double dn2, bool exhauste
 //   METHOD 3:  v = src only (the step's first z; no update, no gate)
 // Entry i of the vectors is written by the warp of row i alone; what every
 // CTA reads (r, p) alternates between two buffers.
+// np: the CTAs (partial sums) of inner_w_kernel, and the index of the last one here
 template <int NB, int METHOD>
-__global__ void __launch_bounds__(kInThreads)
-    inner_u_kernel(int n, const double *__restrict__ Xrm, const double *__restrict__ dinv,
-                   const double *src, double *z, const double *res, double *res_out,
-                   const double *pv, double *pv_out, double *dy, const double *pn, int par,
-                   DevState *st, int *hprog) {
-  __shared__ double scratch[kInWarps];
-  __shared__ double sv[METHOD == 1 ? 32 * NB : 1];
+__device__ __forceinline__ void inner_u_body(int n, int np, const double *__restrict__ Xrm,
+                                             const double *__restrict__ dinv, const double *src,
+                                             double *z, const double *res, double *res_out,
+                                             const double *pv, double *pv_out, double *dy,
+                                             const double *pn, int par, DevState *st, int *hprog,
+                                             double *scratch, double *sv) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * kInWarps + warp;
-  const bool fin = METHOD != 3 && blockIdx.x == gridDim.x - 1;
-  const int np = gridDim.x - 1;  // CTAs of the inner_w_kernel launch
+  const bool fin = METHOD != 3 && (int)blockIdx.x == np;
   double xr[NB], di = 0.0;
 #pragma unroll
   for (int k = 0; k < NB; k++) {
@@ -345,6 +360,18 @@ __global__ void __launch_bounds__(kInThreads)
   }
 }
 
+template <int NB, int METHOD>
+__global__ void __launch_bounds__(kInThreads)
+    inner_u_kernel(int n, const double *__restrict__ Xrm, const double *__restrict__ dinv,
+                   const double *src, double *z, const double *res, double *res_out,
+                   const double *pv, double *pv_out, double *dy, const double *pn, int par,
+                   DevState *st, int *hprog) {
+  __shared__ double scratch[kInWarps];
+  __shared__ double sv[METHOD == 1 ? 32 * NB : 1];
+  inner_u_body<NB, METHOD>(n, gridDim.x - 1, Xrm, dinv, src, z, res, res_out, pv, pv_out, dy, pn,
+                           par, st, hprog, scratch, sv);
+}
+
 // One step of both condition-estimate chains (blockIdx.y): out = M (v / ||v||)
 // with one warp per entry and the CTAs' shares of ||out||^2.
 //   chain 0, sigma_max(R):     M = R, R^T, R, ... (power iteration on R^T R)
@@ -357,14 +384,14 @@ __device__ __forceinline__ double cond_start(int chain, int i) {
 }
 
 template <int NB>
-__global__ void __launch_bounds__(kInThreads)
-    cond_step_kernel(int n, const double *__restrict__ Rcm, const double *__restrict__ Rrm,
-                     const double *__restrict__ Xcm, const double *__restrict__ Xrm, int step,
-                     const double *vin, const double *pin, double *vout, double *pout) {
-  griddep_launch();
-  __shared__ double scratch[kInWarps];
+__device__ __forceinline__ void cond_step_body(int n, int np, const double *__restrict__ Rcm,
+                                               const double *__restrict__ Rrm,
+                                               const double *__restrict__ Xcm,
+                                               const double *__restrict__ Xrm, int step,
+                                               const double *vin, const double *pin, double *vout,
+                                               double *pout, double *scratch) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, chain = blockIdx.y;
-  const int i = blockIdx.x * kInWarps + warp, np = gridDim.x;
+  const int i = blockIdx.x * kInWarps + warp;
   const bool upper = ((step & 1) ^ chain) == 0;  // row i of R or X, else column i
   const double *M = chain == 0 ? (upper ? Rrm : Rcm) : (upper ? Xrm : Xcm);
   double mr[NB], vv[NB];
@@ -407,10 +434,18 @@ __global__ void __launch_bounds__(kInThreads)
     pout[chain * np + blockIdx.x] = (scratch[0] + scratch[1]) + (scratch[2] + scratch[3]);
 }
 
+template <int NB>
 __global__ void __launch_bounds__(kInThreads)
-    cond_finish_kernel(const double *pin, int np, DevState *st) {
-  griddep_wait();
+    cond_step_kernel(int n, const double *__restrict__ Rcm, const double *__restrict__ Rrm,
+                     const double *__restrict__ Xcm, const double *__restrict__ Xrm, int step,
+                     const double *vin, const double *pin, double *vout, double *pout) {
+  griddep_launch();
   __shared__ double scratch[kInWarps];
+  cond_step_body<NB>(n, gridDim.x, Rcm, Rrm, Xcm, Xrm, step, vin, pin, vout, pout, scratch);
+}
+
+__device__ __forceinline__ void cond_finish_body(const double *pin, int np, DevState *st,
+                                                 double *scratch) {
   double s0 = 0.0, s1 = 0.0;
   for (int q = threadIdx.x; q < np; q += kInThreads) {
     s0 += pin[q];
@@ -423,6 +458,114 @@ __global__ void __launch_bounds__(kInThreads)
     const double smin = (winv > 0.0) ? 1.0 / winv : 0.0;
     st->normest = smax;
     st->condest = (smin > 0.0) ? smax / smin : INFINITY;
+  }
+}
+
+__global__ void __launch_bounds__(kInThreads)
+    cond_finish_kernel(const double *pin, int np, DevState *st) {
+  griddep_wait();
+  __shared__ double scratch[kInWarps];
+  cond_finish_body(pin, np, st, scratch);
+}
+
+// Step-2 count: q0 of Theorem 7.1 with kappa := condest and distortion
+// 1.01 eta; Alg. 5 returns dy_(q) after q - 1 updates (as the plan path).
+__device__ int step2_count(double condest, double eta, int max_inner) {
+  const double e = 1.01 * eta;
+  double q0 = 11.0;
+  if (e > 0.0 && isfinite(condest) && condest > 0.0) {
+    const double v = 1.0 + 2.0 * log(1.0 / (condest * kU)) / log(1.0 / e);
+    q0 = v > 11.0 ? v : 11.0;
+  }
+  int q = (int)ceil(q0) - 1;
+  if (q < 1) q = 1;
+  if (q > max_inner) q = max_inner;
+  return q;
+}
+
+// ---------------------------------------------------------------------------
+// The same kernels for the items of a batch (lsq_batch.cu): blockIdx.z is the
+// item.  Ordinary launches inside captured graphs; a CTA beyond its item's
+// entries returns.
+// ---------------------------------------------------------------------------
+
+// Buffers and partial sums of a condition-estimate step in the item's cw.
+__device__ __forceinline__ void b_cond_bufs(const BItem &it, int np, int step, const double *&vi,
+                                            const double *&pi, double *&vo, double *&po) {
+  double *v = it.cw, *p = it.cw + 4 * (size_t)it.n;
+  vi = v + (step & 1) * 2 * (size_t)it.n;
+  vo = v + ((step & 1) ^ 1) * 2 * (size_t)it.n;
+  pi = p + (step & 1) * 2 * (size_t)np;
+  po = p + ((step & 1) ^ 1) * 2 * (size_t)np;
+}
+
+__global__ void __launch_bounds__(kInvThreads) b_tri_inv_kernel(const BItem *__restrict__ items) {
+  extern __shared__ double ism[];
+  const BItem &it = items[blockIdx.z];
+  if ((int)blockIdx.x * kInvCols >= it.n) return;
+  tri_inv_body(it.Rcm, it.rinv, it.Dt, it.n, it.Xcm, it.Xrm, blockIdx.x, ism);
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kInThreads)
+    b_cond_step_kernel(const BItem *__restrict__ items, int step) {
+  __shared__ double scratch[kInWarps];
+  const BItem &it = items[blockIdx.z];
+  const int np = (it.n + kInWarps - 1) / kInWarps;
+  if ((int)blockIdx.x >= np) return;
+  const double *vi, *pi;
+  double *vo, *po;
+  b_cond_bufs(it, np, step, vi, pi, vo, po);
+  cond_step_body<NB>(it.n, np, it.Rcm, it.Rrm, it.Xcm, it.Xrm, step, vi, pi, vo, po, scratch);
+}
+
+// condest / normest and the step-2 count (Theorem 7.1 with kappa := condest)
+__global__ void __launch_bounds__(kInThreads)
+    b_cond_finish_kernel(const BItem *__restrict__ items, int last, int max_inner) {
+  __shared__ double scratch[kInWarps];
+  const BItem &it = items[blockIdx.z];
+  const int np = (it.n + kInWarps - 1) / kInWarps;
+  const double *vi, *pi;
+  double *vo, *po;
+  b_cond_bufs(it, np, last + 1, vi, pi, vo, po);
+  cond_finish_body(pi, np, it.st, scratch);
+  if (threadIdx.x == 0) it.st->q2 = step2_count(it.st->condest, it.eta, max_inner);
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kInThreads) b_inner_w_kernel(const BItem *__restrict__ items) {
+  __shared__ double scratch[kInWarps];
+  const BItem &it = items[blockIdx.z];
+  if ((int)blockIdx.x * kInWarps >= it.n) return;
+  if (it.method == 0)
+    inner_w_body<NB, 0>(it.n, it.Xcm, it.h, it.w, it.c, it.dy, it.dyold, nullptr, it.pn, it.st,
+                        scratch);
+  else
+    inner_w_body<NB, 1>(it.n, it.Xcm, it.h, it.w, it.c, it.dy, it.dyold,
+                        it.st->par ? it.p2 : it.p, it.pn, it.st, scratch);
+}
+
+// first = 1: the step's first z
+template <int NB>
+__global__ void __launch_bounds__(kInThreads)
+    b_inner_u_kernel(const BItem *__restrict__ items, int first) {
+  __shared__ double scratch[kInWarps];
+  __shared__ double sv[32 * NB];
+  const BItem &it = items[blockIdx.z];
+  const int np = (it.n + kInWarps - 1) / kInWarps;
+  if ((int)blockIdx.x > np) return;
+  if (first) {
+    inner_u_body<NB, 3>(it.n, np, it.Xrm, it.dinv, it.method == 0 ? it.dy : it.p, it.z, nullptr,
+                        nullptr, nullptr, nullptr, nullptr, nullptr, 0, it.st, nullptr, scratch,
+                        sv);
+  } else if (it.method == 0) {
+    inner_u_body<NB, 0>(it.n, np, it.Xrm, it.dinv, it.dy, it.z, nullptr, nullptr, nullptr, nullptr,
+                        it.dy, it.pn, 0, it.st, nullptr, scratch, sv);
+  } else {
+    const int par = it.st->par;
+    inner_u_body<NB, 1>(it.n, np, it.Xrm, it.dinv, it.w, it.z, par ? it.res2 : it.res,
+                        par ? it.res : it.res2, par ? it.p2 : it.p, par ? it.p : it.p2, it.dy,
+                        it.pn, par, it.st, nullptr, scratch, sv);
   }
 }
 
@@ -516,6 +659,33 @@ cudaError_t launch_condest(const double *Rcm, const double *Rrm, const double *X
   });
   return launch_pdl(cond_finish_kernel, dim3(1), dim3(kInThreads), 0, s,
                     (const double *)p[1], np, st);
+}
+
+cudaError_t launch_b_cond(const BItem *items, int count, int nmax, int iters, int max_inner,
+                          cudaStream_t s) {
+  const int nb = (nmax + 31) / 32;
+  const size_t smem =
+      sizeof(double) * (size_t)(kInvCols * 32 * nb + (kInvThreads / 32) * kInvCols * 32);
+  b_tri_inv_kernel<<<dim3((nmax + kInvCols - 1) / kInvCols, 1, count), kInvThreads, smem, s>>>(items);
+  const dim3 grid(inner_partials(nmax), 2, count);
+  LSQ_NB_SWITCH(nmax, {
+    for (int k = 0; k <= 2 * iters; k++)
+      b_cond_step_kernel<NB><<<grid, kInThreads, 0, s>>>(items, k);
+  });
+  b_cond_finish_kernel<<<dim3(1, 1, count), kInThreads, 0, s>>>(items, 2 * iters, max_inner);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_b_w(const BItem *items, int count, int nmax, cudaStream_t s) {
+  const dim3 grid(inner_partials(nmax), 1, count);
+  LSQ_NB_SWITCH(nmax, { b_inner_w_kernel<NB><<<grid, kInThreads, 0, s>>>(items); });
+  return cudaGetLastError();
+}
+
+cudaError_t launch_b_u(const BItem *items, int count, int nmax, int first, cudaStream_t s) {
+  const dim3 grid(inner_partials(nmax) + 1, 1, count);
+  LSQ_NB_SWITCH(nmax, { b_inner_u_kernel<NB><<<grid, kInThreads, 0, s>>>(items, first); });
+  return cudaGetLastError();
 }
 
 cudaError_t launch_inner_w(int method, const InnerVecs &v, int par, cudaStream_t s) {

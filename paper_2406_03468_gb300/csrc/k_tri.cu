@@ -1,8 +1,7 @@
 // Triangular solves with the preconditioner R by back substitution (the
 // analysis computes every R^{-1} z and R^{-T} z this way: Sec. 6, notation,
-// and Proposition 6.5), and the condest / normest estimates of R that the
-// step-1 stopping rule and the q0 count use (Sec. 4.2; Alg. 4 reads them off
-// the SVD of SA, whose singular values equal those of R).
+// and Proposition 6.5): c, x0 and the updates of x.  (An inner iteration's
+// solves and the condition estimate are products with R^-1, k_inner.cu.)
 //
 // One CTA per solve: the vector lives in shared memory; R (n x n) is read
 // from L2 in both layouts so that every access is coalesced -- column j of R
@@ -191,91 +190,14 @@ __global__ void __launch_bounds__(kVecThreads)
   }
 }
 
-// y = R v (upper, via the column-major copy) or y = R^T v (via the row-major copy).
-__device__ void block_trmv(const double *__restrict__ Rcm, const double *__restrict__ Rrm, int n,
-                           int trans, const double *sv, double *sy) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double acc = 0.0;
-    if (!trans) {
-      for (int j = i; j < n; j++) acc = fma(Rcm[(size_t)j * n + i], sv[j], acc);
-    } else {
-      for (int j = 0; j <= i; j++) acc = fma(Rrm[(size_t)j * n + i], sv[j], acc);
-    }
-    sy[i] = acc;
-  }
-  __syncthreads();
-}
-
-__device__ double block_normalize(double *sv, int n, double *scratch) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s = fma(sv[i], sv[i], s);
-  s = sqrt(block_sum(s, scratch));
-  const double inv = (s > 0.0) ? 1.0 / s : 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) sv[i] *= inv;
-  __syncthreads();
-  return s;
-}
-
-// sigma_max(R) by power iteration on R^T R and sigma_min(R) by inverse power
-// iteration on (R^T R)^{-1}, from a fixed start vector (the batched engine's
-// items; a plan's estimate is launch_condest in k_inner.cu).
-__device__ void condest_body(const double *__restrict__ Rcm, const double *__restrict__ Rrm,
-                             const double *__restrict__ rinv, const double *__restrict__ Dt, int n,
-                             int iters, DevState *st, double *sm) {
-  double *v = sm, *y = sm + n, *scratch = sm + 2 * n, *tile = scratch + 32;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = 1.0 + 0.25 * (double)((i * 7919) % 17);
-  __syncthreads();
-  block_normalize(v, n, scratch);
-  double smax = 0.0;
-  for (int it = 0; it < iters; it++) {
-    block_trmv(Rcm, Rrm, n, 0, v, y);
-    block_trmv(Rcm, Rrm, n, 1, y, v);
-    block_normalize(v, n, scratch);
-  }
-  block_trmv(Rcm, Rrm, n, 0, v, y);
-  smax = block_normalize(y, n, scratch);
-
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = 1.0 + 0.25 * (double)((i * 104729) % 13);
-  __syncthreads();
-  block_normalize(v, n, scratch);
-  double winv = 0.0;
-  for (int it = 0; it <= iters; it++) {
-    block_trsv(Rcm, Rrm, rinv, Dt, n, 1, v, tile);  // v <- R^{-T} v
-    winv = block_normalize(v, n, scratch);
-    if (it == iters) break;
-    block_trsv(Rcm, Rrm, rinv, Dt, n, 0, v, tile);  // v <- R^{-1} v
-    block_normalize(v, n, scratch);
-  }
-  if (threadIdx.x == 0) {
-    const double smin = (winv > 0.0) ? 1.0 / winv : 0.0;
-    st->normest = smax;
-    st->condest = (smin > 0.0) ? smax / smin : INFINITY;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Batched forms (one CTA of kVecThreads per item, lsq_batch.cu).
 // ---------------------------------------------------------------------------
 
-// Step-2 count: q0 of Theorem 7.1 with kappa := condest and distortion
-// 1.01 eta; Alg. 5 returns dy_(q) after q - 1 updates (as the plan path).
-__device__ int step2_count(double condest, double eta, int max_inner) {
-  const double e = 1.01 * eta;
-  double q0 = 11.0;
-  if (e > 0.0 && isfinite(condest) && condest > 0.0) {
-    const double v = 1.0 + 2.0 * log(1.0 / (condest * kU)) / log(1.0 / e);
-    q0 = v > 11.0 ? v : 11.0;
-  }
-  int q = (int)ceil(q0) - 1;
-  if (q < 1) q = 1;
-  if (q > max_inner) q = max_inner;
-  return q;
-}
-
-// After the QR: R (both layouts), 1/R_ii, t, the scaled diagonal tiles,
-// condest / normest, x0 = R^-1 t (xs; xo = D^-1 xs; ||x0||^2) and q2.
+// After the QR: R (both layouts), 1/R_ii, t, the scaled diagonal tiles and
+// x0 = R^-1 t (xs; xo = D^-1 xs; ||x0||^2).
 __global__ void __launch_bounds__(kVecThreads)
-    b_setup_kernel(const BItem *__restrict__ items, int iters, int max_inner) {
+    b_setup_kernel(const BItem *__restrict__ items) {
   extern __shared__ double sm[];
   const BItem &it = items[blockIdx.x];
   const int n = it.n, d = it.d, nb = (n + 31) / 32;
@@ -297,8 +219,6 @@ __global__ void __launch_bounds__(kVecThreads)
     it.Dt[idx] = (jj < len && l < len) ? Rb[(size_t)(j0 + jj) * n + j0 + l] * it.rinv[j0 + l] : 0.0;
   }
   __syncthreads();
-  condest_body(it.Rcm, it.Rrm, it.rinv, it.Dt, n, iters, it.st, sm);
-  __syncthreads();
   double *sy = sm, *scratch = sm + n, *tile = scratch + 32;
   for (int i = threadIdx.x; i < n; i += blockDim.x) sy[i] = it.t[i];
   __syncthreads();
@@ -312,34 +232,27 @@ __global__ void __launch_bounds__(kVecThreads)
   nrm = block_sum(nrm, scratch);
   if (threadIdx.x == 0) {
     it.st->x0norm2 = nrm;
-    it.st->q2 = step2_count(it.st->condest, it.eta, max_inner);
     it.st->alpha = it.alpha;
     it.st->beta = it.beta;
   }
 }
 
-// The triangular solves of the refinement loop for every item (see
+// The triangular solves outside the inner loop for every item (see
 // launch_b_trsv for the modes).
 __global__ void __launch_bounds__(kVecThreads)
     b_trsv_kernel(const BItem *__restrict__ items, int mode, int step) {
   const BItem &it = items[blockIdx.x];
-  if (mode <= 1 && *(volatile const int *)&it.st->done) return;
   extern __shared__ double sm[];
   const int n = it.n;
   double *sy = sm, *scratch = sm + n, *tile = scratch + 32;
-  const double *src = mode == 0 ? (it.method == 0 ? it.dy : it.p)
-                      : mode == 1 ? it.h : mode == 2 ? it.g : it.dy;
+  const double *src = mode == 2 ? it.g : it.dy;
   for (int i = threadIdx.x; i < n; i += blockDim.x) sy[i] = src[i];
   __syncthreads();
-  block_trsv(it.Rcm, it.Rrm, it.rinv, it.Dt, n, (mode == 1 || mode == 2) ? 1 : 0, sy, tile);
+  block_trsv(it.Rcm, it.Rrm, it.rinv, it.Dt, n, mode == 2 ? 1 : 0, sy, tile);
   double nrm = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const double x = sy[i];
-    if (mode == 0) {
-      it.z[i] = it.dinv[i] * x;
-    } else if (mode == 1) {
-      it.w[i] = x;
-    } else if (mode == 2) {
+    if (mode == 2) {
       it.c[i] = x;
       nrm = fma(x, x, nrm);
     } else {
@@ -618,12 +531,11 @@ cudaError_t prepare_b_kernels(int nmax) {
   return e;
 }
 
-cudaError_t launch_b_setup(const BItem *items, int count, int cond_iters, int max_inner,
-                           int nmax, cudaStream_t s) {
+cudaError_t launch_b_setup(const BItem *items, int count, int nmax, cudaStream_t s) {
   const size_t smem = (size_t)(2 * nmax + 32 + 3 * kTile) * sizeof(double);
   cudaError_t e = ensure_smem_attr((const void *)b_setup_kernel, (int)smem);
   if (e != cudaSuccess) return e;
-  b_setup_kernel<<<count, kVecThreads, smem, s>>>(items, cond_iters, max_inner);
+  b_setup_kernel<<<count, kVecThreads, smem, s>>>(items);
   return cudaGetLastError();
 }
 

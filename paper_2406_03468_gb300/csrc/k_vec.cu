@@ -1,5 +1,7 @@
-// n-vector steps of the inner solvers, one CTA each (n <= LSQ_MAX_N; a plan's
-// iterations run them inside k_inner.cu's kernels, the batched engine here):
+// n-vector kernels around the inner solvers, one CTA each (n <= LSQ_MAX_N): the
+// inner solvers' starts, the step thresholds, the sketched Karlson-Walden
+// estimate's vector steps.  The solvers themselves, whose updates run inside
+// k_inner.cu's kernels:
 //   Polyak heavy ball (Alg. 5, in the loop form of Alg. 4):
 //     Delta = alpha (c - M dy) + beta (dy - dy_old);  (dy, dy_old) <- (dy + Delta, dy)
 //   conjugate gradient on M dy = c from dy = 0 (Alg. 3's inner solver)
@@ -34,7 +36,6 @@ __device__ void inner_init_body(int method, int n, const double *__restrict__ c,
   }
   s = block_sum(s, scratch);
   if (threadIdx.x == 0) {
-    st->rho = s;
     st->rho_ab[0] = s;
     st->iters = 0;
     st->max_iters = max_iters;
@@ -53,59 +54,6 @@ __global__ void __launch_bounds__(kVecThreads)
   inner_init_body(method, n, c, dy, dy_old, res, p, max_iters, use_thresh, st);
 }
 
-__device__ __forceinline__ void finish_update(DevState *st, double dn2, bool exhausted) {
-  const int it = st->iters + 1;
-  st->iters = it;
-  st->dnorm2 = dn2;
-  bool stop = it >= st->max_iters || exhausted;
-  if (st->use_thresh && sqrt(dn2) <= st->thresh1) stop = true;
-  if (stop) st->done = 1;
-}
-
-__device__ void polyak_body(int n, const double *__restrict__ c, const double *__restrict__ w,
-                            double *dy, double *dy_old, DevState *st) {
-  __shared__ double scratch[32];
-  const double alpha = st->alpha, beta = st->beta;
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double y = dy[i];
-    const double delta = alpha * (c[i] - w[i]) + beta * (y - dy_old[i]);
-    dy_old[i] = y;
-    dy[i] = y + delta;
-    s = fma(delta, delta, s);
-  }
-  s = block_sum(s, scratch);
-  if (threadIdx.x == 0) finish_update(st, s, false);
-}
-
-__device__ void cg_body(int n, const double *__restrict__ q, double *p, double *res, double *dy,
-                        DevState *st) {
-  __shared__ double scratch[32];
-  double pq = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) pq = fma(p[i], q[i], pq);
-  pq = block_sum(pq, scratch);
-  const double rho = st->rho;
-  const double gam = rho / pq;
-  double rr = 0.0, ss = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double step = gam * p[i];
-    dy[i] += step;
-    const double r = res[i] - gam * q[i];
-    res[i] = r;
-    rr = fma(r, r, rr);
-    ss = fma(step, step, ss);
-  }
-  rr = block_sum(rr, scratch);
-  ss = block_sum(ss, scratch);
-  const double bet = rr / rho;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = res[i] + bet * p[i];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    st->rho = rr;
-    finish_update(st, ss, !(rr > 0.0));
-  }
-}
-
 // Batched forms (one CTA per item, lsq_batch.cu).  b_init: at step 0 the
 // step-1 threshold (as set_thresh) and the cap max_inner with the threshold
 // test; at step 1 the cap q2 (set by b_setup from condest), no threshold.
@@ -120,13 +68,6 @@ __global__ void __launch_bounds__(kVecThreads)
   const int cap = step == 0 ? max_inner : st->q2;
   inner_init_body(it.method, it.n, it.c, it.dy, it.dyold, it.res, it.p, cap, step == 0 ? 1 : 0,
                   st);
-}
-
-__global__ void __launch_bounds__(kVecThreads) b_update_kernel(const BItem *__restrict__ items) {
-  const BItem &it = items[blockIdx.x];
-  if (*(volatile int *)&it.st->done) return;
-  if (it.method == 0) polyak_body(it.n, it.c, it.w, it.dy, it.dyold, it.st);
-  else cg_body(it.n, it.w, it.p, it.res, it.dy, it.st);
 }
 
 __global__ void b_copy_x_kernel(const BItem *__restrict__ items) {
@@ -208,11 +149,6 @@ cudaError_t launch_inner_init(int method, int n, const double *c, double *dy, do
 cudaError_t launch_b_init(const BItem *items, int count, int step, int max_inner, double gamma,
                           double rho, cudaStream_t s) {
   b_init_kernel<<<count, kVecThreads, 0, s>>>(items, step, max_inner, gamma, rho);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_b_update(const BItem *items, int count, cudaStream_t s) {
-  b_update_kernel<<<count, kVecThreads, 0, s>>>(items);
   return cudaGetLastError();
 }
 

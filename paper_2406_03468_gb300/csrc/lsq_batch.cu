@@ -95,7 +95,7 @@ namespace {
 
 // Byte layout of one item's slice of the workspace.
 struct Slice {
-  size_t SAb, W, Rcm, Rrm, Dt, vhead, vec, qflag, total;
+  size_t SAb, W, Rcm, Rrm, Xcm, Xrm, Dt, vhead, vec, cw, qflag, total;
 };
 
 Slice slice_layout(int64_t nmax) {
@@ -106,9 +106,12 @@ Slice slice_layout(int64_t nmax) {
   L.W = o; o += a256(sizeof(double) * d * (n + 1));
   L.Rcm = o; o += a256(sizeof(double) * n * n);
   L.Rrm = o; o += a256(sizeof(double) * n * n);
+  L.Xcm = o; o += a256(sizeof(double) * n * n);
+  L.Xrm = o; o += a256(sizeof(double) * n * n);
   L.Dt = o; o += a256(sizeof(double) * 2 * nb * 1024);
   L.vhead = o; o += a256(sizeof(double) * 2 * d);
-  L.vec = o; o += a256(sizeof(double) * 17 * n);
+  L.vec = o; o += a256(sizeof(double) * 20 * n);
+  L.cw = o; o += a256(sizeof(double) * (cond_work((int)n)));
   L.qflag = o; o += a256(sizeof(int) * (n + 1));
   L.total = o;
   return L;
@@ -326,12 +329,15 @@ extern "C" lsq_status lsq_batch_solve(lsq_batch B, int count, lsq_batch_item *it
     it.W = (double *)(base + L.W);
     it.Rcm = (double *)(base + L.Rcm);
     it.Rrm = (double *)(base + L.Rrm);
+    it.Xcm = (double *)(base + L.Xcm);
+    it.Xrm = (double *)(base + L.Xrm);
+    it.cw = (double *)(base + L.cw);
     it.Dt = (double *)(base + L.Dt);
     it.vhead = (double *)(base + L.vhead);
     double *v = (double *)(base + L.vec);
     const int64_t nm = B->n_max;
     double **vs[] = {&it.dcol, &it.dinv, &it.rinv, &it.t, &it.xs, &it.xo, &it.c, &it.g, &it.dy,
-                     &it.dyold, &it.z, &it.h, &it.w, &it.res, &it.p};
+                     &it.dyold, &it.z, &it.h, &it.w, &it.res, &it.p, &it.res2, &it.p2, &it.pn};
     for (size_t k = 0; k < sizeof(vs) / sizeof(vs[0]); k++) *vs[k] = v + k * nm;
     it.Ahi = B->planes + poff;
     it.Alo = B->planes + B->elems_max + poff;
@@ -409,14 +415,16 @@ extern "C" lsq_status lsq_batch_solve(lsq_batch B, int count, lsq_batch_item *it
     return e;
   };
   auto setup = [&]() -> cudaError_t {
-    return launch_b_setup(B->d_items, count, kCondIters, 100, nmax, B->s);
+    cudaError_t e = launch_b_setup(B->d_items, count, nmax, B->s);
+    if (e == cudaSuccess) e = launch_b_cond(B->d_items, count, nmax, kCondIters, 100, B->s);
+    return e;
   };
   if (per_sm == 0) {
     // tune: time the residual pass over this batch (it only writes partials,
     // which the solve overwrites) at 1, 2 and 4 CTAs per SM, with x = 0: the
     // same traffic as in the solve
     for (int i = 0; i < count; i++)
-      BCU(cudaMemsetAsync(B->h_items[i].dcol, 0, sizeof(double) * 17 * (size_t)B->n_max, B->s));
+      BCU(cudaMemsetAsync(B->h_items[i].dcol, 0, sizeof(double) * 20 * (size_t)B->n_max, B->s));
     float best = 1e30f;
     cudaEvent_t e0, e1;
     BCU(cudaEventCreate(&e0));
@@ -461,17 +469,17 @@ extern "C" lsq_status lsq_batch_solve(lsq_batch B, int count, lsq_batch_item *it
         if (e == cudaSuccess) e = launch_b_reduce(B->d_items, count, nmax, 0, B->s);
         if (e == cudaSuccess) e = launch_b_trsv(B->d_items, count, 2, step, nmax, B->s);
         if (e == cudaSuccess) e = launch_b_init(B->d_items, count, step, 100, gam, rho, B->s);
+        if (e == cudaSuccess) e = launch_b_u(B->d_items, count, nmax, 1, B->s);
         return e;
       });
       if (st < 0) return st;
     }
     st = capture(B, &G.iter, [&]() -> cudaError_t {
       cudaError_t e = launch_b_redeal(B->d_items, count, B->d_cta, B->grid, 0, B->s);
-      if (e == cudaSuccess) e = launch_b_trsv(B->d_items, count, 0, 0, nmax, B->s);
       if (e == cudaSuccess) e = launch_b_inner(B->d_items, B->d_cta, B->grid, B->s);
       if (e == cudaSuccess) e = launch_b_reduce(B->d_items, count, nmax, 1, B->s);
-      if (e == cudaSuccess) e = launch_b_trsv(B->d_items, count, 1, 0, nmax, B->s);
-      if (e == cudaSuccess) e = launch_b_update(B->d_items, count, B->s);
+      if (e == cudaSuccess) e = launch_b_w(B->d_items, count, nmax, B->s);
+      if (e == cudaSuccess) e = launch_b_u(B->d_items, count, nmax, 0, B->s);
       return e;
     });
     if (st < 0) return st;

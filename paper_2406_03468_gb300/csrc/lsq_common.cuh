@@ -33,7 +33,6 @@ struct DevState {
   double thresh1;        // step-1 stop threshold
   double alpha, beta;    // Polyak coefficients
   double dnorm2;         // ||Delta||^2 of the last inner update
-  double rho;            // CG: r^T r
   double r2;             // ||b - A x||^2 of the last residual pass
   double x0norm2;        // ||x0||^2 (scaled coordinates)
   double cnorm2[LSQ_MAX_REFINE];
@@ -49,7 +48,8 @@ struct DevState {
   // rotation's phibar, rhobar (by the iteration's parity), the next pass's
   // coefficient of s, and the last pass's ||s||^2
   double lq_alpha, lq_beta, lq_phibar[2], lq_rhobar[2], lq_bscale, lq_b2;
-  double rho_ab[2];      // CG on a plan: r^T r by the iteration's parity
+  double rho_ab[2];      // CG: r^T r by the iteration's parity
+  int par;               // batched solves: parity of the iteration (set with ugate)
   int ugate;             // `done` as the reduction before the small kernels saw it (k_inner.cu)
   // sketched Karlson-Walden estimate (Alg. 4's step-2 test): ||b||^2, and
   // for the iterate checked ||x||^2 (scaled coordinates), ||r||^2, the
@@ -70,7 +70,8 @@ struct BItem {
   uint64_t seed;
   double eta, alpha, beta;  // distortion and Polyak coefficients (Sec. 2.3, 4.2)
   double *SAb, *W, *part, *r2part, *dcol, *dinv, *Rcm, *Rrm, *rinv, *Dt, *t, *vhead;
-  double *xs, *xo, *c, *g, *dy, *dyold, *z, *h, *w, *res, *p;
+  double *xs, *xo, *c, *g, *dy, *dyold, *z, *h, *w, *res, *p, *res2, *p2;
+  double *Xcm, *Xrm, *pn, *cw;  // R^-1, partial sums, condition estimate (k_inner.cu)
   float *Ahi, *Alo;     // hi / lo FP32 planes (m x ld32)
   DevState *st;
   int *qflag;           // QR: per-column ready flags (n)
@@ -426,12 +427,16 @@ int b_qr_min_ctas(int n);
 // QR of every item's sketch, one launch per column step k = -1 .. nmax - 1
 // (qcta CTAs per item).
 cudaError_t launch_b_qr_step(const BItem *items, int count, int qcta, int k, cudaStream_t s);
-// R, 1/R_ii, t, the scaled diagonal tiles, condest / normest, x0 and the
-// step-2 count q2 (into st->max_iters of the item's state, read by b_init).
-cudaError_t launch_b_setup(const BItem *items, int count, int cond_iters, int max_inner,
-                           int nmax, cudaStream_t s);
-// mode 0: z = D^-1 R^-1 (dy or p) (gated); 1: w = R^-T h (gated);
-// 2: c = R^-T g and ||c||^2 into st->cnorm2[step]; 3: xs += R^-1 dy, xo = D^-1 xs.
+// R, 1/R_ii, t, the scaled diagonal tiles and x0; then R^-1, condest / normest
+// and the step-2 count q2 (into st->q2, read by b_init).
+cudaError_t launch_b_setup(const BItem *items, int count, int nmax, cudaStream_t s);
+cudaError_t launch_b_cond(const BItem *items, int count, int nmax, int iters, int max_inner,
+                          cudaStream_t s);
+// The inner iteration after the reduction: w = R^-T h and the update's first
+// half; its second half and the next z (first = 1: the step's first z).
+cudaError_t launch_b_w(const BItem *items, int count, int nmax, cudaStream_t s);
+cudaError_t launch_b_u(const BItem *items, int count, int nmax, int first, cudaStream_t s);
+// mode 2: c = R^-T g and ||c||^2 into st->cnorm2[step]; 3: xs += R^-1 dy, xo = D^-1 xs.
 cudaError_t launch_b_trsv(const BItem *items, int count, int mode, int step, int nmax,
                           cudaStream_t s);
 cudaError_t launch_b_resid(const BItem *items, const int *cta_item, int grid, cudaStream_t s);
@@ -441,7 +446,6 @@ cudaError_t launch_b_reduce(const BItem *items, int count, int nmax, int mode, c
 // Step thresholds (step 0) and the inner solver's start for step `step`.
 cudaError_t launch_b_init(const BItem *items, int count, int step, int max_inner, double gamma,
                           double rho, cudaStream_t s);
-cudaError_t launch_b_update(const BItem *items, int count, cudaStream_t s);
 cudaError_t launch_b_copy_x(const BItem *items, int count, cudaStream_t s);
 
 // Sketched Karlson-Walden estimate (k_vec.cu).  launch_bnorm2: st->bnorm2 =

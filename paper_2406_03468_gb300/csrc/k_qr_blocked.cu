@@ -60,7 +60,9 @@ constexpr int kQbThreads = 256;
 constexpr int kQbWarps = kQbThreads / 32;
 static_assert(kQb == 2 * kQbWarps, "the panel's warps take two columns each");
 constexpr int kMaxClusterQ = 16;
-constexpr int kQbMinN = 64;                 // below: the column-by-column kernel
+// Below: the column-by-column kernel.  ms, that kernel / this form (d = 12 n): n = 8
+// 0.072 / 0.057, 16 0.121 / 0.080, 32 0.217 / 0.146, 50 0.336 / 0.245, 60 0.403 / 0.277.
+constexpr int kQbMinN = 8;
 constexpr uint64_t kDrainNs = 2000ull * 1000 * 1000;  // transfers a timed-out CTA still awaits
 constexpr size_t kQbSmemMax = 227 * 1024;
 // Up to here all launches on one stream, the panel's CTAs alone on their SMs.

@@ -551,9 +551,12 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
     }
     const bool planes = P->planes_pending;
     P->planes_pending = false;
+    // CTAs (and partial sums) of the residual pass
+    const int gres =
+        P->csr.rp ? csr_pass_grid(P->m, P->csr.nnz, P->npad, P->nsm, P->gpass) : P->gpass;
     if (P->csr.rp)
-      LSQ_CU(launch_csr_pass(1, P->csr.rp, P->csr.col, P->csr.val, P->m, db, P->xo, P->part,
-                             P->r2part, P->gpass, P->npad, nullptr, nullptr,
+      LSQ_CU(launch_csr_pass(1, P->csr.rp, P->csr.col, P->csr.val, P->m, n, P->csr.nnz, db, P->xo,
+                             P->part, P->r2part, gres, P->npad, nullptr, nullptr,
                              method == 2 ? P->lsqr_s : nullptr, P->s));
     else
       LSQ_CU(launch_pass_resid(dA, P->lda, P->m, n, db, P->xo, P->part, P->r2part, P->gpass,
@@ -562,7 +565,7 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
                                method == 2 ? P->lsqr_s : nullptr));
     if (tk >= 0) LSQ_CU(cudaEventRecord(P->tev[2 * tk + 1], P->s));
     P->launches += 3 + (i == 0 ? 1 : 0) + 1;  // resid, reduce, trsv, [thresh], init
-    LSQ_CU(launch_reduce(P->part, P->gpass, P->npad, n, P->dinv, P->g, P->r2part, &P->st->r2,
+    LSQ_CU(launch_reduce(P->part, gres, P->npad, n, P->dinv, P->g, P->r2part, &P->st->r2,
                          nullptr, P->s));
     passes++;
     LSQ_CU(launch_trsv(P->Rcm, P->Rrm, P->rinv, P->Dt, n, 1, P->g, nullptr, P->c, nullptr, nullptr,
@@ -600,7 +603,7 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
     const bool df = P->use_df && !kw, eft = P->use_eft && !kw;
     // CTAs (and partial sums) of the step's inner passes
     const int gin = (P->csr.rp == nullptr && (df || tier))
-                        ? pass_df_grid(P->m, n, P->ld32, P->gpass) : P->gpass;
+                        ? pass_df_grid(P->m, n, P->ld32, P->gpass) : gres;
     // the step's first z = D^{-1} R^{-1} (dy or p)
     const InnerVecs iv = {n, P->Xcm, P->Xrm, P->dinv, P->h, P->c, P->w, P->z, P->dy, P->dyold,
                           {P->res, P->res2}, {P->p, P->p2}, P->pn, P->st, P->hprog};
@@ -616,9 +619,9 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
         LSQ_CU(cudaEventRecord(P->tev[2 * tj], P->s));
       }
       if (P->csr.rp)
-        LSQ_CU(launch_csr_pass(method == 2 ? 1 : 0, P->csr.rp, P->csr.col, P->csr.val, P->m,
-                               method == 2 ? P->lsqr_s : nullptr, P->z, P->part, P->r2part,
-                               P->gpass, P->npad, P->st,
+        LSQ_CU(launch_csr_pass(method == 2 ? 1 : 0, P->csr.rp, P->csr.col, P->csr.val, P->m, n,
+                               P->csr.nnz, method == 2 ? P->lsqr_s : nullptr, P->z, P->part,
+                               P->r2part, gin, P->npad, P->st,
                                method == 2 ? &P->st->lq_bscale : nullptr,
                                method == 2 ? P->lsqr_s : nullptr, P->s));
       else if (method == 2 && df)

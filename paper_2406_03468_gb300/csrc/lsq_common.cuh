@@ -213,9 +213,13 @@ cudaError_t launch_csr_sketch(const int64_t *rp, const int32_t *col, const doubl
                               const uint32_t *signbits, double *SAb, double *colsq_part, int grid,
                               int npad, cudaStream_t s);
 cudaError_t launch_csr_pass(int mode, const int64_t *rp, const int32_t *col, const double *val,
-                            int64_t m, const double *b, const double *x, double *part,
-                            double *r2_part, int grid, int npad, const DevState *gate,
-                            const double *bscale, double *rout, cudaStream_t s);
+                            int64_t m, int n, int64_t nnz, const double *b, const double *x,
+                            double *part, double *r2_part, int grid, int npad,
+                            const DevState *gate, const double *bscale, double *rout,
+                            cudaStream_t s);
+// CTAs (and partial sums) that a pass takes of `grid`: one wave of them, and
+// 8 rows for every warp.
+int csr_pass_grid(int64_t m, int64_t nnz, int npad, int nsm, int grid);
 // Real embedding of a complex m x n row-major A (lda complex entries per row,
 // (re, im) interleaved, 16-byte aligned) into E (2m x 2n, row-major).
 cudaError_t launch_embed_complex(const double *A, int64_t lda, int64_t m, int n, double *E,

@@ -13,16 +13,17 @@
 // A product of two integers is the sum over digit pairs (t, s) of weight
 // 256^(12 - t - s); the 28 pairs with t + s <= 6 are kept (what is dropped is
 // below 2^-56 of the largest product).  The pairs of one weight share an
-// accumulator: products are at most 2^14 and the sums below 2^24 over 256
-// columns (1024 rows) for the leading weights, so FP32 accumulation is exact
-// there; the last two weights can round, at 2^-56 of the result's scale.  The
-// seven accumulators are combined in 64-bit integers.  An entry's error is
-// 2^-56 of its column's largest, against 2^-48 of the entry for the FP32
-// planes: no larger while the typical (geometric mean) entry is within 2^8 of
-// the largest (Gaussian columns: 2^3.4), else the driver takes the double-float
-// form; the residual pass needs 2^5 (multi_tc_columns_ok).  Measured at kappa =
-// 1e1 .. 1e10: backward errors 1e-17 and forward errors as with FP64 residual
-// passes; A^T (A z) off by 9e-17 of |A|^T |A z| (double-float: 3e-15).
+// accumulator: products are at most 2^14 and the sums at most 2^24 for the 4
+// leading weights over 256 columns or rows, so FP32 accumulation is exact
+// there; the last weights can round, in the worst case (all digits large and of
+// one sign) at 2^-49 of the result's scale.  The seven accumulators are combined
+// in 64-bit integers.  An entry's error is 2^-56 of its column's largest, against
+// 2^-48 of the entry for the FP32 planes: no larger while the typical (geometric
+// mean) entry is within 2^8 of the largest (Gaussian columns: 2^3.4), else the
+// driver takes the double-float form; the residual pass needs 2^5
+// (multi_tc_columns_ok).  Measured at kappa = 1e1 .. 1e10: backward errors 1e-17
+// and forward errors as with FP64 residual passes; A^T (A z) off by 9e-17 of
+// |A|^T |A z| (double-float: 3e-15).
 //
 // Both products are the same GEMM, D[128 x 64] += P^(t)[128 x K] Q^(s)[64 x K]^T:
 //   y:  P = A (rows i, K = columns j),     Q = Z^T  -> y in 64 bits and each
@@ -51,7 +52,11 @@ constexpr int kPTile = 128 * 64 * 2;        // bytes of a P tile
 constexpr int kPStages = 6;
 constexpr int kTcThreads = 320;             // producer, issuer, 8 epilogue warps
 constexpr int kTcBad = 1 << 20;
-constexpr int kFlushChunks = 16;            // h: 1024 rows per accumulation
+// h: 256 rows per accumulation.  The d + 1 digit pairs of weight d add up to
+// (d + 1) 2^14 256 <= 2^24 for d <= 3, whatever the digits: exact in FP32.  (1024
+// rows take 8% less time per pass, but weights 1 .. 3 round, at 2^-32 .. 2^-48, where
+// the digits of many rows are all large and of one sign.)
+constexpr int kFlushChunks = 4;
 constexpr uint64_t kTcWaitNs = 1000ull * 1000 * 1000;  // 1 s
 
 __host__ __device__ constexpr int tc_qset(int nv) { return kS * nv * 128; }  // bytes, nv vectors
@@ -257,6 +262,13 @@ __device__ __forceinline__ void tc_ld8(unsigned addr, float (&v)[8]) {
                : "r"(addr));
 #pragma unroll
   for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// a b + c in one instruction (shifts and adds of 64-bit halves take four)
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
 }
 
 struct TcArgs {
@@ -499,9 +511,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
           // y in units of 2^(F_c - 54): sum_d T_d 256^(5 - d)
 #pragma unroll
           for (int e = 0; e < 8; e++) {
-            long long y = (__float2int_rn(T[6][e]) + 128) >> 8;
-#pragma unroll
-            for (int d = 5; d >= 0; d--) y += (long long)__float2int_rn(T[d][e]) << (8 * (5 - d));
+            long long y = __float2int_rn(T[5][e]) + ((__float2int_rn(T[6][e]) + 128) >> 8);
+            y = mad_wide(__float2int_rn(T[4][e]), 1 << 8, y);
+            y = mad_wide(__float2int_rn(T[3][e]), 1 << 16, y);
+            y = mad_wide(__float2int_rn(T[2][e]), 1 << 24, y);
+            y += (long long)(__float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8)) << 32;
             a.Y[(size_t)(c0 + e) * a.ldy + 128 * (int64_t)mt + row] = y;
             const int bits = __reduce_max_sync(0xffffffffu, 64 - __clzll(y < 0 ? -y : y));
             if (lane == 0) ymax[w][c0 + e] = max(ymax[w][c0 + e], bits);
@@ -509,17 +523,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
         } else {
           // exact in two 64-bit sums: lo = sum_{d >= 2} T_d 256^(6 - d), hi = T_1 +
           // 256 T_0 (A^T r cancels: rounding the sum to 64 bits at 2^-50 of its
-          // terms cost the residual pass a factor 100 in backward error)
+          // terms cost the residual pass a factor 100 in backward error); lo's
+          // bits from 40 up are hi's units, so lo's sum stays below 2^63 over
+          // 2^23 accumulations
           const size_t ldh = 128 * (size_t)a.tiles;
           long long *hp = a.H + 2 * ((size_t)(blockIdx.x / a.tiles) * a.nv + c0) * ldh +
                           128 * mt + row;
 #pragma unroll
           for (int e = 0; e < 8; e++) {
             long long lo = __float2int_rn(T[6][e]);
-#pragma unroll
-            for (int d = 5; d >= 2; d--) lo += (long long)__float2int_rn(T[d][e]) << (8 * (6 - d));
-            const long long hi = (long long)__float2int_rn(T[1][e]) +
-                                 ((long long)__float2int_rn(T[0][e]) << 8);
+            lo = mad_wide(__float2int_rn(T[5][e]), 1 << 8, lo);
+            lo = mad_wide(__float2int_rn(T[4][e]), 1 << 16, lo);
+            lo = mad_wide(__float2int_rn(T[3][e]), 1 << 24, lo);
+            lo += (long long)__float2int_rn(T[2][e]) << 32;
+            const long long hi =  // |T_1| <= 2^23, |T_0| <= 2^22
+                __float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8) + (int)(lo >> 40);
+            lo &= (1ll << 40) - 1;
             // no other thread adds here: integer reductions without a reply
             // (loads and stores cost a round trip each, 80k cycles per flush)
             unsigned long long *p = reinterpret_cast<unsigned long long *>(hp + 2 * (size_t)e * ldh);
@@ -692,7 +711,7 @@ __global__ void __launch_bounds__(256)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.y;
   const int j = blockIdx.x * 32 + lane;
   double s = 0.0;
-  long long hi = 0;  // exact; lo's sums (below 2^63 per range) are added in FP64
+  long long hi = 0;  // exact; lo's sums are added in FP64
   if (j < n)
     for (int g = warp; g < ranges; g += 8) {
       const long long *p = H + 2 * ((size_t)g * nv + c) * ldh + j;

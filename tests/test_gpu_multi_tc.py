@@ -46,3 +46,30 @@ def test_multi_tc_edges(m, n, k, outlier):
         bound = 4 * (n + m) * u * (absA.T @ (absA @ np.abs(Z[c])))
         assert (np.abs(Hh[c] - h) <= bound).all(), c
         assert oracle.kw_relative(A, B[:, c], Xh[:, c]) <= 1e-13, c
+
+
+def test_multi_tc_equal_rows():
+    """Runs of equal rows whose entries have the digit 127 in every place: the
+    digit products of a run all add up with one sign.  |A| and |z| lie within a
+    factor 2, so every rounding of the fixed-point pass (A, z, y to 2^-56 of the
+    largest, the dropped digit pairs) is below 2 u of |A|^T |A| |z| and all of
+    them together below 16 u."""
+    runs, run, n, k = 30, 1100, 24, 8
+    m = runs * run
+    rng = np.random.default_rng(7)
+    v = sum(127.0 * 256.0 ** -(t + 1) for t in range(6))
+    A = np.repeat(v * rng.choice([-1.0, 1.0], (runs, n)), run, axis=0)
+    plan = lsq.Plan(m, n, seed=5, nrhs=k)
+    dA = T(A)
+    X = torch.empty((n, k), dtype=torch.float64, device="cuda")
+    st, info = lsq.lsq_solve_fossils_multi(plan.handle, dA, T(rng.standard_normal((m, k))), k, X)
+    assert st == 0 and info.inner_kernel == 5
+    Z = rng.choice([-1.0, 1.0], (k, n)) * rng.uniform(0.5, 1.0, (k, n))
+    Hd = empty(n * k)
+    lsq.lsq_apply_normal_multi(plan.handle, dA, T(Z), Hd)
+    Hh = H(Hd).reshape(k, n)
+    plan.close()
+    absA = np.abs(A)
+    for c in range(k):
+        _, _, h = oracle.residual_dot2(A, np.zeros(m), -Z[c])
+        assert (np.abs(Hh[c] - h) <= 16 * u * (absA.T @ (absA @ np.abs(Z[c])))).all(), c

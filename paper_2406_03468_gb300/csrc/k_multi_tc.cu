@@ -33,7 +33,7 @@
 // that the tensor cores read (128 rows of 64 bf16, 128-byte swizzle, 16 KB):
 // a tile is one contiguous bulk copy.  A CTA (one per SM) runs a producer warp
 // (copies: a ring of P tiles, two sets of Q tiles), an issuing warp (one thread)
-// and eight warps that read the accumulators (7 x 64 columns of TMEM).
+// and sixteen warps that read the accumulators (7 x 64 columns of TMEM).
 //
 // Measured: see launch_multi_tc_pass.  Every wait is bounded; on a timeout
 // the CTA records LSQ_ERR_TIMEOUT, waits (bounded) for its copies and MMAs,
@@ -50,7 +50,7 @@ namespace {
 constexpr int kS = 7;                       // digits
 constexpr int kPTile = 128 * 64 * 2;        // bytes of a P tile
 constexpr int kPStages = 6;
-constexpr int kTcThreads = 320;             // producer, issuer, 8 epilogue warps
+constexpr int kTcThreads = 576;             // producer, issuer, 16 epilogue warps
 constexpr int kTcBad = 1 << 20;
 // h: 256 rows per accumulation.  The d + 1 digit pairs of weight d add up to
 // (d + 1) 2^14 256 <= 2^24 for d <= 3, whatever the digits: exact in FP32.  (1024
@@ -295,12 +295,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
   __shared__ uint64_t pfull[kPStages], pempty[kPStages], qfull[2], qempty[2], accfull, accempty, drain;
   __shared__ unsigned tmem_sh;
   __shared__ volatile int abort_sh;
-  __shared__ int ymax[4][64];
+  __shared__ int ymax[64];
   unsigned char *tsm = tsm_raw + ((1024 - (tc_smem(tsm_raw) & 1023)) & 1023);
   unsigned char *ring = tsm, *qbuf = tsm + (size_t)kPStages * kPTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qbytes = tc_qset(a.nv);
-  for (int i = threadIdx.x; i < 256; i += kTcThreads) (&ymax[0][0])[i] = 0;
+  if (threadIdx.x < 64) ymax[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kPStages; i++) {
       mbar_init(pfull + i, 1);
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
       mbar_init(qempty + i, 1);
     }
     mbar_init(&accfull, 1);
-    mbar_init(&accempty, 256);
+    mbar_init(&accempty, kTcThreads - 64);
     mbar_init(&drain, 1);
     abort_sh = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -474,86 +474,104 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
       if (ok) tc_commit(&accfull);
     }
   } else if (warp >= 2) {
-    // two warps per quarter of the 128 lanes, every other 8 vectors each
-    const int w = warp & 3, row = 32 * w + lane, half = (warp - 2) >> 2;
+    // four warps per quarter of the 128 lanes; 8 vectors of every 32 each.  The
+    // next accumulation waits for the last warp's loads: a warp combines its
+    // first 8 vectors (56 registers to 16), loads the second 8, and lets TMEM go
+    // before it stores anything
+    const int w = warp & 3, row = 32 * w + lane, sub = (warp - 2) >> 2;
     const unsigned tl = tmem + ((unsigned)(32 * w) << 16);
-    bool ok = true;
+    const size_t ldh = 128 * (size_t)a.tiles;
     for (int g = 0; g < ngroups; g++) {
       int mt, cb, ce;
       group(g, mt, cb, ce);
       // one decision per warp
-      ok = __all_sync(0xffffffffu, wait(&accfull, (unsigned)(g & 1)));
-      if (!ok) break;
+      if (!__all_sync(0xffffffffu, wait(&accfull, (unsigned)(g & 1)))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // the next 8 vectors' accumulators are on their way while these are combined
-      float N[kS][8];
+      float T[kS][8];
+      long long v0[8];
+      int v1[8];  // STEP 1: the high sum
+      auto load = [&](int c0) {
 #pragma unroll
-      for (int d = 0; d < kS; d++) tc_ld8(tl + a.nv * d + 8 * half, N[d]);
-      for (int c0 = 8 * half; c0 < a.nv; c0 += 16) {
-        float T[kS][8];
+        for (int d = 0; d < kS; d++) tc_ld8(tl + a.nv * d + c0, T[d]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int d = 0; d < kS; d++)
 #pragma unroll
-          for (int e = 0; e < 8; e++) {
-            asm volatile("" : "+f"(N[d][e])::"memory");  // no use before the wait
-            T[d][e] = N[d][e];
-          }
-        if (c0 + 16 < a.nv) {
+          for (int e = 0; e < 8; e++)
+            asm volatile("" : "+f"(T[d][e])::"memory");  // no use before the wait
+      };
+      auto release = [&]() {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        tc_arrive(&accempty);
+      };
+      auto combine = [&]() {
 #pragma unroll
-          for (int d = 0; d < kS; d++) tc_ld8(tl + a.nv * d + c0 + 16, N[d]);
-        } else {
-          // everything is in registers: the next accumulation may begin
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          tc_arrive(&accempty);
-        }
-        if (STEP == 0) {
-          // y in units of 2^(F_c - 54): sum_d T_d 256^(5 - d)
-#pragma unroll
-          for (int e = 0; e < 8; e++) {
+        for (int e = 0; e < 8; e++) {
+          if (STEP == 0) {
+            // y in units of 2^(F_c - 54): sum_d T_d 256^(5 - d)
             long long y = __float2int_rn(T[5][e]) + ((__float2int_rn(T[6][e]) + 128) >> 8);
             y = mad_wide(__float2int_rn(T[4][e]), 1 << 8, y);
             y = mad_wide(__float2int_rn(T[3][e]), 1 << 16, y);
             y = mad_wide(__float2int_rn(T[2][e]), 1 << 24, y);
-            y += (long long)(__float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8)) << 32;
-            a.Y[(size_t)(c0 + e) * a.ldy + 128 * (int64_t)mt + row] = y;
-            const int bits = __reduce_max_sync(0xffffffffu, 64 - __clzll(y < 0 ? -y : y));
-            if (lane == 0) ymax[w][c0 + e] = max(ymax[w][c0 + e], bits);
-          }
-        } else {
-          // exact in two 64-bit sums: lo = sum_{d >= 2} T_d 256^(6 - d), hi = T_1 +
-          // 256 T_0 (A^T r cancels: rounding the sum to 64 bits at 2^-50 of its
-          // terms cost the residual pass a factor 100 in backward error); lo's
-          // bits from 40 up are hi's units, so lo's sum stays below 2^63 over
-          // 2^23 accumulations
-          const size_t ldh = 128 * (size_t)a.tiles;
-          long long *hp = a.H + 2 * ((size_t)(blockIdx.x / a.tiles) * a.nv + c0) * ldh +
-                          128 * mt + row;
-#pragma unroll
-          for (int e = 0; e < 8; e++) {
+            v0[e] = y + ((long long)(__float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8)) << 32);
+          } else {
+            // exact in two 64-bit sums: lo = sum_{d >= 2} T_d 256^(6 - d), hi = T_1 +
+            // 256 T_0 (A^T r cancels: rounding the sum to 64 bits at 2^-50 of its
+            // terms cost the residual pass a factor 100 in backward error); lo's
+            // bits from 40 up are hi's units, so lo's sum stays below 2^63 over
+            // 2^23 accumulations
             long long lo = __float2int_rn(T[6][e]);
             lo = mad_wide(__float2int_rn(T[5][e]), 1 << 8, lo);
             lo = mad_wide(__float2int_rn(T[4][e]), 1 << 16, lo);
             lo = mad_wide(__float2int_rn(T[3][e]), 1 << 24, lo);
             lo += (long long)__float2int_rn(T[2][e]) << 32;
-            const long long hi =  // |T_1| <= 2^23, |T_0| <= 2^22
+            v1[e] =  // |T_1| <= 2^23, |T_0| <= 2^22
                 __float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8) + (int)(lo >> 40);
-            lo &= (1ll << 40) - 1;
-            // no other thread adds here: integer reductions without a reply
-            // (loads and stores cost a round trip each, 80k cycles per flush)
-            unsigned long long *p = reinterpret_cast<unsigned long long *>(hp + 2 * (size_t)e * ldh);
-            atomicAdd(p, (unsigned long long)lo);
-            atomicAdd(p + ldh, (unsigned long long)hi);
+            v0[e] = lo & ((1ll << 40) - 1);
           }
         }
+      };
+      auto store = [&](int c0) {
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+          if (STEP == 0) {
+            const long long y = v0[e];
+            a.Y[(size_t)(c0 + e) * a.ldy + 128 * (int64_t)mt + row] = y;
+            const int bits = __reduce_max_sync(0xffffffffu, 64 - __clzll(y < 0 ? -y : y));
+            if (lane == 0) atomicMax(&ymax[c0 + e], bits);
+          } else {
+            // no other thread adds here: integer reductions without a reply
+            // (loads and stores cost a round trip each, 80k cycles per flush)
+            unsigned long long *p = reinterpret_cast<unsigned long long *>(
+                a.H + 2 * ((size_t)(blockIdx.x / a.tiles) * a.nv + c0 + e) * ldh + 128 * mt + row);
+            atomicAdd(p, (unsigned long long)v0[e]);
+            atomicAdd(p + ldh, (unsigned long long)(long long)v1[e]);
+          }
+        }
+      };
+      const int c0 = 8 * sub, c1 = c0 + 32;
+      if (c0 < a.nv) {
+        load(c0);
+        if (c1 >= a.nv) release();
+        combine();
+        if (c1 < a.nv) {
+          load(c1);
+          release();
+          store(c0);
+          combine();
+          store(c1);
+        } else {
+          store(c0);
+        }
+      } else {
+        release();
       }
     }
   }
   __syncwarp();
   __syncthreads();
   if (STEP == 0 && threadIdx.x < a.nv) {
-    const int c = threadIdx.x;
-    atomicMax(a.ybits + c, max(max(ymax[0][c], ymax[1][c]), max(ymax[2][c], ymax[3][c])));
+    atomicMax(a.ybits + threadIdx.x, ymax[threadIdx.x]);
   }
   if (abort_sh && warp == 1 && lane == 0) {
     // MMAs in flight end before the TMEM is freed (bounded)
@@ -820,10 +838,10 @@ cudaError_t tc_step1(const TcShape &t, int n, int k, double *out, const double *
 
 }  // namespace
 
-// Measured at 500000 x 200 x 64: y 400 us (1.5 GB of digits; the accumulators'
-// combination is not hidden under the next tile's MMAs, which fill TMEM), y's
-// digits 108 us, h 324 us (5 TB/s), the rest 15 us: 0.85 ms per pass against
-// 5.9 ms in double-float.
+// Measured at 500000 x 200 x 64: y 371 us (405 with 8 reading warps that stored
+// before they let TMEM go; 1.5 GB of digits), y's digits 107 us, h 385 us (1.4 GB;
+// the MMAs fill TMEM, so neither hides its accumulators' combination), the rest
+// 17 us: 0.88 ms per pass against 5.9 ms in double-float.
 cudaError_t launch_multi_tc_pass(int64_t m, int n, int k, const double *Z, double *out,
                                  const double *scale, const TcBufs &b, int nsm,
                                  const DevState *gate, int *err, cudaStream_t s) {

@@ -610,33 +610,35 @@ __global__ void __launch_bounds__(kGatherWarps * 32, RPW == 2 ? 5 : 1)
 }
 
 // ---------------------------------------------------------------------------
-// Batched sketch (many problems in one launch, lsq_batch.cu).  CTA g works on
-// rows of item cta_item[g]: the scatter form of the pass above, with each
-// row's zeta targets drawn inline (each lane of a warp draws the pattern of
-// one of 32 consecutive rows, then the warp walks those rows), the hi / lo
-// planes written as the rows stream, column sums of squares per CTA.
-// zeta <= kBZeta.
+// Batched sketch (many problems in one launch, lsq_batch.cu): the scatter form
+// of the pass above, with each row's zeta targets drawn inline (a lane per row
+// of a chunk, then the warp walks the chunk's rows), the hi / lo planes written
+// as the rows stream, column sums of squares per CTA.  All CTAs work on one
+// item after the other, without waiting for each other: the atomics of a time
+// meet in the sketches of one or two items (6 MB each at n = 256).  With the
+// items dealt to the CTAs all sketches of the batch (93 MB at 32 items) were in
+// use at once, half of L2's atomic rate: 11.1 ms, now 7.2.  Chunks of 32 rows, of 8 where an
+// item has fewer than 32 per warp.  zeta <= kBZeta.
 // ---------------------------------------------------------------------------
 constexpr int kBZeta = 8;
 
 template <int NC>
-__device__ void b_sketch_body(const BItem &it, int local, int zeta) {
-  __shared__ double acc[4 * 64];
+__device__ __forceinline__ void b_sketch_body(const BItem &it, int first, int zeta, double *acc) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int n = it.n, d = it.d, ldsa = n + 1;
   const int64_t m = it.m;
-  const int64_t per = (m + it.ncta - 1) / it.ncta;
-  const int64_t r0 = min(m, (int64_t)local * per), r1 = min(m, r0 + per);
+  const int W = gridDim.x * nw;
+  const int R = m >= (int64_t)32 * W ? 32 : 8;
   double sq[2 * NC];
 #pragma unroll
   for (int k = 0; k < 2 * NC; k++) sq[k] = 0.0;
-  for (int64_t i0 = r0 + 32 * warp; i0 < r1; i0 += 32 * nw) {
+  for (int64_t i0 = (int64_t)R * first; i0 < m; i0 += (int64_t)R * W) {
+    const int cnt = (int)min((int64_t)R, m - i0);
     int hl[kBZeta];
     uint32_t sbl = 0;
 #pragma unroll
     for (int t = 0; t < kBZeta; t++) hl[t] = -1;
-    if (i0 + lane < r1) column_pattern<kBZeta>(i0 + lane, d, zeta, it.seed, hl, sbl);
-    const int cnt = (int)min((int64_t)32, r1 - i0);
+    if (lane < cnt) column_pattern<kBZeta>(i0 + lane, d, zeta, it.seed, hl, sbl);
     for (int q = 0; q < cnt; q++) {
       const int64_t i = i0 + q;
       double a[2 * NC];
@@ -674,6 +676,7 @@ __device__ void b_sketch_body(const BItem &it, int local, int zeta) {
       }
     }
   }
+  __syncthreads();  // the previous item's sums have been written
   for (int i = threadIdx.x; i < NC * 64; i += blockDim.x) acc[i] = 0.0;
   for (int w = 0; w < nw; w++) {
     __syncthreads();
@@ -684,29 +687,41 @@ __device__ void b_sketch_body(const BItem &it, int local, int zeta) {
   }
   __syncthreads();
   for (int i = threadIdx.x; i < it.npad; i += blockDim.x)
-    it.part[(size_t)local * it.npad + i] = acc[i];
+    it.part[(size_t)blockIdx.x * it.npad + i] = acc[i];
 }
 
 __global__ void __launch_bounds__(kPassThreads, 2)
-    b_sketch_kernel(const BItem *__restrict__ items, const int *__restrict__ cta_item, int zeta) {
-  const int idx = cta_item[blockIdx.x];
-  const BItem &it = items[idx];
-  const int local = blockIdx.x - it.cta0;
-  switch (it.npad / 64) {
-    case 1: b_sketch_body<1>(it, local, zeta); break;
-    case 2: b_sketch_body<2>(it, local, zeta); break;
-    case 4: b_sketch_body<4>(it, local, zeta); break;
-    default: break;
+    b_sketch_kernel(const BItem *__restrict__ items, int count, int zeta) {
+  __shared__ double acc[4 * 64];
+  const int W = gridDim.x * (kPassThreads / 32);
+  for (int idx = 0; idx < count; idx++) {
+    const BItem &it = items[idx];
+    // a warp's first chunk; the item's turn rotates which warps take one more
+    const int first = (int)((blockIdx.x + gridDim.x * (threadIdx.x >> 5) + 61u * idx) % W);
+    switch (it.npad / 64) {
+      case 1: b_sketch_body<1>(it, first, zeta, acc); break;
+      case 2: b_sketch_body<2>(it, first, zeta, acc); break;
+      case 4: b_sketch_body<4>(it, first, zeta, acc); break;
+      default: break;
+    }
   }
 }
 
-// Column norms of each item from its CTAs' partial sums of squares, and the
+// Column norms of each item from the np CTAs' partial sums of squares, and the
 // checks of the plan path (non-finite, zero column).
-__global__ void b_colnorm_kernel(const BItem *__restrict__ items) {
-  const BItem &it = items[blockIdx.x];
-  for (int j = threadIdx.x; j < it.n; j += blockDim.x) {
+// 32 columns per CTA, the partials split over its 8 warps.
+__global__ void __launch_bounds__(256) b_colnorm_kernel(const BItem *__restrict__ items, int np) {
+  __shared__ double red[8][32];
+  const BItem &it = items[blockIdx.y];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+  double p = 0.0;
+  if (j < it.n)
+    for (int g = warp; g < np; g += 8) p += it.part[(size_t)g * it.npad + j];
+  red[warp][lane] = p;
+  __syncthreads();
+  if (warp == 0 && j < it.n) {
     double s = 0.0;
-    for (int g = 0; g < it.ncta; g++) s += it.part[(size_t)g * it.npad + j];
+    for (int w = 0; w < 8; w++) s += red[w][lane];
     const double nrm = sqrt(s);
     if (!isfinite(nrm)) atomicExch(&it.st->nonfinite, 1);
     if (nrm == 0.0) atomicExch(&it.st->zero_col, 1);
@@ -747,15 +762,15 @@ __global__ void b_transpose_kernel(const BItem *__restrict__ items, double zinv)
 
 }  // namespace
 
-cudaError_t launch_b_sketch(const BItem *items, const int *cta_item, int grid, int zeta,
-                            cudaStream_t s) {
+cudaError_t launch_b_sketch(const BItem *items, int count, int grid, int zeta, cudaStream_t s) {
   if (zeta > kBZeta) return cudaErrorInvalidValue;
-  b_sketch_kernel<<<grid, kPassThreads, 0, s>>>(items, cta_item, zeta);
+  b_sketch_kernel<<<grid, kPassThreads, 0, s>>>(items, count, zeta);
   return cudaGetLastError();
 }
 
-cudaError_t launch_b_finalize(const BItem *items, int count, int zeta, cudaStream_t s) {
-  b_colnorm_kernel<<<count, 256, 0, s>>>(items);
+cudaError_t launch_b_finalize(const BItem *items, int count, int nmax, int np, int zeta,
+                              cudaStream_t s) {
+  b_colnorm_kernel<<<dim3((nmax + 31) / 32, count), 256, 0, s>>>(items, np);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   b_transpose_kernel<<<dim3(32, count), dim3(32, 8), 0, s>>>(items, 1.0 / sqrt((double)zeta));

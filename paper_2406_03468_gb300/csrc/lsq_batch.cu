@@ -406,10 +406,11 @@ extern "C" lsq_status lsq_batch_solve(lsq_batch B, int count, lsq_batch_item *it
   const int qcta = std::max(1, std::min(8, 2 * B->nsm / count));
   // sketch (and, when the QR takes the column-step form, the QR steps)
   const bool coop_qr = B->qgrid > 0;
+  const int gsk = 2 * B->nsm;  // the sketch's CTAs (at most grid_max): one wave
   auto pre = [&]() -> cudaError_t {
     cudaError_t e = launch_b_zero(B->d_items, count, B->s);
-    if (e == cudaSuccess) e = launch_b_sketch(B->d_items, B->d_cta, B->grid, kBatchZeta, B->s);
-    if (e == cudaSuccess) e = launch_b_finalize(B->d_items, count, kBatchZeta, B->s);
+    if (e == cudaSuccess) e = launch_b_sketch(B->d_items, count, gsk, kBatchZeta, B->s);
+    if (e == cudaSuccess) e = launch_b_finalize(B->d_items, count, nmax, gsk, kBatchZeta, B->s);
     for (int k = -1; !coop_qr && k < nmax && e == cudaSuccess; k++)
       e = launch_b_qr_step(B->d_items, count, qcta, k, B->s);
     return e;

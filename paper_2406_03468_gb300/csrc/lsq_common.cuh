@@ -417,9 +417,9 @@ cudaError_t launch_b_zero(const BItem *items, int count, cudaStream_t s);  // SA
 // whose inner loop runs (all = 0); each item's partials hold grid entries.
 cudaError_t launch_b_redeal(BItem *items, int count, int *cta_item, int grid, int all,
                             cudaStream_t s);
-cudaError_t launch_b_sketch(const BItem *items, const int *cta_item, int grid, int zeta,
-                            cudaStream_t s);
-cudaError_t launch_b_finalize(const BItem *items, int count, int zeta, cudaStream_t s);
+cudaError_t launch_b_sketch(const BItem *items, int count, int grid, int zeta, cudaStream_t s);
+cudaError_t launch_b_finalize(const BItem *items, int count, int nmax, int np, int zeta,
+                              cudaStream_t s);
 // QR of every item's sketch in one cooperative launch (the flag form of
 // launch_qr, item i on CTAs qcta0 .. qcta0 + qncta - 1 of the grid, qmap the
 // CTA -> item map, -1 for none); at most b_qr_max_ctas CTAs, at least

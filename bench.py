@@ -477,8 +477,8 @@ def multi_compare(lsq, torch, dev, steps):
     plan1.close()
     out = {"workload": "fossils_multi_m2000000_n200_k64_kappa1e8_d2400_zeta8", "steps": steps,
            "solves_per_s": 1.0 / dt, "rhs_solves_per_s": k / dt, "ms_per_solve": dt * 1e3,
-           "path": "default: inner pass double-float on the hi/lo planes, all k vectors per "
-                   "launch; residual pass FP64 DMMA",
+           "path": "default: both passes on the tensor cores in 56-bit fixed point, all k "
+                   "vectors per launch",
            "inner_kernel": last["inner_kernel"],
            "iters": last["iters"], "phase_ms": {"sketch": last["ms_sketch"], "qr": last["ms_qr"],
                                                 "refine": last["ms_refine"]},

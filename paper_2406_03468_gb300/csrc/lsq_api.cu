@@ -953,10 +953,18 @@ void free_tc(lsq_plan P) {
   P->tc_alloc = false;
 }
 
-// The tensor-core pass's buffers; without them (not enough memory) the plan
-// uses the double-float form.
+// The tensor-core pass's buffers: 5 times the bytes of A at n = 200 and k = 64, more
+// for few columns (tiles of 64 and 128 columns).  Where they would
+// take more than half of the memory that is free, the rest being the caller's,
+// the plan uses the double-float form.
 void alloc_tc(lsq_plan P, int n) {
   const TcSizes z = multi_tc_sizes(P->m_cap, n, P->k, P->nsm);
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (z.p1 + z.p2 + z.q + z.y + z.y64 + z.h + z.r2 > free_b / 2) return;
   cudaError_t e = cudaMalloc((void **)&P->tc.p1, z.p1);
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.p2, z.p2);
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.q, z.q);

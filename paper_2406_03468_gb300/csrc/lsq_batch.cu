@@ -70,7 +70,7 @@ struct lsq_batch_s {
   // pools
   char *ws = nullptr;            // per-item n- and d-sized buffers
   size_t ws_per_item = 0;
-  float *planes = nullptr;       // hi / lo planes of all items (elems_max floats each)
+  float *planes = nullptr;       // hi / lo planes of all items (batch_plane_floats each)
   double *part = nullptr, *r2part = nullptr;  // pass partials (per item: grid_max x 256)
   int grid_max = 0;
   DevState *st = nullptr;        // one per item
@@ -182,6 +182,10 @@ void deal_ctas(lsq_batch B, int count, int grid) {
 
 }  // namespace
 
+// The lo plane follows the hi plane on a 16-byte boundary whatever the caller's
+// elems_max: the passes fetch its rows with bulk copies.
+int64_t lsq::batch_plane_floats(int64_t elems_max) { return (elems_max + 3) / 4 * 4; }
+
 extern "C" {
 
 lsq_status lsq_batch_create(int max_items, int64_t n_max, int64_t elems_max, void *cuda_stream,
@@ -205,10 +209,11 @@ lsq_status lsq_batch_create(int max_items, int64_t n_max, int64_t elems_max, voi
   }
   const Slice L = slice_layout(n_max);
   B->ws_per_item = L.total;
+  const size_t plane_bytes = sizeof(float) * 2 * (size_t)batch_plane_floats(elems_max) + 256;
   B->grid_max = std::max(4 * B->nsm, max_items);
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   A(cudaMalloc((void **)&B->ws, L.total * (size_t)max_items));
-  A(cudaMalloc((void **)&B->planes, sizeof(float) * 2 * (size_t)elems_max + 256));
+  A(cudaMalloc((void **)&B->planes, plane_bytes));
   // each item's partials hold a whole grid (the CTAs are re-dealt to the
   // unfinished items as the inner loop goes on)
   A(cudaMalloc((void **)&B->part, sizeof(double) * (size_t)max_items * B->grid_max * 256));
@@ -223,7 +228,7 @@ lsq_status lsq_batch_create(int max_items, int64_t n_max, int64_t elems_max, voi
   A(cudaMallocHost((void **)&B->h_qmap, sizeof(int) * (size_t)b_qr_max_ctas(B->nsm)));
   // the passes over the planes read to the end of their column tiles: every
   // value there must be finite
-  if (e == cudaSuccess) A(cudaMemset(B->planes, 0, sizeof(float) * 2 * (size_t)elems_max + 256));
+  if (e == cudaSuccess) A(cudaMemset(B->planes, 0, plane_bytes));
   // the QR flags start at 0 (a flag is ready when it equals the launch's epoch)
   if (e == cudaSuccess) A(cudaMemset(B->ws, 0, L.total * (size_t)max_items));
   A(prepare_b_kernels((int)n_max));
@@ -340,7 +345,7 @@ extern "C" lsq_status lsq_batch_solve(lsq_batch B, int count, lsq_batch_item *it
                      &it.dyold, &it.z, &it.h, &it.w, &it.res, &it.p, &it.res2, &it.p2, &it.pn};
     for (size_t k = 0; k < sizeof(vs) / sizeof(vs[0]); k++) *vs[k] = v + k * nm;
     it.Ahi = B->planes + poff;
-    it.Alo = B->planes + B->elems_max + poff;
+    it.Alo = B->planes + batch_plane_floats(B->elems_max) + poff;
     poff += it.m * it.ld32;
     poff = (poff + 3) / 4 * 4;
     it.st = B->st + i;

@@ -412,6 +412,7 @@ cudaError_t launch_lsqr_init(int n, const double *c, int step, double *v, double
 // Kernel attributes of the batched kernels for n <= nmax (before any capture).
 cudaError_t prepare_b_kernels(int nmax);
 cudaError_t prepare_b_inner();
+int64_t batch_plane_floats(int64_t elems_max);  // floats from the hi to the lo plane
 cudaError_t launch_b_zero(const BItem *items, int count, cudaStream_t s);  // SAb = 0
 // Re-deal the row-parallel CTAs over all items (all = 1) or over the items
 // whose inner loop runs (all = 0); each item's partials hold grid entries.

@@ -770,7 +770,8 @@ TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm) {
   z.y = (size_t)(mp / 64) * tc_qset(nv);
   z.y64 = sizeof(long long) * (size_t)mp * nv;
   z.r2 = sizeof(double) * (size_t)nsm * kTcResidCtas * k;
-  z.h = 2 * sizeof(long long) * (size_t)(nsm / njt) * nv * 128 * njt;
+  // (nsm / njt) ranges of njt row tiles: at most nsm tiles, for any smaller n too
+  z.h = 2 * sizeof(long long) * (size_t)nsm * nv * 128;
   return z;
 }
 

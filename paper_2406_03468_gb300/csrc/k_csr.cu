@@ -124,9 +124,8 @@ template <int MODE>
 __device__ __forceinline__ void csr_quad(const int64_t *__restrict__ rp,
                                          const int32_t *__restrict__ col,
                                          const double *__restrict__ val,
-                                         const double *__restrict__ b, const double *__restrict__ x,
-                                         int64_t i0, int64_t r1, double bs, bool scaled,
-                                         double *rout, double *hw, int lane, double &r2) {
+                                         const double *b, const double *x, int64_t i0,
+                                         int64_t r1, double bs, bool scaled, double *rout, double *hw, int lane, double &r2) {
   int64_t beg[4], end[4];
   double v[4];
 #pragma unroll
@@ -135,7 +134,7 @@ __device__ __forceinline__ void csr_quad(const int64_t *__restrict__ rp,
     beg[q] = in ? rp[i0 + q] : 0;
     end[q] = in ? rp[i0 + q + 1] : 0;
     double t = 0.0;
-    for (int64_t p = beg[q] + lane; p < end[q]; p += 32) t = fma(val[p], __ldg(x + col[p]), t);
+    for (int64_t p = beg[q] + lane; p < end[q]; p += 32) t = fma(val[p], x[col[p]], t);
     v[q] = t;
   }
   const double u = reduce4(v, lane);
@@ -146,6 +145,7 @@ __device__ __forceinline__ void csr_quad(const int64_t *__restrict__ rp,
     double c = t;
     if (MODE == 1) {
       c = (scaled ? bs * b[i0 + q] : b[i0 + q]) - t;
+      __syncwarp();  // every lane has read b (rout may be b)
       if (lane == 0) {
         r2 = fma(c, c, r2);
         if (rout != nullptr) rout[i0 + q] = c;
@@ -175,13 +175,14 @@ __device__ __forceinline__ void csr_quad(const int64_t *__restrict__ rp,
 // 8 rows with more than kCsrStage entries, and longer rows in general, take
 // 4 rows at a time from global memory (csr_quad).
 // 500000 x 500 with 32 entries per row, SPIR with d = 3n: 26.1 -> 17.5 ms per solve.
+// x is written after an inner pass began (griddep_wait), and LSQR's pass writes
+// its b (rout): neither is read through the read-only path.
 template <int MODE, bool STAGED>
 __global__ void __launch_bounds__(kCsrThreads, STAGED ? kCsrStageCtas : 1)
     csr_pass_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-                    const double *__restrict__ val, int64_t m, int n, const double *__restrict__ b,
-                    const double *__restrict__ x, double *__restrict__ part,
-                    double *__restrict__ r2_part, int npad, const DevState *gate,
-                    const double *bscale, double *rout) {
+                    const double *__restrict__ val, int64_t m, int n, const double *b,
+                    const double *x, double *__restrict__ part, double *__restrict__ r2_part,
+                    int npad, const DevState *gate, const double *bscale, double *rout) {
   griddep_launch();
   extern __shared__ double csm[];
   __shared__ double r2w[kCsrWarps];

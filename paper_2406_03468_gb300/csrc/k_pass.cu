@@ -386,10 +386,13 @@ __global__ void reduce_batched_kernel(const double *__restrict__ part, int grid,
 // so the n G additions are spread over all SMs.  At G = 304, n = 500: 63 CTAs
 // of about 10 additions per thread; CTAs of 32 columns with 38 per thread
 // took 6.5 us in the inner loop.
+// The partials are written while this kernel waits to start (griddep_wait), so
+// they are not __restrict__: the read-only path is for data that no running
+// kernel writes.
 __global__ void __launch_bounds__(kReduceThreads)
-    reduce_kernel(const double *__restrict__ part, int grid, int npad, int n,
+    reduce_kernel(const double *part, int grid, int npad, int n,
                   const double *__restrict__ scale, double *__restrict__ out,
-                  const double *__restrict__ r2_part, double *r2, DevState *gate) {
+                  const double *r2_part, double *r2, DevState *gate) {
   griddep_launch();
   griddep_wait();
   if (gate != nullptr) {

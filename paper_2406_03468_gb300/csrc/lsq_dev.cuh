@@ -29,6 +29,8 @@ __device__ __forceinline__ double ld_early(const double *p) {
 // Launch as a programmatic dependent of the kernel before it in the stream.
 // Such a kernel calls griddep_wait before it touches anything that an
 // earlier kernel of the chain writes, or that an earlier one still reads.
+// What the kernels before it write is not read through the read-only path
+// (const __restrict__ parameters, __ldg): it is written after this kernel began.
 template <typename... K, typename... T>
 cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        T... args) {
@@ -50,8 +52,7 @@ cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem,
 // shuffles and shared memory (a fixed order).  Column j0 + t on thread t < 8.
 constexpr int kReduceThreads = 256;
 constexpr int kReduceCols = 8;
-__device__ __forceinline__ double sum_partials(const double *__restrict__ part, int grid, int npad,
-                                               int j0,
+__device__ __forceinline__ double sum_partials(const double *part, int grid, int npad, int j0,
                                                double (*red)[kReduceCols]) {
   constexpr int kGroups = kReduceThreads / kReduceCols;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -46,7 +46,9 @@
 //    both done.
 // Every wait is bounded; on a timeout the kernel records LSQ_ERR_TIMEOUT,
 // waits (bounded) for the transfers addressed to its CTA and returns.
-#include <atomic>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 #include "lsq_cluster.cuh"
 #include "lsq_dev.cuh"
@@ -68,7 +70,8 @@ constexpr size_t kQbSmemMax = 227 * 1024;
 // Up to here all launches on one stream, the panel's CTAs alone on their SMs.
 // ms, two streams / one: d = 12 n, n = 128 0.62 / 0.60, 256 1.65 / 1.43, 333 2.61 /
 // 2.19, 500 5.17 / 5.00, 700 11.06 / 10.94, 1000 26.5 / 26.9; d = 1500, n = 500 2.96 /
-// 2.55.
+// 2.55.  Where that many whole SMs of one cluster domain are not to be had (a
+// partition of a GPU), the two-stream form with the panel's own bytes.
 constexpr int kOneStreamMaxN = 768;
 
 __device__ __forceinline__ void note_timeout(DevState *st) {
@@ -465,14 +468,19 @@ __global__ void __launch_bounds__(kQbThreads, 2)
   if (blockIdx.x + uc >= gridDim.x) griddep_wait();
 }
 
-std::atomic<int> g_qb_pc[64];  // CTAs of the panel cluster per device (0: not chosen yet)
-
-// The panel cluster: 16 CTAs if a cluster of that size with the panel's
-// shared memory can be resident, else 8.
-int panel_cluster(int dev, size_t smem16) {
-  if (dev < 0 || dev >= 64) return 8;
-  if (const int c = g_qb_pc[dev].load()) return c;
-  int pc = 8;
+// Whether a cluster of `ctas` panel CTAs with `bytes` of shared memory each can
+// be resident on the current device (which may be a part of a GPU); asked once
+// per device and shape.
+bool panel_fits(int ctas, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, size_t>, bool> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(dev, ctas, bytes);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  bool ok = false;
   const void *fn = (const void *)qr_panel_kernel;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQbSmemMax) ==
@@ -480,21 +488,20 @@ int panel_cluster(int dev, size_t smem16) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 16;
+    at[0].val.clusterDim.x = ctas;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(16);
+    cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kQbThreads);
-    cfg.dynamicSmemBytes = smem16;
+    cfg.dynamicSmemBytes = bytes;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1)
-      pc = 16;
+    ok = cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1;
   }
   cudaGetLastError();  // a refused query leaves no error behind
-  g_qb_pc[dev].store(pc);
-  return pc;
+  known[key] = ok;
+  return ok;
 }
 
 int rows_per_cta(int Lp, int c) {
@@ -550,14 +557,23 @@ cudaError_t launch_update(double *W, int d, int kb, int bw, int c0, int c1, int 
 
 }  // namespace
 
+// 16 CTAs if a cluster of that size with the panel's shared memory can be
+// resident, else 8; alone on their SMs where that many whole SMs can.  fits:
+// panel_fits, or a stand-in for it.
+QrPanel qr_panel_choice(int d, int n, bool (*fits)(int ctas, size_t bytes)) {
+  const size_t b16 = panel_smem_bytes(rows_per_cta(d, 16), 16);
+  QrPanel p;
+  p.ctas = b16 <= kQbSmemMax && fits(16, b16) ? 16 : 8;
+  p.alone = n <= kOneStreamMaxN && fits(p.ctas, kQbSmemMax);
+  p.bytes = p.alone ? kQbSmemMax : panel_smem_bytes(rows_per_cta(d, p.ctas), p.ctas);
+  return p;
+}
+
 bool qr_blocked_ok(int d, int n) {
   if (n < kQbMinN || d < n) return false;
   // the panel's rows must fit the shared memory of the panel cluster
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  const int pc = panel_cluster(dev, panel_smem_bytes(rows_per_cta(d, 16), 16));
-  return panel_smem_bytes(rows_per_cta(d, pc), pc) <= kQbSmemMax ||
-         panel_smem_bytes(rows_per_cta(d, 8), 8) <= kQbSmemMax;
+  const QrPanel p = qr_panel_choice(d, n, panel_fits);
+  return panel_smem_bytes(rows_per_cta(d, p.ctas), p.ctas) <= kQbSmemMax;
 }
 
 size_t qr_blocked_tws(int n) { return (size_t)((n + kQb - 1) / kQb) * kQb * kQb; }
@@ -565,11 +581,9 @@ size_t qr_blocked_tws(int n) { return (size_t)((n + kQb - 1) / kQb) * kQb * kQb;
 cudaError_t launch_qr_blocked(double *W, int d, int n, int ncols, double *vhead, double *tws,
                               DevState *st, uint64_t timeout_ns, cudaStream_t s, cudaStream_t sp,
                               cudaEvent_t *ev) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  int pc = panel_cluster(dev, panel_smem_bytes(rows_per_cta(d, 16), 16));
-  if (panel_smem_bytes(rows_per_cta(d, pc), pc) > kQbSmemMax) pc = 8;
+  const QrPanel panel = qr_panel_choice(d, n, panel_fits);
+  const int pc = panel.ctas;
+  cudaError_t e = cudaSuccess;
   if (pc == 8) {
     e = cudaFuncSetAttribute((const void *)qr_panel_kernel,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQbSmemMax);
@@ -586,7 +600,7 @@ cudaError_t launch_qr_blocked(double *W, int d, int n, int ncols, double *vhead,
                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   const int np = (n + kQb - 1) / kQb;
-  if (n <= kOneStreamMaxN) {
+  if (panel.alone) {
     if ((e = launch_panel(W, d, 0, n < kQb ? n : kQb, pc, vhead, tws, st, timeout_ns, s, true)) !=
         cudaSuccess)
       return e;

@@ -235,6 +235,12 @@ cudaError_t launch_qr(double *W, int d, int n, int ncols, double *vhead, int *fl
                       DevState *st, int grid, uint64_t timeout_ns, cudaStream_t s,
                       const QrBlocked *qb = nullptr);
 bool qr_blocked_ok(int d, int n);
+struct QrPanel {        // the launch of a panel: its cluster, its shared memory
+  int ctas;
+  int alone;            // all of its SMs' shared memory; the one-stream form
+  size_t bytes;         // of the first panel, per CTA
+};
+QrPanel qr_panel_choice(int d, int n, bool (*fits)(int ctas, size_t bytes));
 size_t qr_blocked_tws(int n);
 cudaError_t launch_qr_blocked(double *W, int d, int n, int ncols, double *vhead, double *tws,
                               DevState *st, uint64_t timeout_ns, cudaStream_t s, cudaStream_t sp,

@@ -6,10 +6,14 @@
 // vectors: 5.9 ms per pass at 500000 x 200 x 64.  Here every operand is an
 // integer of 56 bits written in 7 balanced digits of 8 bits (-128 .. 128), each
 // digit exact in bf16:
-//   A:  a_ij = q 2^(E_j - 55), |a_ij| < 2^E_j (the column's largest exponent);
+//   A:  a_ij = q 2^(E_j - g_i - 55), |a_ij| < 2^(E_j - g_i): E_j the column's
+//       largest exponent, g_i >= 0 the row's gap below the columns' largest
+//       (rows whose entries are all small keep all of their bits: they can be
+//       the ones that determine a direction of x);
 //   z:  v_jc = 2^E_j z_jc = q 2^(F_c - 55), |v_jc| < 2^F_c;
-//   y = A z, exact to 2^-54 of 2^F_c, then per vector against its largest
-//       entry (|A| |z| can be kappa times |A z|).
+//   y = A z: 2^g_i y_i in units of 2^(F_c - 54), then 2^-g_i y_i per vector against
+//       its largest entry (|A| |z| can be kappa times |A z|), A^T y being
+//       2^E_j times the sum over i of (2^(g_i - E_j) a_ij) (2^-g_i y_i).
 // A product of two integers is the sum over digit pairs (t, s) of weight
 // 256^(12 - t - s); the 28 pairs with t + s <= 6 are kept (what is dropped is
 // below 2^-56 of the largest product).  The pairs of one weight share an
@@ -17,9 +21,9 @@
 // leading weights over 256 columns or rows, so FP32 accumulation is exact
 // there; the last weights can round, in the worst case (all digits large and of
 // one sign) at 2^-49 of the result's scale.  The seven accumulators are combined
-// in 64-bit integers.  An entry's error is 2^-56 of its column's largest, against
-// 2^-48 of the entry for the FP32 planes: no larger while the typical (geometric
-// mean) entry is within 2^8 of the largest (Gaussian columns: 2^3.4), else the
+// in 64-bit integers.  An entry's error is 2^-56 of 2^(E_j - g_i), against 2^-48 of
+// the entry for the FP32 planes: no larger while a column's typical (geometric
+// mean) entry is within 2^8 of that (Gaussian matrices: 2^1.5 .. 2^3.1), else the
 // driver takes the double-float form; the residual pass needs 2^5
 // (multi_tc_columns_ok).  Measured at kappa = 1e1 .. 1e10: backward errors 1e-17
 // and forward errors as with FP64 residual passes; A^T (A z) off by 9e-17 of
@@ -52,6 +56,8 @@ constexpr int kPTile = 128 * 64 * 2;        // bytes of a P tile
 constexpr int kPStages = 6;
 constexpr int kTcThreads = 576;             // producer, issuer, 16 epilogue warps
 constexpr int kTcBad = 1 << 20;
+constexpr int kNoGap = 1 << 20;               // a row of zeros
+constexpr int kNoBits = -8192;                // below every row's bits of y minus its gaps
 // h: 256 rows per accumulation.  The d + 1 digit pairs of weight d add up to
 // (d + 1) 2^14 256 <= 2^24 for d <= 3, whatever the digits: exact in FP32.  (1024
 // rows take 8% less time per pass, but weights 1 .. 3 round, at 2^-32 .. 2^-48, where
@@ -96,6 +102,20 @@ __device__ __forceinline__ int pop_digit(long long &q) {
   return d;
 }
 
+// q 2^-sh rounded to an integer, |q 2^-sh| <= 2^55 (or q = 0)
+__device__ __forceinline__ long long shift_round(long long q, int sh) {
+  if (sh > 0) return sh > 62 ? 0 : (q + (1ll << (sh - 1))) >> sh;
+  return q << min(-sh, 63);
+}
+
+// v 2^-g for g >= 0
+__device__ __forceinline__ double scale_down(double v, int g) {
+  const int e = (__double2hiint(v) >> 20) & 0x7ff;
+  if (e == 0x7ff || v == 0.0) return v;
+  if (e <= g) return ldexp(v, -g);
+  return __longlong_as_double(__double_as_longlong(v) - ((long long)g << 52));
+}
+
 // |a| 2^(55 - E) rounded to an integer, with a's sign (|a| < 2^E)
 __device__ __forceinline__ long long tc_fix(double a, int E) {
   const long long b = __double_as_longlong(a);
@@ -110,34 +130,78 @@ __device__ __forceinline__ long long tc_fix(double a, int E) {
   return b < 0 ? -q : q;
 }
 
-// Per column: the largest biased exponent, and the number and the sum of the
-// exponents (minus 1022) of the entries that are not zero.
+// Per column: the largest biased exponent.
 __global__ void __launch_bounds__(256)
     tc_colmax_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int n, TcCol *col) {
   const int j = threadIdx.x;
   if (j >= n) return;
-  int e = 0, cnt = 0;
-  long long sum = 0;
+  int e = 0;
   const int64_t per = (m + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(m, r0 + per);
 #pragma unroll 8
-  for (int64_t i = r0; i < r1; i++) {
-    const int x = (__double2hiint(__ldcs(A + i * lda + j)) >> 20) & 0x7ff;
-    e = max(e, x);
-    cnt += x != 0;
-    sum += x != 0 ? x - 1022 : 0;
-  }
+  for (int64_t i = r0; i < r1; i++)
+    e = max(e, (__double2hiint(__ldcs(A + i * lda + j)) >> 20) & 0x7ff);
   atomicMax(&col[j].emax, e);
-  atomicAdd(&col[j].cnt, cnt);
-  atomicAdd(reinterpret_cast<unsigned long long *>(&col[j].esum), (unsigned long long)sum);
+}
+
+// Per row its gap g_i, the powers of two that its entry nearest to its column's
+// largest lies below it (0 for a row of zeros and beyond m); and per column the
+// number of entries that are not zero and the sum of the powers of two that they
+// lie below 2^(E_j - g_i).  A warp per row; bound by the read of A.
+__global__ void __launch_bounds__(256)
+    tc_rowgap_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int64_t mp, int n,
+                     TcCol *col, short *__restrict__ gap) {
+  __shared__ unsigned long long sums[256];
+  __shared__ int cnts[256];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  sums[threadIdx.x] = 0;
+  cnts[threadIdx.x] = 0;
+  int em[8], cnt[8];
+  long long sum[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    em[k] = 32 * k + lane < n ? col[32 * k + lane].emax : 0;
+    cnt[k] = 0;
+    sum[k] = 0;
+  }
+  __syncthreads();
+  for (int64_t i = (int64_t)blockIdx.x * 8 + warp; i < mp; i += (int64_t)gridDim.x * 8) {
+    int x[8], g = kNoGap;
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+      x[k] = i < m && 32 * k + lane < n
+                 ? (__double2hiint(__ldcs(A + i * lda + 32 * k + lane)) >> 20) & 0x7ff : 0;
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+      if (x[k] != 0) g = min(g, em[k] - x[k]);
+    g = __reduce_min_sync(0xffffffffu, g);
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+      if (x[k] != 0) {
+        sum[k] += em[k] - x[k] - g;
+        cnt[k]++;
+      }
+    if (lane == 0) gap[i] = (short)(g == kNoGap ? 0 : g);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    atomicAdd(&sums[32 * k + lane], (unsigned long long)sum[k]);
+    atomicAdd(&cnts[32 * k + lane], cnt[k]);
+  }
+  __syncthreads();
+  if (threadIdx.x < n) {
+    atomicAdd(&col[threadIdx.x].gaps, sums[threadIdx.x]);
+    atomicAdd(&col[threadIdx.x].cnt, cnts[threadIdx.x]);
+  }
 }
 
 // Digits of a 64 x 64 tile of A into both layouts.  Grid (row tiles up to 128
 // rows, column tiles up to 128 columns); zeros beyond m and n.
 __global__ void __launch_bounds__(256)
     tc_slice_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int n,
-                    const TcCol *__restrict__ col, unsigned char *__restrict__ P1,
-                    unsigned char *__restrict__ P2, int nkc, int64_t nic) {
+                    const TcCol *__restrict__ col, const short *__restrict__ gap,
+                    unsigned char *__restrict__ P1, unsigned char *__restrict__ P2, int nkc,
+                    int64_t nic) {
   __shared__ long long q[64][65];
   const int64_t it = blockIdx.x;  // 64-row tile
   const int jt = blockIdx.y;      // 64-column tile
@@ -145,7 +209,7 @@ __global__ void __launch_bounds__(256)
     const int r = t >> 6, c = t & 63;
     const int64_t i = it * 64 + r;
     const int j = jt * 64 + c;
-    q[r][c] = (i < m && j < n) ? tc_fix(__ldcs(A + i * lda + j), col[j].emax - 1022) : 0;
+    q[r][c] = (i < m && j < n) ? tc_fix(__ldcs(A + i * lda + j), col[j].emax - 1022 - gap[i]) : 0;
   }
   __syncthreads();
   for (int t = threadIdx.x; t < 1024; t += 256) {
@@ -213,7 +277,7 @@ __global__ void __launch_bounds__(256)
   if (ez != 0 && !bad) q = tc_fix(z, e - E);
   if (j == 0) {
     F[c] = bad ? kTcBad : e;
-    ybits[c] = 0;
+    ybits[c] = kNoBits;
   }
   if (j < nkc * 64) {
     unsigned char *base = Q + (size_t)(j >> 6) * tc_qset(nv) + tc_off(c, j & 63);
@@ -278,7 +342,8 @@ struct TcArgs {
   int ranges;            // STEP 1: CTAs per row tile, each a range of the chunks
   int n;
   int nv;                // vectors, a multiple of 16
-  int *ybits;            // STEP 0: bits of the largest |y| per vector
+  const short *gap;      // STEP 0: the rows' gaps
+  int *ybits;            // STEP 0: bits of the largest |y| 2^(-2 gap) per vector
   long long *Y;          // STEP 0: y, vector c at c ldy
   int64_t ldy;
   long long *H;          // STEP 1: partial sums [range][nv][lo, hi][128 tiles]
@@ -300,7 +365,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
   unsigned char *ring = tsm, *qbuf = tsm + (size_t)kPStages * kPTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qbytes = tc_qset(a.nv);
-  if (threadIdx.x < 64) ymax[threadIdx.x] = 0;
+  if (threadIdx.x < 64) ymax[threadIdx.x] = kNoBits;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kPStages; i++) {
       mbar_init(pfull + i, 1);
@@ -484,6 +549,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
     for (int g = 0; g < ngroups; g++) {
       int mt, cb, ce;
       group(g, mt, cb, ce);
+      const int gap2 = STEP == 0 ? 2 * a.gap[128 * (int64_t)mt + row] : 0;
       // one decision per warp
       if (!__all_sync(0xffffffffu, wait(&accfull, (unsigned)(g & 1)))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -537,7 +603,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
           if (STEP == 0) {
             const long long y = v0[e];
             a.Y[(size_t)(c0 + e) * a.ldy + 128 * (int64_t)mt + row] = y;
-            const int bits = __reduce_max_sync(0xffffffffu, 64 - __clzll(y < 0 ? -y : y));
+            const int bits = __reduce_max_sync(0xffffffffu, 64 - __clzll(y < 0 ? -y : y) - gap2);
             if (lane == 0) atomicMax(&ymax[c0 + e], bits);
           } else {
             // no other thread adds here: integer reductions without a reply
@@ -583,30 +649,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-// y's digits, 55 bits against the vector's largest |y| < 2^ybits: one CTA per 64
-// rows, a thread 8 rows of one vector (16 bytes of a tile row per digit).
+// The digits of 2^-g_i y_i (Y holds 2^g_i y_i), 55 bits against the vector's
+// largest, < 2^ybits: one CTA per 64 rows, a thread 8 rows of one vector (16 bytes
+// of a tile row per digit).
 __global__ void __launch_bounds__(256)
     tc_yprep_kernel(const long long *__restrict__ Y, int64_t ldy, int nv,
-                    const int *__restrict__ ybits, unsigned char *__restrict__ Q,
-                    const DevState *gate) {
+                    const int *__restrict__ ybits, const short *__restrict__ gap,
+                    unsigned char *__restrict__ Q, const DevState *gate) {
   if (gate != nullptr && *(volatile const int *)&gate->done) return;
   const int64_t ic = blockIdx.x;
   for (int t = threadIdx.x; t < nv * 8; t += 256) {
-    const int c = t >> 3, g = t & 7, sh = ybits[c] - 55;
+    const int c = t >> 3, g = t & 7, sh0 = ybits[c] - 55;
+    const uint4 gp = *reinterpret_cast<const uint4 *>(gap + ic * 64 + 8 * g);  // 8 gaps, 0 .. 2046
+    const unsigned gw[4] = {gp.x, gp.y, gp.z, gp.w};
     const longlong2 *yp = reinterpret_cast<const longlong2 *>(Y + (size_t)c * ldy + ic * 64 + 8 * g);
     uint4 w[kS];
     unsigned *wp = reinterpret_cast<unsigned *>(w);
 #pragma unroll
     for (int h = 0; h < 4; h++) {
       const longlong2 v = __ldcs(yp + h);
-      long long q0 = v.x, q1 = v.y;
-      if (sh > 0) {
-        q0 = (q0 + (1ll << (sh - 1))) >> sh;
-        q1 = (q1 + (1ll << (sh - 1))) >> sh;
-      } else {
-        q0 <<= -sh;
-        q1 <<= -sh;
-      }
+      long long q0 = shift_round(v.x, sh0 + 2 * (int)(gw[h] & 0xffffu));
+      long long q1 = shift_round(v.y, sh0 + 2 * (int)(gw[h] >> 16));
 #pragma unroll
       for (int s = kS - 1; s >= 0; s--) {
         const int d0 = s > 0 ? pop_digit(q0) : (int)q0, d1 = s > 0 ? pop_digit(q1) : (int)q1;
@@ -619,15 +682,17 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// The residual's middle step, r = b - A x per entry in FP64 from y = A x (in
-// units of 2^(F_c - 54)), in place of y; partial ||r_c||^2 and the largest biased
-// exponent of every r_c.  A CTA takes blocks of 64 rows (b through shared
-// memory: it is row-major, y is vector by vector).
+// The residual's middle step, r_i = b_i - (A x)_i per entry in FP64 from Y = 2^g_i
+// (A x)_i (in units of 2^(F_c - 54)), and 2^-g_i r_i in place of it; partial
+// ||r_c||^2 and the largest biased exponent of every vector's 2^-g_i r_i.  A CTA
+// takes blocks of 64 rows (b through shared memory: it is row-major, y is vector
+// by vector).
 constexpr int kRThreads = 256;
 __global__ void __launch_bounds__(kRThreads)
     tc_resid_kernel(long long *__restrict__ Y, int64_t ldy, int64_t m, int k,
                     const double *__restrict__ B, int64_t ldb, const int *__restrict__ F,
-                    int *__restrict__ rexp, double *__restrict__ r2part) {
+                    const short *__restrict__ gap, int *__restrict__ rexp,
+                    double *__restrict__ r2part) {
   __shared__ double sb[64][65];
   __shared__ double r2s[64];
   __shared__ int ex[64];
@@ -643,19 +708,24 @@ __global__ void __launch_bounds__(kRThreads)
       sb[r][c] = i0 + r < m ? __ldcs(B + (i0 + r) * ldb + c) : 0.0;
     }
     __syncthreads();
+    const int gp[2] = {gap[i0 + lane], gap[i0 + 32 + lane]};
     for (int c = warp; c < k; c += kRThreads / 32) {
-      const double sc = F[c] == kTcBad ? __longlong_as_double(0x7ff8000000000000ll)
-                                       : ldexp(1.0, F[c] - 54);
+      const int f = F[c];
       double s2 = 0.0;
       int e = 0;
 #pragma unroll
       for (int h = 0; h < 2; h++) {
         const int r = 32 * h + lane;
         long long *p = Y + (size_t)c * ldy + i0 + r;
+        const int ex = f - 54 - gp[h] + 1023;  // the unit's biased exponent
+        const double sc = f == kTcBad ? __longlong_as_double(0x7ff8000000000000ll)
+                          : ex >= 1 && ex <= 2046 ? __longlong_as_double((long long)ex << 52)
+                                                  : ldexp(1.0, ex - 1023);
         const double v = i0 + r < m ? fma(-(double)*p, sc, sb[r][c]) : 0.0;
-        *p = __double_as_longlong(v);
+        const double w = scale_down(v, gp[h]);
+        *p = __double_as_longlong(w);
         s2 = fma(v, v, s2);
-        e = max(e, (__double2hiint(v) >> 20) & 0x7ff);
+        e = max(e, (__double2hiint(w) >> 20) & 0x7ff);
       }
       s2 = warp_sum(s2);
       e = __reduce_max_sync(0xffffffffu, e);
@@ -779,18 +849,17 @@ cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int
                                     int nsm, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(b.col, 0, sizeof(TcCol) * (size_t)n, s);
   if (e != cudaSuccess) return e;
-  tc_colmax_kernel<<<nsm * 4, 256, 0, s>>>(A, lda, m, n, b.col);
   const int64_t mp = up64(m, 128);
+  tc_colmax_kernel<<<nsm * 4, 256, 0, s>>>(A, lda, m, n, b.col);
+  tc_rowgap_kernel<<<nsm * 4, 256, 0, s>>>(A, lda, m, mp, n, b.col, b.gap);
   tc_slice_kernel<<<dim3((unsigned)(mp / 64), up(n, 128) / 64), 256, 0, s>>>(
-      A, lda, m, n, b.col, b.p1, b.p2, up(n, 64) / 64, mp / 64);
+      A, lda, m, n, b.col, b.gap, b.p1, b.p2, up(n, 64) / 64, mp / 64);
   return cudaGetLastError();
 }
 
 bool multi_tc_columns_ok(int n, const TcCol *col, double bits) {
   for (int j = 0; j < n; j++)
-    if (col[j].cnt > 0 &&
-        (double)(col[j].emax - 1022) - (double)col[j].esum / (double)col[j].cnt > bits)
-      return false;
+    if (col[j].cnt > 0 && (double)col[j].gaps / (double)col[j].cnt > bits) return false;
   return true;
 }
 
@@ -818,7 +887,7 @@ cudaError_t tc_shape(int64_t m, int n, int k, int nsm, TcShape *t) {
 void tc_step0(const TcShape &t, int n, int k, const double *Z, const TcBufs &b, int nsm,
               const DevState *gate, int *err, cudaStream_t s) {
   tc_zprep_kernel<<<t.nv, 256, 0, s>>>(Z, n, k, t.nv, t.nkc, b.col, b.q, b.F, b.ybits, gate);
-  const TcArgs a = {b.p1, b.q, t.nkc, (int)(t.mp / 128), 1, n, t.nv, b.ybits, b.y64, t.mp, nullptr,
+  const TcArgs a = {b.p1, b.q, t.nkc, (int)(t.mp / 128), 1, n, t.nv, b.gap, b.ybits, b.y64, t.mp, nullptr,
                     gate, err};
   tc_gemm_kernel<0><<<(int)std::min<int64_t>(nsm, t.mp / 128), kTcThreads, t.smem, s>>>(a);
 }
@@ -826,7 +895,7 @@ void tc_step0(const TcShape &t, int n, int k, const double *Z, const TcBufs &b, 
 // out = scale .* A^T y from y's digits
 cudaError_t tc_step1(const TcShape &t, int n, int k, double *out, const double *scale,
                      const TcBufs &b, const DevState *gate, int *err, cudaStream_t s) {
-  const TcArgs a = {b.p2, b.y, (int)(t.mp / 64), t.njt, t.ranges, n, t.nv, nullptr, nullptr, 0, b.h,
+  const TcArgs a = {b.p2, b.y, (int)(t.mp / 64), t.njt, t.ranges, n, t.nv, nullptr, nullptr, nullptr, 0, b.h,
                     gate, err};
   cudaError_t e =
       cudaMemsetAsync(b.h, 0, 2 * sizeof(long long) * (size_t)t.ranges * t.nv * 128 * t.njt, s);
@@ -850,7 +919,7 @@ cudaError_t launch_multi_tc_pass(int64_t m, int n, int k, const double *Z, doubl
   const cudaError_t e = tc_shape(m, n, k, nsm, &t);
   if (e != cudaSuccess) return e;
   tc_step0(t, n, k, Z, b, nsm, gate, err, s);
-  tc_yprep_kernel<<<(unsigned)(t.mp / 64), 256, 0, s>>>(b.y64, t.mp, t.nv, b.ybits, b.y, gate);
+  tc_yprep_kernel<<<(unsigned)(t.mp / 64), 256, 0, s>>>(b.y64, t.mp, t.nv, b.ybits, b.gap, b.y, gate);
   return tc_step1(t, n, k, out, scale, b, gate, err, s);
 }
 
@@ -863,7 +932,8 @@ cudaError_t launch_multi_tc_resid(int64_t m, int n, int k, const double *B, int6
   if (e != cudaSuccess) return e;
   tc_step0(t, n, k, X, b, nsm, nullptr, err, s);
   const int g = (int)std::min<int64_t>((int64_t)nsm * kTcResidCtas, t.mp / 64);
-  tc_resid_kernel<<<g, kRThreads, 0, s>>>(b.y64, t.mp, m, k, B, ldb, b.F, b.ybits + 64, b.r2part);
+  tc_resid_kernel<<<g, kRThreads, 0, s>>>(b.y64, t.mp, m, k, B, ldb, b.F, b.gap,
+                                          b.ybits + 64, b.r2part);
   tc_rprep_kernel<<<(unsigned)(t.mp / 64), 256, 0, s>>>(b.y64, t.mp, k, t.nv, b.ybits + 64, b.y,
                                                        b.F, b.ybits);
   tc_r2_kernel<<<k, 32, 0, s>>>(b.r2part, g, k, r2);

@@ -788,7 +788,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
     LSQ_CU(launch_multi_tc_prepare(dA, P->lda, P->m, n, P->tc, P->nsm, P->s));
     LSQ_CU(cudaMemcpyAsync(P->col_host, P->tc.col, sizeof(TcCol) * n, cudaMemcpyDeviceToHost,
                            P->s));
-    P->launches += 2;
+    P->launches += 3;
   }
   LSQ_CU(cudaEventRecord(P->ev[1], P->s));
   LSQ_CU(launch_qr(P->W, d, n, n + k, P->vbuf, P->qflag, next_epoch(P), P->st,
@@ -945,7 +945,7 @@ void configure_fields(lsq_plan P, const lsq_options *opt) {
 }
 
 void free_tc(lsq_plan P) {
-  void *bufs[] = {P->tc.p1, P->tc.p2, P->tc.q, P->tc.y, P->tc.y64, P->tc.h, P->tc.col, P->tc.F,
+  void *bufs[] = {P->tc.p1, P->tc.p2, P->tc.q, P->tc.y, P->tc.y64, P->tc.h, P->tc.col, P->tc.gap, P->tc.F,
                   P->tc.ybits, P->tc.r2part};
   for (void *b : bufs)
     if (b) cudaFree(b);
@@ -972,6 +972,8 @@ void alloc_tc(lsq_plan P, int n) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.y64, z.y64);
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.h, z.h);
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.col, sizeof(TcCol) * 256);
+  if (e == cudaSuccess)
+    e = cudaMalloc((void **)&P->tc.gap, sizeof(short) * (size_t)((P->m_cap + 127) / 128 * 128));
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.F, sizeof(int) * 64);
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.ybits, sizeof(int) * 128);
   if (e == cudaSuccess) e = cudaMalloc((void **)&P->tc.r2part, z.r2);

@@ -317,13 +317,14 @@ struct TcSizes {
   size_t p1, p2, q, y, y64, h, r2;  // bytes
 };
 struct TcCol {              // a column of A (zeroed, then tc_colmax_kernel)
-  long long esum;           // sum of the exponents of its nonzero entries
+  unsigned long long gaps;  // powers of two that its nonzero entries lie below 2^(E_j - g_i)
   int emax, cnt;            // largest biased exponent, nonzero entries
 };
 struct TcBufs {
   unsigned char *p1, *p2, *q, *y;
   long long *y64, *h;
   TcCol *col;               // n
+  short *gap;               // rows' gaps g_i, m up to 128
   int *F, *ybits;           // 64, 128
   double *r2part;
 };
@@ -331,8 +332,8 @@ TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm);
 cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
                                     int nsm, cudaStream_t s);
 // Whether every column's typical entry (the mean exponent of its nonzero
-// entries) is within `bits` of its largest: fixed point to the largest entry
-// holds it to 2^(bits - 56).
+// entries) is within `bits` of what fixed point holds it against, its column's
+// largest less its row's gap: it is then held to 2^(bits - 56).
 bool multi_tc_columns_ok(int n, const TcCol *col, double bits);
 // The residual pass: out = scale .* A^T (B - A X), r2[c] = ||b_c - A x_c||^2 (X n
 // x k column-major, B m x k row-major).

@@ -845,13 +845,18 @@ TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm) {
   return z;
 }
 
-cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
-                                    int nsm, cudaStream_t s) {
+cudaError_t launch_multi_tc_stats(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
+                                  int nsm, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(b.col, 0, sizeof(TcCol) * (size_t)n, s);
   if (e != cudaSuccess) return e;
-  const int64_t mp = up64(m, 128);
   tc_colmax_kernel<<<nsm * 4, 256, 0, s>>>(A, lda, m, n, b.col);
-  tc_rowgap_kernel<<<nsm * 4, 256, 0, s>>>(A, lda, m, mp, n, b.col, b.gap);
+  tc_rowgap_kernel<<<nsm * 4, 256, 0, s>>>(A, lda, m, up64(m, 128), n, b.col, b.gap);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
+                                    cudaStream_t s) {
+  const int64_t mp = up64(m, 128);
   tc_slice_kernel<<<dim3((unsigned)(mp / 64), up(n, 128) / 64), 256, 0, s>>>(
       A, lda, m, n, b.col, b.gap, b.p1, b.p2, up(n, 64) / 64, mp / 64);
   return cudaGetLastError();

@@ -765,6 +765,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   if (ldb < k) return fail(LSQ_ERR_INVALID, "ldb < nrhs");
   P->launches = 0;
   P->tev_used = 0;
+  P->multi_planes = P->use_tc = false;  // until the planes and digits are this A's
   double *dn2 = P->mstate, *thr = P->mstate + k, *x0n2 = P->mstate + 2 * k;
   double *r2 = P->mstate + 3 * k, *cn2 = P->mstate + 4 * k;
   std::memset(P->st_host, 0, sizeof(DevState));
@@ -785,10 +786,10 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
                                 P->SAb, P->W, P->dcol, P->dinv, P->st, P->s));
   LSQ_CU(launch_sketch_b_to_w(P->SBb, d, n, k, P->zeta, P->W, P->st, P->s));
   if (P->tc_alloc && P->want32) {
-    LSQ_CU(launch_multi_tc_prepare(dA, P->lda, P->m, n, P->tc, P->nsm, P->s));
+    LSQ_CU(launch_multi_tc_stats(dA, P->lda, P->m, n, P->tc, P->nsm, P->s));
     LSQ_CU(cudaMemcpyAsync(P->col_host, P->tc.col, sizeof(TcCol) * n, cudaMemcpyDeviceToHost,
                            P->s));
-    P->launches += 3;
+    P->launches += 2;
   }
   LSQ_CU(cudaEventRecord(P->ev[1], P->s));
   LSQ_CU(launch_qr(P->W, d, n, n + k, P->vbuf, P->qflag, next_epoch(P), P->st,
@@ -808,13 +809,19 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   // FP64 tensor-core contraction
   choose_inner_kernel(P);
   const bool multi_df = P->use_df;
-  P->use_tc = multi_df && P->tc_alloc && multi_tc_columns_ok(n, P->col_host, 8.0);
+  const bool use_tc = multi_df && P->tc_alloc && multi_tc_columns_ok(n, P->col_host, 8.0);
   // the residual's A x and A^T r stand in for FP64 sums: only where 56-bit fixed
   // point is no further off than FP64's rounding
-  const bool tc_resid = P->use_tc && multi_tc_columns_ok(n, P->col_host, 5.0);
-  P->multi_planes = P->want32;  // the sketch above wrote the planes of this A
+  const bool tc_resid = use_tc && multi_tc_columns_ok(n, P->col_host, 5.0);
   if (P->st_host->nonfinite) return fail(LSQ_ERR_NONFINITE, "A or B holds NaN or Inf");
   if (P->st_host->zero_col) return fail(LSQ_ERR_INVALID, "A has a zero column (column scaling)");
+  // the digits, 10 times the work of the statistics, only where they are read
+  if (use_tc) {
+    LSQ_CU(launch_multi_tc_prepare(dA, P->lda, P->m, n, P->tc, P->s));
+    P->launches++;
+  }
+  P->use_tc = use_tc;
+  P->multi_planes = P->want32;  // planes (and digits) of this A
   const int max_inner = P->o.max_inner ? P->o.max_inner : 100;
   const int nref = P->o.max_refine ? P->o.max_refine : 2;
   const int q2 = step2_updates(P->st_host->condest, P->eta, max_inner);

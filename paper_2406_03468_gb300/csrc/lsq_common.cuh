@@ -311,8 +311,9 @@ cudaError_t launch_pass_atax_df_multi(const float *Ahi, const float *Alo, int64_
                                       int n, const double *Z, int k, double *part, int grid,
                                       int npad, const DevState *gate, int *err, cudaStream_t s);
 // The same pass on the tensor cores in fixed point (k_multi_tc.cu): n <= 256,
-// k <= 64.  prepare: the columns' largest exponents and A's digits in both
-// layouts, once per solve; pass: out (n x k column-major) = scale .* A^T (A Z).
+// k <= 64.  stats: the columns' largest exponents and the rows' gaps; prepare: A's
+// digits in both layouts, once per solve that takes this form; pass: out (n x k
+// column-major) = scale .* A^T (A Z).
 struct TcSizes {
   size_t p1, p2, q, y, y64, h, r2;  // bytes
 };
@@ -329,8 +330,10 @@ struct TcBufs {
   double *r2part;
 };
 TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm);
+cudaError_t launch_multi_tc_stats(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
+                                  int nsm, cudaStream_t s);
 cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
-                                    int nsm, cudaStream_t s);
+                                    cudaStream_t s);
 // Whether every column's typical entry (the mean exponent of its nonzero
 // entries) is within `bits` of what fixed point holds it against, its column's
 // largest less its row's gap: it is then held to 2^(bits - 56).

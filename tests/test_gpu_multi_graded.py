@@ -54,3 +54,28 @@ def test_small_rows_keep_their_bits(e, noise):
         err = [np.linalg.norm(v - x) / np.linalg.norm(x) for v in (X[:, c], X64[:, c], fq)]
         assert err[0] <= 10 * max(err[1], 2.0 ** -50), (c, err)
         assert err[0] <= 10 * max(err[2], 2.0 ** -50), (c, err)
+
+
+def test_apply_after_a_refused_solve():
+    """A refused solve leaves no digits or planes behind: the pass that follows
+    works on the matrix it is given (bound: 4 (n + m) u |A|^T |A| |z|)."""
+    m, n, k = 3000, 24, 8
+    rng = np.random.default_rng(3)
+    A, B = rng.standard_normal((m, n)), rng.standard_normal((m, k))
+    plan = lsq.Plan(m, n, seed=1, nrhs=k)
+    X = torch.empty((n, k), dtype=torch.float64, device="cuda")
+    assert lsq.lsq_solve_fossils_multi(plan.handle, T(A), T(B), k, X)[0] == 0
+    bad = A.copy()
+    bad[7, 3] = np.nan
+    with pytest.raises(lsq.LsqError):
+        lsq.lsq_solve_fossils_multi(plan.handle, T(bad), T(B), k, X)
+    C, Z = rng.standard_normal((m, n)), rng.standard_normal((k, n))
+    Hd = torch.empty(n * k, dtype=torch.float64, device="cuda")
+    lsq.lsq_apply_normal_multi(plan.handle, T(C), T(Z), Hd)
+    Hh = H(Hd).reshape(k, n)
+    plan.close()
+    absC = np.abs(C)
+    for c in range(k):
+        h = oracle.residual_dot2(C, np.zeros(m), -Z[c])[2]
+        bound = 4 * (n + m) * 2.0 ** -53 * (absC.T @ (absC @ np.abs(Z[c])))
+        assert (np.abs(Hh[c] - h) <= bound).all(), c

@@ -110,7 +110,12 @@ typedef struct {
   int32_t sparse;        /* 1: the plan solves CSR matrices (lsq_solve_csr) and allocates
                             no FP32 planes or fixed-point copy of A; precision must be
                             FP64, nrhs and kw_stop 0.  0 (default): dense A */
-  int32_t reserved[3];
+  int32_t multi_df;      /* many right-hand sides: not 0 keeps the inner passes in double-float
+                            on the planes and the residual passes in FP64.  0 (default):
+                            both run on the tensor cores in 56-bit fixed point where that
+                            is no further off and the plan has the memory for it
+                            (lsq_multi_form says what ran) */
+  int32_t reserved[2];
 } lsq_options;
 
 #define LSQ_MAX_N 1024
@@ -138,10 +143,11 @@ typedef struct {
                                      2: FP32 tier pass (hi plane), 3: double-float pass on
                                      the hi / lo planes (one batched launch for many
                                      right-hand sides), 4: FP64 tensor-core (DMMA)
-                                     many-right-hand-side pass, 5: the double-float
-                                     pass for many right-hand sides that applies each
-                                     row block of A to all k vectors (A read once) */
-  double bytes_a;                 /* bytes of A (and its FP32 copy) streamed by the solve */
+                                     many-right-hand-side pass, 5: the pass for many
+                                     right-hand sides that applies each row block of A to
+                                     all k vectors: in double-float on the planes, or in
+                                     fixed point on the tensor cores (lsq_multi_form) */
+  double bytes_a;                 /* bytes of A (its FP32 copy, its digits) streamed by the solve */
   double be_sketch_est;           /* kw_stop: the last sketched Karlson-Walden estimate
                                      (absolute; divide by ||A D^-1||_F), else 0 */
 } lsq_info;
@@ -240,14 +246,20 @@ lsq_status lsq_solve_complex(lsq_plan plan, int method, const double *dA, int64_
 /* FOSSILS for k = opt.nrhs right-hand sides sharing one sketch S [A B] and
  * one QR (Alg. 1 with the augmented columns Q^T S B; Alg. 2 / Alg. 5 per
  * column, each column with its own Polyak vectors and step-1 threshold, the
- * step ending when every column meets its own).  The residual pass
- * G = A^T (B - A X) is an FP64 tensor-core (DMMA) contraction over row
- * blocks of A.  The inner pass H = A^T (A Z) runs in double-float on the
- * hi / lo planes, each row block of A applied to all k vectors in one read
- * of A.  With inner_fp64_fma = 1, or column norms outside [2^-40, 2^40], it
- * is also a DMMA contraction.  dB: m x k row-major with leading
- * dimension ldb >= k (0 => k); dX: n x k row-major (device).  Requires
- * n <= 256.  info (may be NULL) reports the largest ||c_i|| over columns. */
+ * step ending when every column meets its own).  The inner pass
+ * H = A^T (A Z) and the residual pass G = A^T (B - A X) run on the tensor cores
+ * in 56-bit fixed point (A scaled by powers of two along its rows and columns)
+ * where that holds A's entries as well as the forms it stands in for: the
+ * columns' typical entries within 2^8 (residual: 2^5) of what they are held
+ * against.  Else, with multi_df, or when the digits of A (about 5 times its bytes at
+ * n = 200, more for few columns) would take more than half of the memory that
+ * is free when the plan is made: the inner pass runs in double-float on the hi /
+ * lo planes, each row block of A applied to all k vectors in one read of A, and
+ * the residual pass is an FP64 tensor-core (DMMA) contraction.  With
+ * inner_fp64_fma = 1, or column norms outside [2^-40, 2^40], both are DMMA
+ * contractions.  dB: m x k row-major with leading dimension ldb >= k (0 => k); dX: n x
+ * k row-major (device).  Requires n <= 256.  info (may be NULL) reports the
+ * largest ||c_i|| over columns. */
 lsq_status lsq_solve_fossils_multi(lsq_plan plan, const double *dA, const double *dB,
                                    int64_t ldb, double *dX, lsq_info *info);
 
@@ -297,6 +309,13 @@ lsq_status lsq_get_sketch_raw(lsq_plan plan, double *dSAb);
 lsq_status lsq_get_R(lsq_plan plan, double *dR, double *dt, double *dx0, double *condest,
                      double *normest);
 
+/* What the plan's last lsq_solve_fossils_multi ran on the tensor cores in fixed
+ * point: LSQ_MULTI_TC_INNER for the inner passes, plus LSQ_MULTI_TC_RESID for the
+ * residual passes; 0: neither, or no such solve yet.  NULL: 0. */
+#define LSQ_MULTI_TC_INNER 1
+#define LSQ_MULTI_TC_RESID 2
+int32_t lsq_multi_form(lsq_plan plan);
+
 /* One fused streaming pass over A: dh = A^T (A dz) (the operator of
  * Sec. 2.1's preconditioned normal equations before the R solves; Alg. 1's
  * Apply), with the inner-pass kernel the solve would use: after lsq_sketch
@@ -309,9 +328,9 @@ lsq_status lsq_apply_normal(lsq_plan plan, const double *dA, const double *dz, d
  * vectors (Alg. 1's Apply for each right-hand side of
  * lsq_solve_fossils_multi), with the inner-pass kernel that solve uses.
  * After lsq_solve_fossils_multi on the same A (it writes the hi / lo FP32
- * planes) and unless inner_fp64_fma is set: double-float on the planes,
- * every row block of A applied to all k vectors while it is in shared
- * memory; otherwise the FP64 tensor-core (DMMA) contraction on dA.  dZ, dH:
+ * planes and the digits) and unless inner_fp64_fma is set: the form that
+ * lsq_multi_form names, fixed point or double-float on the planes; otherwise
+ * the FP64 tensor-core (DMMA) contraction on dA.  dZ, dH:
  * n x k column-major (vector c at offset c n), device.  No scaling is
  * applied.  Errors: LSQ_ERR_INVALID (NULL argument, nrhs = 0 plan). */
 lsq_status lsq_apply_normal_multi(lsq_plan plan, const double *dA, const double *dZ, double *dH);

@@ -16,7 +16,7 @@ __all__ = [
     "LsqError", "LsqOptions", "LsqInfo", "lsq_options_default", "lsq_plan_create",
     "lsq_plan_destroy", "lsq_plan_configure", "lsq_sketch", "lsq_solve_fossils", "lsq_solve_spir",
     "lsq_solve_spir_lsqr", "lsq_solve_host", "lsq_solve_complex", "lsq_solve_csr",
-    "lsq_solve_fossils_multi",
+    "lsq_solve_fossils_multi", "lsq_multi_form",
     "lsq_sketch_pattern", "lsq_get_sketch", "lsq_get_sketch_raw", "lsq_get_R", "lsq_apply_normal",
     "lsq_apply_normal_multi", "lsq_residual", "lsq_sketched_kw",
     "lsq_trsv", "lsq_apply_normal_noalloc", "lsq_last_error", "Plan", "lsq_server_create",
@@ -30,6 +30,7 @@ LSQ_OK = 0
 LSQ_PENDING = 1
 LSQ_WARN_RANK_DEFICIENT = 2
 LSQ_PREC_AUTO, LSQ_PREC_FP64, LSQ_PREC_FP32_INNER = 0, 1, 2
+LSQ_MULTI_TC_INNER, LSQ_MULTI_TC_RESID = 1, 2
 LSQ_MAX_REFINE = 8
 
 _STATUS = {0: "LSQ_OK", 1: "LSQ_PENDING", 2: "LSQ_WARN_RANK_DEFICIENT", -1: "LSQ_ERR_INVALID",
@@ -53,7 +54,8 @@ class LsqOptions(ctypes.Structure):
                 ("fixed_inner", ctypes.c_int32), ("timing", ctypes.c_int32),
                 ("inner_fp64_fma", ctypes.c_int32), ("nrhs", ctypes.c_int32),
                 ("qr_wait_us", ctypes.c_int32), ("kw_stop", ctypes.c_int32),
-                ("sparse", ctypes.c_int32), ("reserved", ctypes.c_int32 * 3)]
+                ("sparse", ctypes.c_int32), ("multi_df", ctypes.c_int32),
+                ("reserved", ctypes.c_int32 * 2)]
 
 
 class LsqInfo(ctypes.Structure):
@@ -105,6 +107,7 @@ EXPORTED = {
     "lsq_solve_host": (_i32, [_vp, _i32, _vp, _vp, _vp, ctypes.POINTER(LsqInfo)]),
     "lsq_solve_fossils_multi": (_i32, [_vp, _vp, _vp, ctypes.c_int64, _vp,
                                        ctypes.POINTER(LsqInfo)]),
+    "lsq_multi_form": (_i32, [_vp]),
     "lsq_solve_complex": (_i32, [_vp, _i32, _vp, ctypes.c_int64, _vp, _vp, _vp,
                                  ctypes.POINTER(LsqInfo)]),
     "lsq_solve_csr": (_i32, [_vp, _i32, ctypes.c_int64, _vp, _vp, _vp, _vp, _vp,
@@ -251,6 +254,12 @@ def lsq_solve_fossils_multi(plan, A, B, ldb, X, info=None):
     st = _check(_lib().lsq_solve_fossils_multi(plan, _ptr(A), _ptr(B), int(ldb), _ptr(X),
                                                ctypes.byref(inf)))
     return st, inf
+
+
+def lsq_multi_form(plan):
+    """LSQ_MULTI_TC_INNER (1) + LSQ_MULTI_TC_RESID (2) for the passes of the last
+    many-right-hand-side solve that ran on the tensor cores in fixed point."""
+    return _lib().lsq_multi_form(plan)
 
 
 def lsq_solve_host(plan, method, A, b, x, info=None):

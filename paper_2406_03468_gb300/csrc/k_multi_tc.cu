@@ -845,6 +845,12 @@ TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm) {
   return z;
 }
 
+double multi_tc_pass_bytes(int64_t m, int n) {
+  const double mp = (double)up64(m, 128);
+  // the first layout whole, of the second the rows below n up to 8
+  return mp / 128 * tc_cols(n).tiles * kPTile + mp / 64 * kS * 128.0 * up(n, 8);
+}
+
 cudaError_t launch_multi_tc_stats(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
                                   int nsm, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(b.col, 0, sizeof(TcCol) * (size_t)n, s);

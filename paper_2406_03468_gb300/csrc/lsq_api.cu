@@ -136,7 +136,7 @@ struct lsq_plan_s {
   bool multi_planes = false;        // the planes hold the A of the last multi solve
   double *SBb = nullptr, *cpartB = nullptr, *mpart = nullptr, *mr2part = nullptr, *mT = nullptr;
   TcBufs tc{};                // tensor-core pass: digits of A, z, y, partial sums
-  bool tc_alloc = false, use_tc = false;
+  bool tc_alloc = false, use_tc = false, use_tc_resid = false;  // the last two: the last solve's
   TcCol *col_host = nullptr;
   double *mpartdf = nullptr;  // partials of the batched double-float pass (k x gpass x npad)
   double *mXs = nullptr, *mXo = nullptr, *mC = nullptr, *mG = nullptr, *mDY = nullptr;
@@ -765,7 +765,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   if (ldb < k) return fail(LSQ_ERR_INVALID, "ldb < nrhs");
   P->launches = 0;
   P->tev_used = 0;
-  P->multi_planes = P->use_tc = false;  // until the planes and digits are this A's
+  P->multi_planes = P->use_tc = P->use_tc_resid = false;  // until the planes and digits are this A's
   double *dn2 = P->mstate, *thr = P->mstate + k, *x0n2 = P->mstate + 2 * k;
   double *r2 = P->mstate + 3 * k, *cn2 = P->mstate + 4 * k;
   std::memset(P->st_host, 0, sizeof(DevState));
@@ -785,7 +785,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   LSQ_CU(launch_sketch_finalize(P->cpart, P->gpass, P->npad, n, d, P->zeta, P->o.col_scale,
                                 P->SAb, P->W, P->dcol, P->dinv, P->st, P->s));
   LSQ_CU(launch_sketch_b_to_w(P->SBb, d, n, k, P->zeta, P->W, P->st, P->s));
-  if (P->tc_alloc && P->want32) {
+  if (P->tc_alloc && P->want32 && !P->o.multi_df) {
     LSQ_CU(launch_multi_tc_stats(dA, P->lda, P->m, n, P->tc, P->nsm, P->s));
     LSQ_CU(cudaMemcpyAsync(P->col_host, P->tc.col, sizeof(TcCol) * n, cudaMemcpyDeviceToHost,
                            P->s));
@@ -809,7 +809,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   // FP64 tensor-core contraction
   choose_inner_kernel(P);
   const bool multi_df = P->use_df;
-  const bool use_tc = multi_df && P->tc_alloc && multi_tc_columns_ok(n, P->col_host, 8.0);
+  const bool use_tc = multi_df && P->tc_alloc && !P->o.multi_df && multi_tc_columns_ok(n, P->col_host, 8.0);
   // the residual's A x and A^T r stand in for FP64 sums: only where 56-bit fixed
   // point is no further off than FP64's rounding
   const bool tc_resid = use_tc && multi_tc_columns_ok(n, P->col_host, 5.0);
@@ -821,6 +821,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
     P->launches++;
   }
   P->use_tc = use_tc;
+  P->use_tc_resid = tc_resid;
   P->multi_planes = P->want32;  // planes (and digits) of this A
   const int max_inner = P->o.max_inner ? P->o.max_inner : 100;
   const int nref = P->o.max_refine ? P->o.max_refine : 2;
@@ -847,7 +848,8 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
     const int cap = fixed ? P->o.fixed_inner : (i == 0 ? max_inner : q2);
     const int use_thresh = (!fixed && i == 0) ? 1 : 0;
     LSQ_CU(launch_multi_init(n, k, P->mC, P->mDY, P->mDYold, cap, use_thresh, P->st, P->s));
-    P->launches += 5;
+    // resid; trsv, [thresh], init
+    P->launches += (tc_resid ? 7 : 2) + 2 + (i == 0 ? 1 : 0);
     for (int it = 0; it < cap; it++) {
       LSQ_CU(launch_multi_xprod(n, k, 0, P->Xrm, P->mDY, P->dinv, P->mZ, P->st, P->s));
       int tj = -1;
@@ -867,7 +869,7 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
       }
       LSQ_CU(launch_multi_xprod(n, k, 1, P->Xcm, P->mH, nullptr, P->mW, P->st, P->s));
       LSQ_CU(launch_multi_polyak(n, k, P->mC, P->mW, P->mDY, P->mDYold, dn2, thr, P->st, P->s));
-      P->launches += 6;
+      P->launches += 3 + (use_tc ? 5 : 2);  // two products, the update; the pass
       if (use_thresh && (it % kStopPollEvery) == kStopPollEvery - 1 && it + 1 < cap) {
         LSQ_TRY(read_state(P));
         if (P->st_host->done) break;
@@ -895,13 +897,18 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
     }
     info->refine_steps = nref;
     info->path = LSQ_PREC_FP64;
-    info->inner_kernel = !multi_df ? 4 : multi_df_supported(n, k, P->ld32) ? 5 : 3;
+    info->inner_kernel = !multi_df ? 4 : use_tc || multi_df_supported(n, k, P->ld32) ? 5 : 3;
     info->passes = 2 + nref + iters[0] + iters[1];
     info->status = status;
     info->condest = S.condest;
     info->normest = S.normest;
     info->launches = P->launches;
-    info->bytes_a = 8.0 * (double)P->m * n * (1 + nref + iters[0] + (nref > 1 ? iters[1] : 0));
+    // the sketch; the digits (A read three times); the passes
+    const double mn8 = 8.0 * (double)P->m * n, dig = use_tc ? multi_tc_pass_bytes(P->m, n) : 0.0;
+    int updates = 0;
+    for (int i = 0; i < nref; i++) updates += iters[i];
+    info->bytes_a = mn8 + (use_tc ? 3.0 * mn8 + dig : 0.0) + nref * (tc_resid ? dig : mn8) +
+                    updates * (use_tc ? dig : mn8);
     float ms = 0;
     cudaEventElapsedTime(&ms, P->ev[0], P->ev[1]);
     info->ms_sketch = ms;
@@ -1145,7 +1152,7 @@ lsq_status lsq_plan_create(const lsq_options *opt, void *cuda_stream, lsq_plan *
     A(dalloc(&P->Alo, (size_t)P->m_cap * ((n + 3) / 4 * 4)));
     P->want32 = true;
   }
-  if (e == cudaSuccess && P->k > 0 && P->Ahi) alloc_tc(P, n);
+  if (e == cudaSuccess && P->k > 0 && P->Ahi && !P->o.multi_df) alloc_tc(P, n);
   for (auto &ev : P->ev) A(cudaEventCreate(&ev));
   A(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
   A(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
@@ -1288,6 +1295,11 @@ lsq_status lsq_solve_fossils_multi(lsq_plan plan, const double *dA, const double
                                    int64_t ldb, double *dX, lsq_info *info) {
   if (!plan) return fail(LSQ_ERR_INVALID, "plan is NULL");
   return run_solve_multi(plan, dA, dB, ldb, dX, info);
+}
+
+int32_t lsq_multi_form(lsq_plan P) {
+  if (!P) return 0;
+  return (P->use_tc ? LSQ_MULTI_TC_INNER : 0) | (P->use_tc_resid ? LSQ_MULTI_TC_RESID : 0);
 }
 
 lsq_status lsq_solve_host(lsq_plan P, int method, const double *hA, const double *hb, double *hx,

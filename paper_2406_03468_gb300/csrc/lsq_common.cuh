@@ -330,6 +330,7 @@ struct TcBufs {
   double *r2part;
 };
 TcSizes multi_tc_sizes(int64_t m, int n, int k, int nsm);
+double multi_tc_pass_bytes(int64_t m, int n);  // digits of A that a pass reads (both layouts)
 cudaError_t launch_multi_tc_stats(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,
                                   int nsm, cudaStream_t s);
 cudaError_t launch_multi_tc_prepare(const double *A, int64_t lda, int64_t m, int n, const TcBufs &b,

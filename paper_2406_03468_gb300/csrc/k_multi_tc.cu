@@ -15,19 +15,26 @@
 //       its largest entry (|A| |z| can be kappa times |A z|), A^T y being
 //       2^E_j times the sum over i of (2^(g_i - E_j) a_ij) (2^-g_i y_i).
 // A product of two integers is the sum over digit pairs (t, s) of weight
-// 256^(12 - t - s); the 28 pairs with t + s <= 6 are kept (what is dropped is
-// below 2^-56 of the largest product).  The pairs of one weight share an
-// accumulator: products are at most 2^14 and the sums at most 2^24 for the 4
-// leading weights over 256 columns or rows, so FP32 accumulation is exact
-// there; the last weights can round, in the worst case (all digits large and of
-// one sign) at 2^-49 of the result's scale.  The seven accumulators are combined
-// in 64-bit integers.  An entry's error is 2^-56 of 2^(E_j - g_i), against 2^-48 of
-// the entry for the FP32 planes: no larger while a column's typical (geometric
-// mean) entry is within 2^8 of that (Gaussian matrices: 2^1.5 .. 2^3.1), else the
-// driver takes the double-float form; the residual pass needs 2^5
-// (multi_tc_columns_ok).  Measured at kappa = 1e1 .. 1e10: backward errors 1e-17
-// and forward errors as with FP64 residual passes; A^T (A z) off by 9e-17 of
-// |A|^T |A z| (double-float: 3e-15).
+// 256^(12 - t - s).  The inner pass keeps the 28 pairs with t + s <= 6: what is
+// dropped is 2^-56.3 (rms of random digits; 2^-53.4 at most) of the largest
+// product per term, 2^-52.5 over 200 full-scale terms.  The residual pass, which
+// stands in for FP64 sums, keeps the 34 with t + s <= 7 (dropped: 2^-61.7 at most):
+// with 28 its answers were up to 2.9 times further off than with FP64 residual
+// passes (n = 16, kappa 1e3 .. 1e6; 3.8 times with one large entry per row), with
+// 34 they are no further off (1e6, consistent: 0.4 times).  The pairs of one weight
+// share an accumulator: products are at most 2^14 and the sums at most 2^24 for the
+// 4 leading weights over 256 columns or rows, so FP32 accumulation is exact there;
+// the others reach 2^24 and round only where the digits of many terms are all
+// large and of one sign, at 2^-49 of the result's scale.  The accumulators (7 or 8)
+// are combined in 64-bit integers.  An entry's error is 2^-56 of 2^(E_j - g_i),
+// against 2^-48 of the entry for the FP32 planes: no larger while a column's
+// typical (geometric mean) entry is within 2^8 of that (Gaussian matrices: 2^1.5 ..
+// 2^3.1), else the driver takes the double-float form; the residual pass needs 2^5
+// (multi_tc_columns_ok).  Per row, A x of the residual pass is off by 2^-54 .. 2^-57
+// of |A| |x| (rms; sequential FP64 sums: 2^-53 .. 2^-55; n = 16 .. 200, graded x, one
+// large entry per row, rows graded by 2^30).  Measured at kappa = 1e1 .. 1e10:
+// backward errors 1e-17; A^T (A z) of the inner pass off by 9e-17 of |A|^T |A z|
+// (double-float: 3e-15).
 //
 // Both products are the same GEMM, D[128 x 64] += P^(t)[128 x K] Q^(s)[64 x K]^T:
 //   y:  P = A (rows i, K = columns j),     Q = Z^T  -> y in 64 bits and each
@@ -37,7 +44,7 @@
 // that the tensor cores read (128 rows of 64 bf16, 128-byte swizzle, 16 KB):
 // a tile is one contiguous bulk copy.  A CTA (one per SM) runs a producer warp
 // (copies: a ring of P tiles, two sets of Q tiles), an issuing warp (one thread)
-// and sixteen warps that read the accumulators (7 x 64 columns of TMEM).
+// and sixteen warps that read the accumulators (7 or 8 x 64 columns of TMEM).
 //
 // Measured: see launch_multi_tc_pass.  Every wait is bounded; on a timeout
 // the CTA records LSQ_ERR_TIMEOUT, waits (bounded) for its copies and MMAs,
@@ -344,6 +351,7 @@ struct TcArgs {
   int nv;                // vectors, a multiple of 16
   const short *gap;      // STEP 0: the rows' gaps
   int *ybits;            // STEP 0: bits of the largest |y| 2^(-2 gap) per vector
+  int ysh;               // STEP 0, W = 8: Y in units of 2^(F_c - 54 - ysh)
   long long *Y;          // STEP 0: y, vector c at c ldy
   int64_t ldy;
   long long *H;          // STEP 1: partial sums [range][nv][lo, hi][128 tiles]
@@ -352,8 +360,8 @@ struct TcArgs {
 };
 
 // STEP 0: y (P = A), one accumulation per row tile; STEP 1: h (P = A^T), one
-// per kFlushChunks chunks of the CTA's range.
-template <int STEP>
+// per kFlushChunks chunks of the CTA's range.  W: the weights kept, t + s < W.
+template <int STEP, int W>
 __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) {
   if (a.gate != nullptr && *(volatile const int *)&a.gate->done) return;
   extern __shared__ __align__(1024) unsigned char tsm_raw[];
@@ -513,11 +521,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
             if (kk < ks) {
               const unsigned acc = (c > cb || t > 0 || kk > 0) ? 1u : 0u;
               const uint64_t da = tc_desc(pb + 2 * kk);
-              for (int s = 0; s < kS - t; s += gq) {
-                const unsigned gd = min(gq, kS - t - s);
+              const int se = min(kS, W - t);  // digits of Q for this one of P
+              // weight 7's accumulator begins with (1, 6), in an MMA of its own
+              const int sw = W > kS && t == 1 ? se - 1 : se;
+              for (int s = 0; s < sw; s += gq) {
+                const unsigned gd = min(gq, sw - s);
                 tc_mma(tmem + a.nv * (s + t), da, tc_desc(qb + s * qstep + 2 * kk),
                        idesc | (gd * (a.nv >> 3)) << 17, acc);
               }
+              if (sw < se)
+                tc_mma(tmem + a.nv * (sw + t), da, tc_desc(qb + sw * qstep + 2 * kk),
+                       idesc | (a.nv >> 3) << 17, c > cb || kk > 0 ? 1u : 0u);
             }
           }
           if (++q == dpt || t == kS - 1) {
@@ -553,15 +567,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
       // one decision per warp
       if (!__all_sync(0xffffffffu, wait(&accfull, (unsigned)(g & 1)))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      float T[kS][8];
+      float T[W][8];
       long long v0[8];
       int v1[8];  // STEP 1: the high sum
       auto load = [&](int c0) {
 #pragma unroll
-        for (int d = 0; d < kS; d++) tc_ld8(tl + a.nv * d + c0, T[d]);
+        for (int d = 0; d < W; d++) tc_ld8(tl + a.nv * d + c0, T[d]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int d = 0; d < kS; d++)
+        for (int d = 0; d < W; d++)
 #pragma unroll
           for (int e = 0; e < 8; e++)
             asm volatile("" : "+f"(T[d][e])::"memory");  // no use before the wait
@@ -574,12 +588,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
 #pragma unroll
         for (int e = 0; e < 8; e++) {
           if (STEP == 0) {
-            // y in units of 2^(F_c - 54): sum_d T_d 256^(5 - d)
-            long long y = __float2int_rn(T[5][e]) + ((__float2int_rn(T[6][e]) + 128) >> 8);
+            // y in units of 2^(F_c - 54): sum_d T_d 256^(5 - d); W = 8: ysh bits
+            // more, as many as |y| < n 2^F_c leaves room for
+            long long y = __float2int_rn(T[5][e]);
+            if (W == kS) y += (__float2int_rn(T[6][e]) + 128) >> 8;
             y = mad_wide(__float2int_rn(T[4][e]), 1 << 8, y);
             y = mad_wide(__float2int_rn(T[3][e]), 1 << 16, y);
             y = mad_wide(__float2int_rn(T[2][e]), 1 << 24, y);
-            v0[e] = y + ((long long)(__float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8)) << 32);
+            y += (long long)(__float2int_rn(T[1][e]) + (__float2int_rn(T[0][e]) << 8)) << 32;
+            if (W > kS) {
+              const long long low = mad_wide(__float2int_rn(T[6][e]), 1 << 8,
+                                             (long long)__float2int_rn(T[W - 1][e]));
+              y = (y << a.ysh) + ((low + (1ll << (15 - a.ysh))) >> (16 - a.ysh));
+            }
+            v0[e] = y;
           } else {
             // exact in two 64-bit sums: lo = sum_{d >= 2} T_d 256^(6 - d), hi = T_1 +
             // 256 T_0 (A^T r cancels: rounding the sum to 64 bits at 2^-50 of its
@@ -587,6 +609,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(const TcArgs a) 
             // bits from 40 up are hi's units, so lo's sum stays below 2^63 over
             // 2^23 accumulations
             long long lo = __float2int_rn(T[6][e]);
+            if (W > kS) lo += (__float2int_rn(T[W - 1][e]) + 128) >> 8;
             lo = mad_wide(__float2int_rn(T[5][e]), 1 << 8, lo);
             lo = mad_wide(__float2int_rn(T[4][e]), 1 << 16, lo);
             lo = mad_wide(__float2int_rn(T[3][e]), 1 << 24, lo);
@@ -683,7 +706,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // The residual's middle step, r_i = b_i - (A x)_i per entry in FP64 from Y = 2^g_i
-// (A x)_i (in units of 2^(F_c - 54)), and 2^-g_i r_i in place of it; partial
+// (A x)_i (in units of 2^(F_c - 54 - ysh)), and 2^-g_i r_i in place of it; partial
 // ||r_c||^2 and the largest biased exponent of every vector's 2^-g_i r_i.  A CTA
 // takes blocks of 64 rows (b through shared memory: it is row-major, y is vector
 // by vector).
@@ -691,7 +714,7 @@ constexpr int kRThreads = 256;
 __global__ void __launch_bounds__(kRThreads)
     tc_resid_kernel(long long *__restrict__ Y, int64_t ldy, int64_t m, int k,
                     const double *__restrict__ B, int64_t ldb, const int *__restrict__ F,
-                    const short *__restrict__ gap, int *__restrict__ rexp,
+                    const short *__restrict__ gap, int ysh, int *__restrict__ rexp,
                     double *__restrict__ r2part) {
   __shared__ double sb[64][65];
   __shared__ double r2s[64];
@@ -717,7 +740,7 @@ __global__ void __launch_bounds__(kRThreads)
       for (int h = 0; h < 2; h++) {
         const int r = 32 * h + lane;
         long long *p = Y + (size_t)c * ldy + i0 + r;
-        const int ex = f - 54 - gp[h] + 1023;  // the unit's biased exponent
+        const int ex = f - 54 - ysh - gp[h] + 1023;  // the unit's biased exponent
         const double sc = f == kTcBad ? __longlong_as_double(0x7ff8000000000000ll)
                           : ex >= 1 && ex <= 2046 ? __longlong_as_double((long long)ex << 52)
                                                   : ldexp(1.0, ex - 1023);
@@ -876,6 +899,13 @@ bool multi_tc_columns_ok(int n, const TcCol *col, double bits) {
 
 namespace {
 
+// bits that |y| < n 2^F_c leaves above 2^62: n <= 256 >> ysh
+int tc_ysh(int n) {
+  int sh = 0;
+  while (sh < 8 && n <= (128 >> sh)) sh++;
+  return sh;
+}
+
 struct TcShape {
   int nv, nkc, njt, ranges;
   int64_t mp;
@@ -889,29 +919,34 @@ cudaError_t tc_shape(int64_t m, int n, int k, int nsm, TcShape *t) {
   t->ranges = nsm / t->njt;
   t->mp = up64(m, 128);
   t->smem = (size_t)kPStages * kPTile + 2 * (size_t)tc_qset(t->nv) + 1024;
-  cudaError_t e = ensure_smem_attr((const void *)tc_gemm_kernel<0>, (int)t->smem);
-  if (e == cudaSuccess) e = ensure_smem_attr((const void *)tc_gemm_kernel<1>, (int)t->smem);
+  const void *fn[] = {(const void *)tc_gemm_kernel<0, 7>, (const void *)tc_gemm_kernel<1, 7>,
+                      (const void *)tc_gemm_kernel<0, 8>, (const void *)tc_gemm_kernel<1, 8>};
+  cudaError_t e = cudaSuccess;
+  for (const void *f : fn)
+    if (e == cudaSuccess) e = ensure_smem_attr(f, (int)t->smem);
   return e;
 }
 
 // y = A z in 64 bits
+template <int W>
 void tc_step0(const TcShape &t, int n, int k, const double *Z, const TcBufs &b, int nsm,
               const DevState *gate, int *err, cudaStream_t s) {
   tc_zprep_kernel<<<t.nv, 256, 0, s>>>(Z, n, k, t.nv, t.nkc, b.col, b.q, b.F, b.ybits, gate);
-  const TcArgs a = {b.p1, b.q, t.nkc, (int)(t.mp / 128), 1, n, t.nv, b.gap, b.ybits, b.y64, t.mp, nullptr,
+  const TcArgs a = {b.p1, b.q, t.nkc, (int)(t.mp / 128), 1, n, t.nv, b.gap, b.ybits, tc_ysh(n), b.y64, t.mp, nullptr,
                     gate, err};
-  tc_gemm_kernel<0><<<(int)std::min<int64_t>(nsm, t.mp / 128), kTcThreads, t.smem, s>>>(a);
+  tc_gemm_kernel<0, W><<<(int)std::min<int64_t>(nsm, t.mp / 128), kTcThreads, t.smem, s>>>(a);
 }
 
 // out = scale .* A^T y from y's digits
+template <int W>
 cudaError_t tc_step1(const TcShape &t, int n, int k, double *out, const double *scale,
                      const TcBufs &b, const DevState *gate, int *err, cudaStream_t s) {
-  const TcArgs a = {b.p2, b.y, (int)(t.mp / 64), t.njt, t.ranges, n, t.nv, nullptr, nullptr, nullptr, 0, b.h,
+  const TcArgs a = {b.p2, b.y, (int)(t.mp / 64), t.njt, t.ranges, n, t.nv, nullptr, nullptr, 0, nullptr, 0, b.h,
                     gate, err};
   cudaError_t e =
       cudaMemsetAsync(b.h, 0, 2 * sizeof(long long) * (size_t)t.ranges * t.nv * 128 * t.njt, s);
   if (e != cudaSuccess) return e;
-  tc_gemm_kernel<1><<<t.ranges * t.njt, kTcThreads, t.smem, s>>>(a);
+  tc_gemm_kernel<1, W><<<t.ranges * t.njt, kTcThreads, t.smem, s>>>(a);
   tc_reduce_kernel<<<dim3(up(n, 32) / 32, k), 256, 0, s>>>(
       b.h, t.ranges, t.nv, 128 * t.njt, n, b.col, b.F, b.ybits, scale, out, gate);
   return cudaGetLastError();
@@ -929,9 +964,9 @@ cudaError_t launch_multi_tc_pass(int64_t m, int n, int k, const double *Z, doubl
   TcShape t;
   const cudaError_t e = tc_shape(m, n, k, nsm, &t);
   if (e != cudaSuccess) return e;
-  tc_step0(t, n, k, Z, b, nsm, gate, err, s);
+  tc_step0<kS>(t, n, k, Z, b, nsm, gate, err, s);
   tc_yprep_kernel<<<(unsigned)(t.mp / 64), 256, 0, s>>>(b.y64, t.mp, t.nv, b.ybits, b.gap, b.y, gate);
-  return tc_step1(t, n, k, out, scale, b, gate, err, s);
+  return tc_step1<kS>(t, n, k, out, scale, b, gate, err, s);
 }
 
 cudaError_t launch_multi_tc_resid(int64_t m, int n, int k, const double *B, int64_t ldb,
@@ -941,14 +976,14 @@ cudaError_t launch_multi_tc_resid(int64_t m, int n, int k, const double *B, int6
   cudaError_t e = tc_shape(m, n, k, nsm, &t);
   if (e == cudaSuccess) e = cudaMemsetAsync(b.ybits + 64, 0, sizeof(int) * 64, s);
   if (e != cudaSuccess) return e;
-  tc_step0(t, n, k, X, b, nsm, nullptr, err, s);
+  tc_step0<kS + 1>(t, n, k, X, b, nsm, nullptr, err, s);
   const int g = (int)std::min<int64_t>((int64_t)nsm * kTcResidCtas, t.mp / 64);
-  tc_resid_kernel<<<g, kRThreads, 0, s>>>(b.y64, t.mp, m, k, B, ldb, b.F, b.gap,
+  tc_resid_kernel<<<g, kRThreads, 0, s>>>(b.y64, t.mp, m, k, B, ldb, b.F, b.gap, tc_ysh(n),
                                           b.ybits + 64, b.r2part);
   tc_rprep_kernel<<<(unsigned)(t.mp / 64), 256, 0, s>>>(b.y64, t.mp, k, t.nv, b.ybits + 64, b.y,
                                                        b.F, b.ybits);
   tc_r2_kernel<<<k, 32, 0, s>>>(b.r2part, g, k, r2);
-  return tc_step1(t, n, k, out, scale, b, nullptr, err, s);
+  return tc_step1<kS + 1>(t, n, k, out, scale, b, nullptr, err, s);
 }
 
 }  // namespace lsq

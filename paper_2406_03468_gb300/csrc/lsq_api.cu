@@ -810,8 +810,8 @@ lsq_status run_solve_multi(lsq_plan P, const double *dA, const double *dB, int64
   choose_inner_kernel(P);
   const bool multi_df = P->use_df;
   const bool use_tc = multi_df && P->tc_alloc && !P->o.multi_df && multi_tc_columns_ok(n, P->col_host, 8.0);
-  // the residual's A x and A^T r stand in for FP64 sums: only where 56-bit fixed
-  // point is no further off than FP64's rounding
+  // the residual's A x and A^T r stand in for FP64 sums: only where entries are held to
+  // 2^-51 and better, which leaves both products no further off than FP64's rounding
   const bool tc_resid = use_tc && multi_tc_columns_ok(n, P->col_host, 5.0);
   if (P->st_host->nonfinite) return fail(LSQ_ERR_NONFINITE, "A or B holds NaN or Inf");
   if (P->st_host->zero_col) return fail(LSQ_ERR_INVALID, "A has a zero column (column scaling)");

@@ -6,8 +6,9 @@
 // eta = sqrt(n/d), the step-1 stopping rule, the q0 count of Theorem 7.1 for
 // step 2).  Every step is one of this library's kernels, enqueued on the
 // plan's stream; the host only waits (a) once after the sketch and QR, for
-// condest and the input checks, and (b) every few inner iterations of step 1
-// to learn whether the device-side stop test has fired.
+// condest and the input checks, (b) in step 1, a few updates ahead of the device,
+// for the word in which the device reports its progress and whether its stop
+// test has fired, and (c) at the end of each step.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -17,6 +18,7 @@
 #include <string>
 #include <map>
 #include <mutex>
+#include <thread>
 #include <vector>
 
 #include "lsq_common.cuh"
@@ -47,7 +49,7 @@ lsq_status fail(lsq_status st, const std::string &msg) {
 
 constexpr uint64_t kBarrierTimeoutNs = 5ull * 1000 * 1000 * 1000;  // 5 s per inter-CTA wait
 constexpr int kCondestIters = 10;
-constexpr int kStopPollEvery = 4;  // many right-hand sides, step 1: read the stop flag every 4 updates
+constexpr int kStopPollEvery = 4;  // step 1, many right-hand sides or a blocking device: updates per stop test
 constexpr int kRunAhead = 3;       // step 1: updates enqueued beyond the one the device has finished
 constexpr int kHostChunksMax = 16;             // host entry: row chunks of A at most
 constexpr double kHostChunkBytes = 128.0e6;    // and at least this many bytes each
@@ -296,7 +298,9 @@ lsq_status read_state(lsq_plan P) {
 // Wait until the device has finished update `need` of the running inner loop
 // or stopped it (*done); no synchronisation, so the iterations behind it stay
 // enqueued.  The stream running empty first means the loop never started
-// (done before the first update) or an error: the state tells.
+// (done before the first update) or an error: the state tells.  A spin, as the
+// synchronisation it stands for is by default; a device that is set to block its
+// waiting threads takes stop_polled instead.
 lsq_status wait_progress(lsq_plan P, int need, bool *done) {
   volatile const int *hp = P->hprog;
   for (int spin = 0;; spin++) {
@@ -307,6 +311,7 @@ lsq_status wait_progress(lsq_plan P, int need, bool *done) {
     }
     if (v >= need) return LSQ_OK;
     if ((spin & 255) == 255) {
+      std::this_thread::yield();
       const cudaError_t q = cudaStreamQuery(P->s);
       if (q == cudaErrorNotReady) continue;
       LSQ_CU(q);
@@ -317,6 +322,21 @@ lsq_status wait_progress(lsq_plan P, int need, bool *done) {
       }
     }
   }
+}
+
+// The same by a synchronisation every kStopPollEvery updates, in which the thread
+// waits as the device's flags say.
+lsq_status stop_polled(lsq_plan P, int it, bool *done) {
+  if (it % kStopPollEvery != kStopPollEvery - 1) return LSQ_OK;
+  LSQ_TRY(read_state(P));
+  *done = P->st_host->done != 0;
+  return LSQ_OK;
+}
+
+bool blocking_sync() {
+  unsigned flags = 0;
+  return cudaGetDeviceFlags(&flags) == cudaSuccess &&
+         (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
 }
 
 // Timing events (opt-in): a growing pool of begin/end pairs.
@@ -609,6 +629,7 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
                           {P->res, P->res2}, {P->p, P->p2}, P->pn, P->st, P->hprog};
     LSQ_CU(launch_inner_z(method, iv, P->s));
     P->launches++;
+    const bool blocking = use_thresh && blocking_sync();
     *P->hprog = 0;  // every earlier update has finished (the step before ended in read_state)
     for (int it = 0; it < cap; it++) {
       // h = D^{-1} A^T (A z);  w = R^{-T} h, the update, the next z
@@ -653,7 +674,8 @@ lsq_status run_solve(lsq_plan P, int method, const double *dA, const double *db,
       LSQ_CU(launch_inner_u(method, iv, it & 1, P->s));
       if (use_thresh && it + 1 >= kRunAhead && it + 1 < cap) {
         bool done = false;
-        LSQ_TRY(wait_progress(P, it + 1 - kRunAhead, &done));
+        if (blocking) LSQ_TRY(stop_polled(P, it, &done));
+        else LSQ_TRY(wait_progress(P, it + 1 - kRunAhead, &done));
         if (done) break;
       }
       if (kw && it % 5 == 0) {

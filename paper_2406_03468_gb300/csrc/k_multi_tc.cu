@@ -97,30 +97,43 @@ __device__ __forceinline__ unsigned tc_off(int r, int k) {
   return (unsigned)(r * 128 + (((k >> 3) ^ (r & 7)) << 4) + ((k & 7) << 1));
 }
 
-// a small integer as bf16 bits (exact up to 256): 2^23 + 2^22 + d in FP32 holds
-// d in its low bits; the difference is the float d
-__device__ __forceinline__ unsigned bf16_of(int d) {
-  return __float_as_uint(__int_as_float(0x4b400000 + d) - 12582912.0f) >> 16;
-}
-// the lowest balanced digit of q, removed from it
-__device__ __forceinline__ int pop_digit(long long &q) {
-  const int d = (int)(signed char)(q & 255);
-  q = (q - d) >> 8;
-  return d;
+// The kS balanced digits of q0 and q1 as bf16, a pair per word.  128 added to
+// each of the 6 lower digits makes them bytes; 2^23 + 2^22 + b in FP32 holds b in
+// its low byte, and subtracting 2^23 + 2^22 + 128 leaves the digit as a float, of
+// which bf16 keeps all bits (exact up to 256).
+__device__ __forceinline__ void tc_digits(long long q0, long long q1, unsigned (&w)[kS]) {
+  const unsigned long long u0 = (unsigned long long)q0 + 0x808080808080ull;
+  const unsigned long long u1 = (unsigned long long)q1 + 0x808080808080ull;
+  const unsigned lo0 = (unsigned)u0, hi0 = (unsigned)(u0 >> 32);
+  const unsigned lo1 = (unsigned)u1, hi1 = (unsigned)(u1 >> 32);
+#pragma unroll
+  for (int s = 0; s < kS; s++) {
+    const int k = kS - 1 - s;  // byte
+    const float f0 =
+        s == 0 ? __int_as_float(0x4b400000 + ((int)hi0 >> 16)) - 12582912.0f
+               : __uint_as_float(__byte_perm(k < 4 ? lo0 : hi0, 0x4b400000u, 0x7640 | (k & 3))) -
+                     12583040.0f;
+    const float f1 =
+        s == 0 ? __int_as_float(0x4b400000 + ((int)hi1 >> 16)) - 12582912.0f
+               : __uint_as_float(__byte_perm(k < 4 ? lo1 : hi1, 0x4b400000u, 0x7640 | (k & 3))) -
+                     12583040.0f;
+    w[s] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+  }
 }
 
-// q 2^-sh rounded to an integer, |q 2^-sh| <= 2^55 (or q = 0)
+// q 2^-sh rounded to an integer, |q 2^-sh| <= 2^55 (or q = 0).  No branches: the
+// rows of a warp differ in sh.
 __device__ __forceinline__ long long shift_round(long long q, int sh) {
-  if (sh > 0) return sh > 62 ? 0 : (q + (1ll << (sh - 1))) >> sh;
-  return q << min(-sh, 63);
+  const long long r = q >> min(max(sh - 1, 0), 63), l = q << min(max(1 - sh, 0), 63);
+  return ((sh > 0 ? r : l) + 1) >> 1;
 }
 
-// v 2^-g for g >= 0
+// v 2^-g for g >= 0, zero below the normal range (integer operations: FP64 ones
+// take 64 cycles per warp)
 __device__ __forceinline__ double scale_down(double v, int g) {
-  const int e = (__double2hiint(v) >> 20) & 0x7ff;
-  if (e == 0x7ff || v == 0.0) return v;
-  if (e <= g) return ldexp(v, -g);
-  return __longlong_as_double(__double_as_longlong(v) - ((long long)g << 52));
+  const long long b = __double_as_longlong(v);
+  const int e = (int)((b >> 52) & 0x7ff);
+  return e == 0x7ff ? v : e <= g ? 0.0 : __longlong_as_double(b - ((long long)g << 52));
 }
 
 // |a| 2^(55 - E) rounded to an integer, with a's sign (|a| < 2^E)
@@ -229,11 +242,10 @@ __global__ void __launch_bounds__(256)
     for (int h = 0; h < 4; h++) {
       long long q0 = second ? q[8 * g + 2 * h][r] : q[r][8 * g + 2 * h];
       long long q1 = second ? q[8 * g + 2 * h + 1][r] : q[r][8 * g + 2 * h + 1];
+      unsigned d[kS];
+      tc_digits(q0, q1, d);
 #pragma unroll
-      for (int s = kS - 1; s >= 0; s--) {
-        const int d0 = s > 0 ? pop_digit(q0) : (int)q0, d1 = s > 0 ? pop_digit(q1) : (int)q1;
-        wp[4 * s + h] = bf16_of(d0) | (bf16_of(d1) << 16);
-      }
+      for (int s = 0; s < kS; s++) wp[4 * s + h] = d[s];
     }
     unsigned char *base;
     int row;
@@ -288,11 +300,11 @@ __global__ void __launch_bounds__(256)
   }
   if (j < nkc * 64) {
     unsigned char *base = Q + (size_t)(j >> 6) * tc_qset(nv) + tc_off(c, j & 63);
+    unsigned d[kS];
+    tc_digits(q, 0, d);
 #pragma unroll
-    for (int s = kS - 1; s >= 0; s--) {
-      const int d = s > 0 ? pop_digit(q) : (int)q;
-      *reinterpret_cast<unsigned short *>(base + (size_t)s * nv * 128) = (unsigned short)bf16_of(d);
-    }
+    for (int s = 0; s < kS; s++)
+      *reinterpret_cast<unsigned short *>(base + (size_t)s * nv * 128) = (unsigned short)d[s];
   }
 }
 
@@ -693,11 +705,10 @@ __global__ void __launch_bounds__(256)
       const longlong2 v = __ldcs(yp + h);
       long long q0 = shift_round(v.x, sh0 + 2 * (int)(gw[h] & 0xffffu));
       long long q1 = shift_round(v.y, sh0 + 2 * (int)(gw[h] >> 16));
+      unsigned d[kS];
+      tc_digits(q0, q1, d);
 #pragma unroll
-      for (int s = kS - 1; s >= 0; s--) {
-        const int d0 = s > 0 ? pop_digit(q0) : (int)q0, d1 = s > 0 ? pop_digit(q1) : (int)q1;
-        wp[4 * s + h] = bf16_of(d0) | (bf16_of(d1) << 16);
-      }
+      for (int s = 0; s < kS; s++) wp[4 * s + h] = d[s];
     }
     unsigned char *base = Q + (size_t)ic * tc_qset(nv) + tc_off(c, 8 * g);
 #pragma unroll
@@ -786,11 +797,10 @@ __global__ void __launch_bounds__(256)
     for (int h = 0; h < 4; h++) {
       const double2 v = c < k ? __ldcs(yp + h) : make_double2(0.0, 0.0);
       long long q0 = tc_fix(v.x, E), q1 = tc_fix(v.y, E);
+      unsigned d[kS];
+      tc_digits(q0, q1, d);
 #pragma unroll
-      for (int s = kS - 1; s >= 0; s--) {
-        const int d0 = s > 0 ? pop_digit(q0) : (int)q0, d1 = s > 0 ? pop_digit(q1) : (int)q1;
-        wp[4 * s + h] = bf16_of(d0) | (bf16_of(d1) << 16);
-      }
+      for (int s = 0; s < kS; s++) wp[4 * s + h] = d[s];
     }
     unsigned char *base = Q + (size_t)ic * tc_qset(nv) + tc_off(c, 8 * g);
 #pragma unroll
@@ -955,7 +965,7 @@ cudaError_t tc_step1(const TcShape &t, int n, int k, double *out, const double *
 }  // namespace
 
 // Measured at 500000 x 200 x 64: y 371 us (405 with 8 reading warps that stored
-// before they let TMEM go; 1.5 GB of digits), y's digits 107 us, h 385 us (1.4 GB;
+// before they let TMEM go; 1.5 GB of digits), y's digits 101 us, h 385 us (1.4 GB;
 // the MMAs fill TMEM, so neither hides its accumulators' combination), the rest
 // 17 us: 0.88 ms per pass against 5.9 ms in double-float.
 cudaError_t launch_multi_tc_pass(int64_t m, int n, int k, const double *Z, double *out,

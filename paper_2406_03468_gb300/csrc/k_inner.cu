@@ -317,8 +317,6 @@ __device__ __forceinline__ void inner_u_body(int n, int np, const double *__rest
       }
       ss = in_sum(ss, scratch);
       if (threadIdx.x == 0) {
-        st->lq_alpha = alpha;
-        st->lq_beta = beta;
         st->lq_rhobar[par ^ 1] = -cs * alpha;
         st->lq_phibar[par ^ 1] = sn * phibar;
         st->lq_bscale = beta > 0.0 ? -alpha / beta : 0.0;

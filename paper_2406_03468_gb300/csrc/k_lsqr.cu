@@ -50,8 +50,6 @@ __global__ void __launch_bounds__(kVecThreads)
   }
   if (threadIdx.x == 0) {
     const double alpha = live ? cn / beta : 0.0;
-    st->lq_alpha = alpha;
-    st->lq_beta = beta;
     st->lq_phibar[0] = beta;
     st->lq_rhobar[0] = alpha;
     st->lq_bscale = live ? alpha / beta : 0.0;

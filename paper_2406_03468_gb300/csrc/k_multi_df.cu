@@ -12,7 +12,7 @@
 // so A leaves HBM once per pass and the work is FP32-pipe arithmetic: two
 // double-float multiply-adds per element of A and per vector.
 //
-// Arithmetic is the single-vector double-float pass's (k_pass.cu): A =
+// Arithmetic is the single-vector double-float pass's (lsq_dfpass.cuh): A =
 // hi + lo exactly to 2^-48 |a|, each z_c split hi + lo after scaling by a
 // power of two 2^-Fz_c (|z_c| < 1), products by TwoProd (fma) with the cross
 // terms hi*lo + lo*hi added to the error word, sums by TwoSum.  Each

@@ -617,7 +617,10 @@ __global__ void __launch_bounds__(kGatherWarps * 32, RPW == 2 ? 5 : 1)
 // item after the other, without waiting for each other: the atomics of a time
 // meet in the sketches of one or two items (6 MB each at n = 256).  With the
 // items dealt to the CTAs all sketches of the batch (93 MB at 32 items) were in
-// use at once, half of L2's atomic rate: 11.1 ms, now 7.2.  Chunks of 32 rows, of 8 where an
+// use at once, half of L2's atomic rate: 11.1 ms, now 7.2.  Many small
+// items are a chain over the items; whole solves of 256 of 500 x 16 still take 7.0
+// ms (32.8 when the sketch dealt the items and the inner iteration was the former
+// one), 256 of 2000 x 32 12.1 (36.2), 64 of 2000 x 32 5.4 (12.4).  Chunks of 32 rows, of 8 where an
 // item has fewer than 32 per warp.  zeta <= kBZeta.
 // ---------------------------------------------------------------------------
 constexpr int kBZeta = 8;

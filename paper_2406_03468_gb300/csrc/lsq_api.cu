@@ -989,7 +989,11 @@ void free_tc(lsq_plan P) {
   P->tc_alloc = false;
 }
 
-// The tensor-core pass's buffers: 5 times the bytes of A at n = 200 and k = 64, more
+// The tensor-core pass has no lower size: ms per solve in this form / in
+// double-float (multi_df), Gaussian A: 500 x 16 x 8 6.0 / 5.7, 2000 x 16 x 8 6.2 / 5.9,
+// 5000 x 16 x 8 5.8 / 6.1, 5000 x 16 x 64 6.4 / 6.6, 20000 x 32 x 16 7.3 / 10.8, 300000 x
+// 256 x 8 46 / 473.
+// Its buffers: 5 times the bytes of A at n = 200 and k = 64, more
 // for few columns (tiles of 64 and 128 columns).  Where they would
 // take more than half of the memory that is free, the rest being the caller's,
 // the plan uses the double-float form.

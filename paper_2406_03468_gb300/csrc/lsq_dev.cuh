@@ -1,7 +1,8 @@
-// Device helpers shared by the streaming passes over the FP32 planes of A
-// (k_pass.cu, k_multi_df.cu): error-free FP32 arithmetic (TwoSum, exact
-// widening to FP64, packed f32x2 double-float steps), mbarrier operations
-// and TMA bulk copies.  Internal to liblsq; nothing here is part of the ABI.
+// Device helpers shared by the passes over A and over its FP32 planes
+// (lsq_dfpass.cuh, k_multi_df.cu, k_multi_tc.cu and others): error-free FP32
+// arithmetic (TwoSum, exact widening to FP64, packed f32x2 double-float steps),
+// programmatic dependent launches, sums of partials, mbarrier operations and TMA
+// bulk copies.  Internal to liblsq; nothing here is part of the ABI.
 #pragma once
 
 #include <stdint.h>

@@ -19,13 +19,14 @@
 // takes 32 / G rows at a time.  G is the smallest of 8, 16, 32 with P <= 8
 // (df_tile): the row product's reduction is log2 G shuffle steps for 32 / G
 // rows at once, and no lane holds columns beyond the next multiple of 2 G.  A
-// pass that is not bound by HBM is bound by its issue slots: per row about
-// 24 P / 2 packed operations and 11 log2 G for the reduction, over 32 / G
-// rows.  Measured, against one row per warp in tiles of 64, 128, 256, 512 or
-// 1024 columns with FP64 conversions of z: 1e6 x 500 580 us (672; 6.9 TB/s,
-// 102% of the measured copy peak), 120000 x 128 28 us (41); whole iterations
-// 100000 x 257 57 us (102), 60000 x 600 80 us (157), 100000 x 64 23 us (47),
-// LSQR 200000 x 250 110 us (146).
+// pass that is not bound by HBM is bound by its arithmetic: per row about 24 P / 2
+// packed operations and 11 log2 G for the reduction, over 32 / G rows (400000 x
+// 128: FMA pipe 55% busy, issue slots 54%, DRAM 66% of its nominal rate; 200000 x
+// 500: 62%, 55%, 78%).  Measured, against one row per warp in tiles of 64, 128, 256,
+// 512 or 1024 columns with FP64 conversions of z: 1e6 x 500 592 us (672; 6.76 TB/s,
+// the measured copy rate), 120000 x 128 28 us (41); whole iterations 100000 x 257 57
+// us (102), 60000 x 600 80 us (157), 100000 x 64 23 us (47), LSQR 200000 x 250 110
+// us (146).
 //
 // Rows reach shared memory by TMA bulk copies (cp.async.bulk with mbarrier
 // completion), kStages blocks of consecutive rows per warp in flight (at

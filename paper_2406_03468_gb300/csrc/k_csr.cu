@@ -198,7 +198,15 @@ __global__ void __launch_bounds__(kCsrThreads, STAGED ? kCsrStageCtas : 1)
   int64_t r0, r1;
   csr_rows(m, r0, r1);
   if (STAGED) {
-    for (int j = threadIdx.x; j < n; j += kCsrThreads) xs[j] = x[j];
+    double xv[LSQ_MAX_N / kCsrThreads];  // all loads before the first store: one latency
+#pragma unroll
+    for (int k = 0; k < LSQ_MAX_N / kCsrThreads; k++) {
+      const int j = threadIdx.x + k * kCsrThreads;
+      xv[k] = j < n ? x[j] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < LSQ_MAX_N / kCsrThreads; k++)
+      if (threadIdx.x + k * kCsrThreads < n) xs[threadIdx.x + k * kCsrThreads] = xv[k];
     double *sv = xs + npad + (size_t)warp * kCsrStage;
     int *sc = reinterpret_cast<int *>(xs + npad + (size_t)kCsrWarps * kCsrStage) + warp * kCsrStage;
     __syncthreads();

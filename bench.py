@@ -427,9 +427,9 @@ def tier_compare(lsq, torch, dev, steps):
 
 def multi_compare(lsq, torch, dev, steps):
     """Config 4: 2e6 x 200, k = 64 right-hand sides sharing one sketch and QR.
-    The default plan runs the inner pass for all k vectors in one launch of
-    the double-float pass on the hi / lo planes (HBM roofline over the 8mn
-    bytes of the planes); a strict-FP64 plan (inner_fp64_fma = 1) runs it as
+    The default plan runs the inner and residual passes for all k vectors on
+    the tensor cores in fixed point (lsq_multi_form says what ran; HBM roofline
+    over the 8mn bytes of A); a strict-FP64 plan (inner_fp64_fma = 1) runs it as
     the FP64 tensor-core (DMMA) contraction (tensor roofline), timed over the
     same number of solves; both against the single-RHS path solving one
     column.  Four columns of X are checked against the oracle."""
@@ -452,8 +452,9 @@ def multi_compare(lsq, torch, dev, steps):
             infos.append(inf.as_dict())
         torch.cuda.synchronize()
         dt = (time.perf_counter() - t0) / nsteps
-        plan.close()
         last = infos[-1]
+        last["form"] = lsq.lsq_multi_form(plan.handle)
+        plan.close()
         return dt, last, last["ms_inner_pass"] / max(1, last["n_inner_pass"]), X.cpu().numpy().copy()
 
     dt, last, pass_ms, Xd = run({}, steps)
@@ -477,16 +478,20 @@ def multi_compare(lsq, torch, dev, steps):
     plan1.close()
     out = {"workload": "fossils_multi_m2000000_n200_k64_kappa1e8_d2400_zeta8", "steps": steps,
            "solves_per_s": 1.0 / dt, "rhs_solves_per_s": k / dt, "ms_per_solve": dt * 1e3,
-           "path": "default: both passes on the tensor cores in 56-bit fixed point, all k "
-                   "vectors per launch",
-           "inner_kernel": last["inner_kernel"],
+           "path": "default, all k vectors per launch: inner passes %s, residual passes %s"
+                   % ("in 56-bit fixed point on the tensor cores" if last["form"] & 1
+                      else "in double-float on the planes",
+                      "in 56-bit fixed point on the tensor cores" if last["form"] & 2
+                      else "FP64 (DMMA)"),
+           "inner_kernel": last["inner_kernel"], "multi_form": last["form"],
            "iters": last["iters"], "phase_ms": {"sketch": last["ms_sketch"], "qr": last["ms_qr"],
                                                 "refine": last["ms_refine"]},
            "single_rhs_solves_per_s": 1.0 / dt1,
            "inner_pass": {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"],
                           "unit": "GB/s", "frac": achieved / pk["hbm_gbs"], "ms": pass_ms,
                           "bytes": plane_bytes,
-                          "bytes_note": "the hi/lo planes read once per pass (8mn)",
+                          "bytes_note": "8mn, the bytes of A; in fixed point a pass reads its "
+                                        "digits, 28 bytes per entry",
                           "peak_kind": kind},
            "fp64_dmma": {"rhs_solves_per_s": k / dt64, "steps": steps,
                          "inner_kernel": last64["inner_kernel"],

@@ -89,3 +89,44 @@ def test_leading_weights_are_exact():
         exact = int((q[:, j].astype(object) * s.astype(object)).sum())   # units of 2^-80
         h = exact / 2 ** 80 * z0
         assert np.abs(Hh[:, j] - h).max() <= 16 * u * h, j
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 7, 8, 13, 15, 33, 65])
+def test_few_columns_strides_and_zeros(n):
+    """Few columns (A x then has bits to spare in 64), lda > n and ldb > k with
+    NaN between the rows, rows of zeros, a right-hand side of zeros."""
+    m, k = 70 * n + 643, 24
+    rng = np.random.default_rng(n)
+    A = np.full((m, n + 3), np.nan)
+    A[:, :n] = rng.standard_normal((m, n)) * 2.0 ** rng.integers(-3, 4, (m, 1))
+    A[5:300:7, :n] = 0.0
+    B = np.full((m, k + 5), np.nan)
+    B[:, :k] = A[:, :n] @ rng.standard_normal((n, k)) + 0.1 * rng.standard_normal((m, k))
+    B[:, 3] = 0.0
+    plan = lsq.Plan(m, n, seed=5, nrhs=k, lda=n + 3)
+    X = torch.empty((n, k), dtype=torch.float64, device="cuda")
+    st, _ = lsq.lsq_solve_fossils_multi(plan.handle, T(A), T(B), k + 5, X)
+    assert st == 0 and lsq.lsq_multi_form(plan.handle) == 3
+    Xh = H(X)
+    plan.close()
+    A = np.ascontiguousarray(A[:, :n])
+    assert not Xh[:, 3].any()
+    for c in (0, 9, k - 1):
+        assert oracle.kw_relative(A, np.ascontiguousarray(B[:, c]), Xh[:, c]) <= 1e-13, c
+
+
+def test_plan_pointed_at_other_sizes():
+    """One plan, its digits and sums reused for fewer rows and columns and back."""
+    rng = np.random.default_rng(2)
+    k = 40
+    plan = lsq.Plan(3001, 200, seed=5, nrhs=k)
+    for m, n in [(3001, 200), (1203, 90), (2999, 129), (700, 16), (3001, 200)]:
+        lsq.lsq_plan_configure(plan.handle, lsq.lsq_options_default(m=m, n=n, seed=5, nrhs=k))
+        A, B = rng.standard_normal((m, n)), rng.standard_normal((m, k))
+        X = torch.empty((n, k), dtype=torch.float64, device="cuda")
+        st, _ = lsq.lsq_solve_fossils_multi(plan.handle, T(A), T(B), k, X)
+        assert st == 0 and lsq.lsq_multi_form(plan.handle) == 3
+        Xh = H(X)
+        for c in (0, k - 1):
+            assert oracle.kw_relative(A, B[:, c], Xh[:, c]) <= 1e-13, (m, n, c)
+    plan.close()
